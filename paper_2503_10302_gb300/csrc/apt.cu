@@ -63,64 +63,161 @@ using namespace pcdev;
 using pc::AptArgs;
 using pc::AptProbDev;
 
-constexpr int MAXGC = 4;   // groups handled per thread per site
-
-struct Geo {
+// Everything a phase of the kernel needs to know about its CTA, at the start
+// of dynamic shared memory.  The phases are functions of their own that read
+// it from there: each gets its own register allocation, and nothing but the
+// loop counters lives in registers across them (as one inlined kernel the
+// phases shared the 128-register limit and every edit of one moved the code
+// of the others).  Both CTAs of a split problem have it at the same address.
+struct __align__(16) Ctl {
   int Lx, Ly, Lz, N, H, hx;
   uint32_t mhx, mLy, mLy2;
+  int T, Tp, A, B, Bc, Gc, g0;
+  // this CTA holds, for every label, the temperature groups [g0, g0 + Gu) of
+  // the Glp groups per label (APT; ladder / pilot: A = 1, groups g0 ..);
+  // split problems run as a cluster of two CTAs, rank 0 holding the hotter
+  // (lower-beta, first) half
+  int Gu, Glp, split, rank;
+  int nbonds;        // bonds present (3N with periodic axes)
+  int nreal;         // spins present (N without vacancies)
+  uint32_t open;     // bit a: axis a open; bit 3: vacancies
+  uint32_t ent;
+  // replica groups in quads: quad q holds groups [q gq, (q + 1) gq), W = 1 << lw
+  // words apart; the threads in nch chunks of tpc, chunk q sweeping quads q, q + nch, ..
+  int nq, gq, lw, nch, tpc;
+  uint32_t k0, k1, tag_main, tag_ref;
+  int joint, icm_big, stage_swt;
+  int oThr, oThh, oHist, oS, oV, oJn, oStage, oSwt;   // word offsets of the arrays below
+  const uint32_t *swapidx, *swaptab;   // the problem's swap tables in global memory
+  int8_t *best_spins;                  // where this CTA's best state goes
+  int64_t m64[4];      // best E, best sweep, hit sweep, target
+  int64_t sum1[64], sum2[64];   // ladder sums
+  int32_t m32[8];      // best buffer, flag, icm counters x3, any-swap flag, -, local best buffer
+  int32_t E[64], Eacc[64], temp_of[64];
+  int32_t satt[128], sacc[128];   // swap attempts / accepts of this launch
+  uint32_t ikx[64];    // per pair: Philox word 0
+  int32_t ibit[64];    // per pair: replica choice bit; [32 ..]: 4-label matching per temperature
+  int32_t inm[64];     // per pair: mismatch count
+  int32_t isz[64];     // per pair: cluster size
+  uint32_t imask[24];  // [3][8] per group: cluster-flip masks, whole flips
+  uint32_t swm[24];    // [8] per group: in-group swap nibble mask; [8] cross-group flags;
+                       // [6] ICM matching nibble masks (4 labels)
+  int32_t gmap[8];     // global group of each local group
+  int32_t xch[24];     // split problems: [2][4] boundary energies by attempt parity;
+                       // [8] accepted boundary labels; [12..17] the peer's best at launch
+                       // end; [18..21] boundary draws
 };
+// Arrays after Ctl:
+//   thr  [64][16]    p-bit thresholds of each buffer, entry I + 6
+//   thh  [64][16]    their top halves, 16-bit, each group's 256 bytes on a 256-byte boundary
+//   hist [T][n_bins] pilot histogram
+//   stage [2][4][64] peer boundary spins by attempt parity, one bit per site (split)
+//   swt  [T-1][kSwtLen] first entries of each pair's swap table (split)
+//   S    [nq][2][H][W]  spin words: group q gq + u, colour c, site j at ((2 q + c) H + j) W + u, so
+//                    the words of a site's groups move as one vector access
+//   V    ICM cluster bits [2][H], overlap bits [2][H], transposed overlaps [N/32][32], root masks
+//   jn   [2][H]      coupling signs (bits 0-5), missing bonds (8-13), vacancy (15) and, from bit
+//                    16, the site's place: x odd in its row pair, wraps of +x -x +y -y +z -z
 
-// Neighbours (other colour, colour-local index) of site (c, j), in the
-// direction order +x, -x, +y, -y, +z, -z; periodic boundaries.
-__device__ __forceinline__ void neighbours(const Geo &g, int c, int j, int (&n)[6]) {
-  const int row = (int)fdiv((uint32_t)j, g.mhx);   // j / hx
-  const int jx = j - row * g.hx;
-  const int z = (int)fdiv((uint32_t)row, g.mLy);   // row / Ly
-  const int y = row - z * g.Ly;
-  const int p = (y + z + c) & 1;                   // x = 2 jx + p
-  const int base = row * g.hx;
-  int jxp, jxm;
-  if (p == 0) {
-    jxp = jx;
-    jxm = (jx == 0) ? g.hx - 1 : jx - 1;
-  } else {
-    jxp = (jx + 1 == g.hx) ? 0 : jx + 1;
-    jxm = jx;
-  }
-  n[0] = base + jxp;
-  n[1] = base + jxm;
-  const int yp = (y + 1 == g.Ly) ? 0 : y + 1, ym = (y == 0) ? g.Ly - 1 : y - 1;
-  const int zp = (z + 1 == g.Lz) ? 0 : z + 1, zm = (z == 0) ? g.Lz - 1 : z - 1;
-  n[2] = (yp + g.Ly * z) * g.hx + jx;
-  n[3] = (ym + g.Ly * z) * g.hx + jx;
-  n[4] = (y + g.Ly * zp) * g.hx + jx;
-  n[5] = (y + g.Ly * zm) * g.hx + jx;
+// Entries of each pair's swap table (|dE| = 0, 2, .., 2 (kSwtLen - 1)) that a
+// split problem's CTAs keep in shared memory; larger |dE| read the table in
+// global memory.
+constexpr int kSwtLen = 256;
+
+extern __shared__ __align__(16) uint32_t smem_words[];
+__device__ __forceinline__ uint32_t *dyn_smem() { return smem_words; }
+__device__ __forceinline__ Ctl &ctl() { return *reinterpret_cast<Ctl *>(dyn_smem()); }
+
+// Groups per quad and words per quad and site: as few quads of at most four
+// groups as hold Gc, evenly filled (8 -> 4 + 4, 6 -> 3 + 3).  A thread's four
+// groups share the site's neighbours and couplings and one 16-byte access
+// per neighbour.
+__host__ __device__ inline int quads_of(int Gc) { return (Gc + 3) >> 2; }
+__host__ __device__ inline int quad_groups(int Gc) { return (Gc + quads_of(Gc) - 1) / quads_of(Gc); }
+__host__ __device__ inline int quad_shift(int Gc) { const int g = quad_groups(Gc); return g > 2 ? 2 : g - 1; }
+// spin words per site of a CTA with Gc groups
+__host__ __device__ inline int site_words(int Gc) { return quads_of(Gc) << quad_shift(Gc); }
+
+// First word of local group g in S, and the word of canonical site kk = c H + j.
+__device__ __forceinline__ int group_off(const Ctl &k, int g) {
+  const int q = g / k.gq;
+  return ((2 * k.H * q) << k.lw) + (g - q * k.gq);
+}
+__device__ __forceinline__ uint32_t &spin_word(const Ctl &k, uint32_t *S, int g, int kk) {
+  return S[group_off(k, g) + (kk << k.lw)];
+}
+
+// Neighbours (other colour, colour-local index) of site (c, j) with packed
+// word jb, in the direction order +x, -x, +y, -y, +z, -z; periodic wraps.
+__device__ __forceinline__ void neighbours(const Ctl &k, int j, uint32_t jb, int (&n)[6]) {
+  const int hx = k.hx, sy = hx, sz = hx * k.Ly, wy = sz - sy, wz = sz * (k.Lz - 1);
+  n[0] = j + ((jb & (1u << 16)) ? ((jb & (1u << 17)) ? 1 - hx : 1) : 0);
+  n[1] = j + ((jb & (1u << 16)) ? 0 : ((jb & (1u << 18)) ? hx - 1 : -1));
+  n[2] = j + ((jb & (1u << 19)) ? -wy : sy);
+  n[3] = j + ((jb & (1u << 20)) ? wy : -sy);
+  n[4] = j + ((jb & (1u << 21)) ? -wz : sz);
+  n[5] = j + ((jb & (1u << 22)) ? wz : -sz);
+}
+
+// The place bits (16 ..) of site (c, j).
+__device__ __forceinline__ uint32_t place_bits(const Ctl &k, int c, int j) {
+  const int row = (int)fdiv((uint32_t)j, k.mhx);   // j / hx
+  const int jx = j - row * k.hx;
+  const int z = (int)fdiv((uint32_t)row, k.mLy);   // row / Ly
+  const int y = row - z * k.Ly;
+  const uint32_t p = (uint32_t)((y + z + c) & 1);  // x = 2 jx + p
+  return (p << 16) | (jx + 1 == k.hx ? 1u << 17 : 0u) | (jx == 0 ? 1u << 18 : 0u) |
+         (y + 1 == k.Ly ? 1u << 19 : 0u) | (y == 0 ? 1u << 20 : 0u) | (z + 1 == k.Lz ? 1u << 21 : 0u) |
+         (z == 0 ? 1u << 22 : 0u);
 }
 
 // lin = x + Lx (y + Ly z) of site (c, j).
-__device__ __forceinline__ int lin_of(const Geo &g, int c, int j) {
-  const int row = (int)fdiv((uint32_t)j, g.mhx);
-  const int jx = j - row * g.hx;
-  const int z = (int)fdiv((uint32_t)row, g.mLy);
-  const int y = row - z * g.Ly;
-  return 2 * jx + ((y + z + c) & 1) + g.Lx * row;
+__device__ __forceinline__ int lin_of(const Ctl &k, int c, int j) {
+  const int row = (int)fdiv((uint32_t)j, k.mhx);
+  const int jx = j - row * k.hx;
+  const int z = (int)fdiv((uint32_t)row, k.mLy);
+  const int y = row - z * k.Ly;
+  return 2 * jx + ((y + z + c) & 1) + k.Lx * row;
 }
 
+// The first NG of the W words of a (quad, site), which start on a W-word
+// boundary.
+template <int NG>
+__device__ __forceinline__ void load_vec(const uint32_t *p, uint32_t (&v)[NG]) {
+  if constexpr (NG >= 3) {
+    const uint4 t = *reinterpret_cast<const uint4 *>(p);
+    v[0] = t.x; v[1] = t.y; v[2] = t.z;
+    if constexpr (NG == 4) v[3] = t.w;
+  } else if constexpr (NG == 2) {
+    const uint2 t = *reinterpret_cast<const uint2 *>(p);
+    v[0] = t.x; v[1] = t.y;
+  } else {
+    v[0] = *p;
+  }
+}
+template <int NG>
+__device__ __forceinline__ void store_vec(uint32_t *p, const uint32_t (&v)[NG]) {
+  if constexpr (NG >= 3) {
+    *reinterpret_cast<uint4 *>(p) = make_uint4(v[0], v[1], v[2], NG == 4 ? v[NG - 1] : 0u);
+  } else if constexpr (NG == 2) {
+    *reinterpret_cast<uint2 *>(p) = make_uint2(v[0], v[1]);
+  } else {
+    *p = v[0];
+  }
+}
 
-// Threshold of nibble i (thr points at the group's 128 entries: 8 buffers x
-// 16, entry I + 6 for I = -6..6).  SCALE 1: C holds I + 6 per nibble;
-// SCALE 2: C holds the satisfied count of a site with all six bonds, whose
-// entry is 2C.
-// thrh holds the thresholds' top halves t as 16-bit entries in the same
-// [buffer][16] order, each group's 256 bytes starting on a 256-byte
-// boundary of shared memory (tb, a shared-window address), so the entry of
-// nibble i sits at tb | (32 i + 2 SCALE c_i), 32 i + 2 SCALE c_i <= 248:
-// the offsets of 4 nibbles are formed in one word and each address is one
-// byte permute of that word with tb.  The sign of d = v - t for the main
-// half v is the decision, and the top 4 bits of each d are shifted into w
-// so that bit 3 of nibble i carries half i's sign.  A zero product of the
-// differences (mod 2^32) flags a possible tie, which refine8_grp settles
-// exactly (a product that only wraps to 0 costs a needless refine).
+// Eq. neuron for the 8 nibbles of one word.  SCALE 2: C holds per nibble
+// the satisfied count of a site with all six bonds, whose entry is 2C;
+// SCALE 1: C holds the threshold index I + 6.  thh holds the thresholds' top
+// halves t as 16-bit entries [buffer][16], each group's 256 bytes starting
+// on a 256-byte boundary of shared memory (tb, a shared-window address), so
+// the entry of nibble i sits at tb | (32 i + 2 SCALE c_i), at most 248: the
+// offsets of 4 nibbles are formed in one word and each address is one byte
+// permute of that word with tb.  The sign of d = v - t for the main half v is
+// the decision, and the top 4 bits of each d are shifted into w so that bit 3
+// of nibble i carries half i's sign.  A zero product of the differences
+// (mod 2^32) flags a possible tie, which refine8_grp settles exactly (a
+// product that only wraps to 0 costs a needless refine).
 template <int SCALE>
 __device__ __forceinline__ uint32_t decide8_grp(const uint4 &x, uint32_t C, uint32_t tb, bool &tie) {
   // byte k of Dlo: offset of nibble 2k (64 k + 2 SCALE c); of Dhi: nibble 2k+1
@@ -130,9 +227,7 @@ __device__ __forceinline__ uint32_t decide8_grp(const uint4 &x, uint32_t C, uint
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
     // byte 0 from the offsets, bytes 1-3 from tb
-    const uint32_t addr = __byte_perm((i & 1) ? Dhi : Dlo, tb, 0x7650u + (uint32_t)(i >> 1));
-    uint32_t th;
-    asm("ld.shared.u16 %0, [%1];" : "=r"(th) : "r"(addr));
+    const uint32_t th = lds_u16(__byte_perm((i & 1) ? Dhi : Dlo, tb, 0x7650u + (uint32_t)(i >> 1)));
     const uint32_t d = half_lo(x, i) - th;
     w = __funnelshift_l(d, w, 4);
     tp *= d;
@@ -141,9 +236,11 @@ __device__ __forceinline__ uint32_t decide8_grp(const uint4 &x, uint32_t C, uint
   return (w >> 3) & 0x11111111u;
 }
 
+// Threshold of nibble i (thr points at the group's 128 entries: 8 buffers x
+// 16, entry I + 6 for I = -6..6).  SCALE 1: C holds I + 6 per nibble;
+// SCALE 2: C holds the satisfied count, whose entry is 2C.
 template <int SCALE>
-__device__ __noinline__ uint32_t refine8_grp(uint32_t w, uint4 x, uint4 y, uint32_t C,
-                                             const uint32_t *thr) {
+__device__ __noinline__ uint32_t refine8_grp(uint32_t w, uint4 x, uint4 y, uint32_t C, const uint32_t *thr) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const uint32_t t = thr[16 * i + SCALE * ((C >> (4 * i)) & 0xFu)];
@@ -156,123 +253,67 @@ __device__ __noinline__ uint32_t refine8_grp(uint32_t w, uint4 x, uint4 y, uint3
   return w;
 }
 
-struct Shared {
-  uint32_t *S;       // [Gc][2][H]
-  uint32_t *thr;     // [Gc*8][16] p-bit thresholds, entry I + 6
-  uint16_t *thrh;    // [Gc*8][16] their high halves (16-bit)
-  int32_t *temp_of;  // [Gc*8]
-  int32_t *buf_of;   // [Gc*8] (unused by the fixed-slot APT mode)
-  int32_t *E;        // [Gc*8]
-  int32_t *Eacc;     // [Gc*8]
-  int32_t *satt, *sacc;   // [64] swap attempts / accepts of this launch
-  int32_t *hist;     // pilot histogram [T][n_bins]
-  int64_t *sum1, *sum2;   // ladder sums [Gc*8]
-  int64_t *m64;      // best E, best sweep, hit sweep, target
-  int32_t *m32;      // best buffer, flag, icm counters x3, any-swap flag
-  uint16_t *jn;      // [2][H] coupling signs (bits 0-5) and missing bonds (8-13)
-  uint32_t *V;       // ICM cluster bits [2][H], overlap bits [2][H], transposed overlaps [N/32][32]
-  uint32_t *ikx;     // [64] per pair: Philox word 0, then k
-  int32_t *ibit;     // [64] per pair: replica choice bit
-  int32_t *inm;      // [64] per pair: mismatch count
-  int32_t *isz;      // [64] per pair: cluster size
-  uint32_t *imask;   // [3][8] per half-group: cluster-flip, whole-flip label 0, label 1
-  uint32_t *swm;     // [8] per group: in-group swap nibble mask; [8] cross-group flags;
-                     // [6] ICM matching nibble masks (4 labels)
-  int32_t *gmap;     // [8] global group of each local group
-  int32_t *xch;      // split problems: [2][4] boundary energies by attempt parity;
-                     // [8] accepted boundary labels; [12..17] the peer's best at launch end
-  uint32_t *stage;   // [2][4][64] peer boundary spins by attempt parity, one bit per site
-  uint32_t *swt;     // split problems: [T-1][kSwtLen] first entries of each pair's swap table
-};
-
-// Entries of each pair's swap table (|dE| = 0, 2, .., 2 (kSwtLen - 1)) that a
-// split problem's CTAs keep in shared memory; larger |dE| read the table in
-// global memory.
-constexpr int kSwtLen = 256;
-
-struct Cta {
-  Geo geo;
-  int T, Tp, A, B, Bc, Gc, g0;
-  // this CTA holds, for every label, the temperature groups [g0, g0 + Gu) of
-  // the Glp groups per label (APT; ladder / pilot: A = 1, groups g0 ..);
-  // split problems run as a cluster of two CTAs, rank 0 holding the hotter
-  // (lower-beta, first) half
-  int Gu, Glp, split, rank;
-  int nbonds;        // bonds present (3N with periodic axes)
-  int nreal;         // spins present (N without vacancies)
-  uint32_t open;     // bit a: axis a open
-  uint32_t ent;
-  // thread chunking of the site loop: nch chunks of tpc threads, gc groups each
-  int nch, tpc, gc;
-};
-
 // Satisfied-bond counts of NG groups in byte lanes: e8[u][0] byte k counts
 // nibble 2k, e8[u][1] byte k nibble 2k + 1.  A site adds at most 6 to a
 // lane, so a thread reduces them after at most kFlushSites sites.
 constexpr int kFlushSites = 32;
 
-// The NG groups [gbeg, gbeg + NG) of site (c, j): every neighbour word is
+// The NG groups of quad `quad` at site (c, j): the neighbour vectors are
 // loaded first, then the NG decisions run as one branch-free block whose
-// Philox chains are independent, ties (a zero product of a word's eight
-// differences, about 2^-13 per word) are settled after it, and the stores
-// come last.  The field of 8 spins is C = n_neg 0x11111111 + sum_d eps_d W_d
-// with eps_d = +1 (J > 0), -1 (J < 0) or 0 (absent bond): per nibble the
-// count of satisfied present bonds (W ^ 1 for a negative bond is 1 - W),
-// exact mod 2^32 because every final nibble lies in 0..6.
-template <int NG, bool UPDATE, bool ENERGY, bool OPEN>
-__device__ __forceinline__ void site_groups(const AptArgs &a, const Cta &k, const Shared &sh, int c, int j,
-                                            uint32_t sweep, int gbeg, uint32_t (&e8)[NG][2]) {
-  const int H = k.geo.H;
-  const uint32_t tb0 = (uint32_t)__cvta_generic_to_shared(sh.thrh) + 256u * (uint32_t)gbeg;
+// Philox chains are independent, ties (about 2^-13 per word) are settled
+// after it, and the store comes last.  The field of 8 spins is
+// C = n_neg 0x11111111 + sum_d eps_d W_d with eps_d = +1 (J > 0), -1 (J < 0)
+// or 0 (absent bond): per nibble the count of satisfied present bonds
+// (W ^ 1 for a negative bond is 1 - W), exact mod 2^32 because every final
+// nibble lies in 0..6.
+template <int NG, int W, bool UPDATE, bool ENERGY, bool OPEN>
+__device__ __forceinline__ void quad_site(const Ctl &k, uint32_t *Sq, const uint32_t *jn, uint32_t tb0, int c, int j,
+                                          int quad, uint32_t sweep, const PhiloxB (&pb)[NG], uint32_t (&e8)[NG][2]) {
+  const int H = k.H;
+  const uint32_t *Wo = Sq + (1 - c) * H * W;
+  uint32_t *Wc = Sq + (c * H + j) * W;
+  const uint32_t jb = jn[c * H + j];
   int n[6];
-  neighbours(k.geo, c, j, n);
-  const uint32_t jb = sh.jn[c * H + j];
+  neighbours(k, j, jb, n);
   const uint32_t miss = OPEN ? (jb >> 8) & 0x3Fu : 0u;
   const uint32_t K = OPEN ? (uint32_t)__popc(miss) * 0x11111111u : 0u;
-  uint32_t eps[6];
-#pragma unroll
-  for (int d = 0; d < 6; ++d) {
-    const uint32_t e = 1u - 2u * ((jb >> d) & 1u);
-    eps[d] = (OPEN && ((miss >> d) & 1u)) ? 0u : e;
-  }
-  const uint32_t K0 = (uint32_t)__popc(jb & 0x3Fu & ~miss) * 0x11111111u;
   uint32_t C[NG], w[NG];
 #pragma unroll
-  for (int u = 0; u < NG; ++u) {
-    const uint32_t *Wo = sh.S + (size_t)(2 * (gbeg + u) + (1 - c)) * H;
-    uint32_t s = K0;
+  for (int u = 0; u < NG; ++u) C[u] = (uint32_t)__popc(jb & 0x3Fu & ~miss) * 0x11111111u;
 #pragma unroll
-    for (int d = 0; d < 6; ++d) s += eps[d] * Wo[n[d]];
-    C[u] = s;
+  for (int d = 0; d < 6; ++d) {
+    uint32_t e = 1u - 2u * ((jb >> d) & 1u), nv[NG];
+    if (OPEN && ((miss >> d) & 1u)) e = 0u;
+    load_vec<NG>(Wo + n[d] * W, nv);
+#pragma unroll
+    for (int u = 0; u < NG; ++u) C[u] += e * nv[u];
   }
   if (UPDATE) {
-    const uint32_t c2 = (uint32_t)c << 16, tag = (k.ent << 8) | a.tag_main;
+    const PhiloxA pa = philox_a((uint32_t)j, (k.ent << 8) | k.tag_main, k.k1);
     uint32_t tmask = 0u;
 #pragma unroll
     for (int u = 0; u < NG; ++u) {
-      const uint4 x = philox((uint32_t)j, sweep, c2 | (uint32_t)sh.gmap[gbeg + u], tag, a.k0, a.k1);
+      const uint4 x = philox_ab(pa, pb[u], k.k0, k.k1);
+      // threshold index I + 6 = 2C + k per nibble when bonds are absent
       bool tie = false;
-      // threshold index I + 6 = 2C + k per nibble (2C with every bond)
-      const uint32_t D = OPEN ? 2u * C[u] + K : C[u];
-      w[u] = decide8_grp<OPEN ? 1 : 2>(x, D, tb0 + 256u * (uint32_t)u, tie);
+      w[u] = decide8_grp<OPEN ? 1 : 2>(x, OPEN ? 2u * C[u] + K : C[u], tb0 + 256u * (uint32_t)u, tie);
       tmask |= tie ? (1u << u) : 0u;
     }
     if (tmask) {
+      const uint32_t *thr = dyn_smem() + k.oThr;
 #pragma unroll
       for (int u = 0; u < NG; ++u) {
         if (!((tmask >> u) & 1u)) continue;
-        const uint32_t g = (uint32_t)sh.gmap[gbeg + u];
-        const uint4 x = philox((uint32_t)j, sweep, c2 | g, tag, a.k0, a.k1);
-        const uint4 y = philox((uint32_t)j, sweep, c2 | g, (k.ent << 8) | a.tag_ref, a.k0, a.k1);
-        const uint32_t D = OPEN ? 2u * C[u] + K : C[u];
-        w[u] = refine8_grp<OPEN ? 1 : 2>(w[u], x, y, D, sh.thr + 128 * (gbeg + u));
+        const int g = quad * k.gq + u;
+        const uint32_t c2 = ((uint32_t)c << 16) | (uint32_t)k.gmap[g];
+        const uint4 x = philox((uint32_t)j, sweep, c2, (k.ent << 8) | k.tag_main, k.k0, k.k1);
+        const uint4 y = philox((uint32_t)j, sweep, c2, (k.ent << 8) | k.tag_ref, k.k0, k.k1);
+        w[u] = refine8_grp<OPEN ? 1 : 2>(w[u], x, y, OPEN ? 2u * C[u] + K : C[u], thr + 128 * g);
       }
     }
-#pragma unroll
-    for (int u = 0; u < NG; ++u) sh.S[(size_t)(2 * (gbeg + u) + c) * H + j] = w[u];
+    store_vec<NG>(Wc, w);
   } else {
-#pragma unroll
-    for (int u = 0; u < NG; ++u) w[u] = sh.S[(size_t)(2 * (gbeg + u) + c) * H + j];
+    load_vec<NG>(Wc, w);
   }
   if (ENERGY) {
 #pragma unroll
@@ -285,50 +326,57 @@ __device__ __forceinline__ void site_groups(const AptArgs &a, const Cta &k, cons
   }
 }
 
-// The sites j = j0, j0 + tpc, .. below j1 of colour c for the NG groups
-// from gbeg; at most kFlushSites sites per thread, so that the byte lanes
-// of the energy counts cannot overflow.  Every lane of a warp calls it
-// (the warp reduction at the end).
-template <int NG, bool UPDATE, bool ENERGY, bool OPEN>
-__device__ __forceinline__ void site_loop(const AptArgs &a, const Cta &k, const Shared &sh, int c,
-                                          uint32_t sweep, int j0, int j1, int gbeg) {
-  uint32_t e8[NG][2];
+// Colour c of one quad: sites lt, lt + tpc, .. in blocks of at most
+// kFlushSites per thread, so that the byte lanes of the energy counts cannot
+// overflow.  Whole warps call it (the warp reductions).  The counts leave a
+// warp through one warp-wide add per packed word (two 16-bit lanes, at most
+// 32 x 192 each) and one atomic per buffer, all buffers' lanes at once.
+template <int NG, int W, bool UPDATE, bool ENERGY, bool OPEN>
+__device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int quad, int lt, int tpc) {
+  const int H = k.H;
+  uint32_t *Sq = dyn_smem() + k.oS + 2 * quad * H * W;
+  const uint32_t *jn = dyn_smem() + k.oJn;
+  const uint32_t tb0 = (uint32_t)__cvta_generic_to_shared(dyn_smem() + k.oThh) + 256u * (uint32_t)(quad * k.gq);
+  PhiloxB pb[NG];
+  if (UPDATE) {
 #pragma unroll
-  for (int u = 0; u < NG; ++u) e8[u][0] = e8[u][1] = 0u;
-  for (int j = j0; j < j1; j += k.tpc) site_groups<NG, UPDATE, ENERGY, OPEN>(a, k, sh, c, j, sweep, gbeg, e8);
-  if (ENERGY) {
-    // lanes of a warp share the chunk (and NG); reduce 16-bit lanes across
-    // the warp: word m of a group holds nibbles m (low) and m + 4 (high)
-    const int lane = threadIdx.x & 31;
+    for (int u = 0; u < NG; ++u)
+      pb[u] = philox_b(sweep, ((uint32_t)c << 16) | (uint32_t)k.gmap[quad * k.gq + u], k.k0, k.k1);
+  }
+  for (int b0 = 0; b0 < H; b0 += ENERGY ? kFlushSites * tpc : H) {
+    const int b1 = ENERGY ? min(H, b0 + kFlushSites * tpc) : H;
+    uint32_t e8[NG][2];
 #pragma unroll
-    for (int u = 0; u < NG; ++u) {
+    for (int u = 0; u < NG; ++u) e8[u][0] = e8[u][1] = 0u;
+    for (int j = b0 + lt; j < b1; j += tpc)
+      quad_site<NG, W, UPDATE, ENERGY, OPEN>(k, Sq, jn, tb0, c, j, quad, sweep, pb, e8);
+    if (ENERGY) {
+      const int lane = threadIdx.x & 31;
+      uint32_t mine = 0u;
 #pragma unroll
-      for (int m = 0; m < 4; ++m) {
-        uint32_t v = (e8[u][m & 1] >> (8 * (m >> 1))) & 0x00FF00FFu;
+      for (int u = 0; u < NG; ++u)
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-        if (lane == 0) {
-          const int b = 8 * (gbeg + u) + m;
-          atomicAdd(&sh.Eacc[b], (int)(v & 0xFFFFu));
-          atomicAdd(&sh.Eacc[b + 4], (int)(v >> 16));
+        for (int m = 0; m < 4; ++m) {
+          // low 16 bits: nibble m, high 16 bits: nibble m + 4
+          const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, (e8[u][m & 1] >> (8 * (m >> 1))) & 0x00FF00FFu);
+          if ((lane >> 3) == u && (lane & 3) == m) mine = v;
         }
-      }
+      if (lane < 8 * NG) atomicAdd(&k.Eacc[8 * quad * k.gq + lane], (int)((lane & 4) ? mine >> 16 : mine & 0xFFFFu));
     }
   }
 }
 
-// Sites of colour c in blocks of kFlushSites per thread (one block unless
-// H > kFlushSites * tpc).
-template <int NG, bool UPDATE, bool ENERGY, bool OPEN>
-__device__ __forceinline__ void site_blocks(const AptArgs &a, const Cta &k, const Shared &sh, int c,
-                                            uint32_t sweep, int lt, int gbeg) {
-  const int H = k.geo.H, span = kFlushSites * k.tpc;
-  if (!ENERGY || H <= span) {
-    site_loop<NG, UPDATE, ENERGY, OPEN>(a, k, sh, c, sweep, lt, H, gbeg);
-    return;
+template <bool UPDATE, bool ENERGY, bool OPEN>
+__device__ __forceinline__ void colour_phase_t(Ctl &k, int c, uint32_t sweep) {
+  const int q = (int)threadIdx.x / k.tpc, lt = (int)threadIdx.x - q * k.tpc;
+  for (int quad = q; quad < k.nq; quad += k.nch) {
+    switch (k.gq) {
+      case 4: quad_sites<4, 4, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc); break;
+      case 3: quad_sites<3, 4, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc); break;
+      case 2: quad_sites<2, 2, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc); break;
+      default: quad_sites<1, 1, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc); break;
+    }
   }
-  for (int b0 = 0; b0 < H; b0 += span)
-    site_loop<NG, UPDATE, ENERGY, OPEN>(a, k, sh, c, sweep, b0 + lt, min(H, b0 + span), gbeg);
 }
 
 // One colour phase of a sweep over the CTA's groups.  UPDATE: Eq. synapse +
@@ -337,99 +385,96 @@ __device__ __forceinline__ void site_blocks(const AptArgs &a, const Cta &k, cons
 // colour-1 endpoint, so the colour-1 pass gives E = nbonds - 2 * satisfied).
 // A site missing k of its six bonds (open boundaries) counts its satisfied
 // present bonds C, so I = 2C - (6 - k); the threshold row is indexed by
-// I + 6 = 2C + k, formed for eight spins at once as 2C + k * 0x11111111.
-template <bool UPDATE, bool ENERGY, bool OPEN>
-__device__ __forceinline__ void colour_phase_t(const AptArgs &a, const Cta &k, const Shared &sh,
-                                               int c, uint32_t sweep, int gtot) {
-  const int tid = threadIdx.x;
-  const int q = tid / k.tpc, lt = tid - q * k.tpc;
-  // groups [0, gtot) over the nch thread chunks (at most MAXGC per chunk)
-  const int gper = gtot == k.Gc ? k.gc : (gtot + k.nch - 1) / k.nch;
-  const int gbeg = q * gper;
-  int gcnt = gtot - gbeg;
-  if (gcnt > gper) gcnt = gper;
-  if (gcnt >= 4)
-    site_blocks<4, UPDATE, ENERGY, OPEN>(a, k, sh, c, sweep, lt, gbeg);
-  else if (gcnt == 3)
-    site_blocks<3, UPDATE, ENERGY, OPEN>(a, k, sh, c, sweep, lt, gbeg);
-  else if (gcnt == 2)
-    site_blocks<2, UPDATE, ENERGY, OPEN>(a, k, sh, c, sweep, lt, gbeg);
-  else if (gcnt == 1)
-    site_blocks<1, UPDATE, ENERGY, OPEN>(a, k, sh, c, sweep, lt, gbeg);
-}
-
-// Periodic problems take the path without absent-bond handling.
+// I + 6 = 2C + k.  Periodic problems take the path without absent bonds.
 template <bool UPDATE, bool ENERGY>
-__device__ __forceinline__ void colour_phase(const AptArgs &a, const Cta &k, const Shared &sh, int c,
-                                             uint32_t sweep, int gtot) {
+__device__ __noinline__ void colour_phase(int c, uint32_t sweep) {
+  Ctl &k = ctl();
   if (k.open)
-    colour_phase_t<UPDATE, ENERGY, true>(a, k, sh, c, sweep, gtot);
+    colour_phase_t<UPDATE, ENERGY, true>(k, c, sweep);
   else
-    colour_phase_t<UPDATE, ENERGY, false>(a, k, sh, c, sweep, gtot);
+    colour_phase_t<UPDATE, ENERGY, false>(k, c, sweep);
 }
 
-// E_b = nbonds - 2 * (satisfied bonds); resets the accumulators.
-__device__ __forceinline__ void finish_energies(const Cta &k, const Shared &sh) {
-  for (int b = threadIdx.x; b < 8 * k.Gc; b += blockDim.x) {
-    sh.E[b] = k.nbonds - 2 * sh.Eacc[b];
-    sh.Eacc[b] = 0;
+// Energies of label 0 only (two labels): its groups lead quad 0, all threads
+// share the sites.
+template <bool OPEN>
+__device__ __forceinline__ void label0_energies_t(Ctl &k) {
+  const int lt = (int)threadIdx.x, tpc = (int)blockDim.x;
+  switch (k.Gu) {
+    case 4: quad_sites<4, 4, false, true, OPEN>(k, 1, 0u, 0, lt, tpc); break;
+    case 3: quad_sites<3, 4, false, true, OPEN>(k, 1, 0u, 0, lt, tpc); break;
+    case 2: quad_sites<2, 4, false, true, OPEN>(k, 1, 0u, 0, lt, tpc); break;
+    default: quad_sites<1, 2, false, true, OPEN>(k, 1, 0u, 0, lt, tpc); break;
   }
 }
+__device__ __noinline__ void label0_energies() {
+  Ctl &k = ctl();
+  if (k.open)
+    label0_energies_t<true>(k);
+  else
+    label0_energies_t<false>(k);
+}
 
-// Minimum-energy selection (Algorithm S2 output): strict improvement, lowest
-// slot index (r * A + a) on ties; copies the state of the new best replica.
-// The two CTAs of a split problem track their own candidates (rank 1 into a
-// scratch state) and combine them at the end of the launch: the global best
-// is the lower energy, found at the earlier sweep, rank 0 (the lower slots)
-// on ties, and the target is first hit at the earlier of the two hits.
-__device__ void best_update(const AptArgs &a, const Cta &k, const Shared &sh, int p,
-                            int64_t sweeps) {
-  if (threadIdx.x < 32) {
-    // the lowest energy, ties to the lowest slot r A + label: one warp
-    // minimum of the key (E + 2^18) 2^8 + slot (|E| <= 3N < 2^18, slot < 2^8)
-    const int lane = threadIdx.x;
-    uint32_t key = 0xFFFFFFFFu;
-    int bestb = 0;
-    for (int b = lane; b < 8 * k.Gc; b += 32) {
-      const int gb = 8 * sh.gmap[b >> 3] + (b & 7);
-      const int r = gb % k.Tp, lab = gb / k.Tp;
-      if (r >= k.T) continue;
-      const uint32_t kb = ((uint32_t)(sh.E[b] + (1 << 18)) << 8) | (uint32_t)(r * k.A + lab);
-      if (kb < key) {
-        key = kb;
-        bestb = b;
-      }
-    }
-    const uint32_t mn = __reduce_min_sync(0xFFFFFFFFu, key);
-    // the lane holding the minimum (keys are distinct), or lane 0 if no
-    // buffer holds a temperature
-    if (mn != 0xFFFFFFFFu ? key == mn : lane == 0) {
-      const int bestE = mn != 0xFFFFFFFFu ? (int)(mn >> 8) - (1 << 18) : 0x7FFFFFFF;
-      int flag = 0;
-      if ((int64_t)bestE < sh.m64[0]) {
-        sh.m64[0] = bestE;
-        sh.m64[1] = sweeps;
-        sh.m32[0] = 8 * sh.gmap[bestb >> 3] + (bestb & 7);
-        sh.m32[7] = bestb;
-        flag = 1;
-      }
-      if (sh.m64[2] < 0 && sh.m64[0] <= sh.m64[3]) sh.m64[2] = sweeps;
-      sh.m32[1] = flag;
+// Warp 0, after the barrier that ends an energy pass: E_b = nbonds - 2
+// (satisfied bonds), the accumulators back to 0 (half: label 0 was counted
+// alone after a cluster move, which keeps each pair's E_a + E_b, so label 1
+// follows), then the minimum-energy selection (Algorithm S2 output): strict
+// improvement, lowest slot index (r * A + a) on ties.  The two CTAs of a
+// split problem track their own candidates (rank 1 into a scratch state) and
+// combine them at the end of the launch: the global best is the lower
+// energy, found at the earlier sweep, rank 0 (the lower slots) on ties, and
+// the target is first hit at the earlier of the two hits.  m32[1] tells the
+// CTA that the state of buffer m32[7] is to be kept (copy_best).
+__device__ __noinline__ void measure(int half, int64_t sweeps) {
+  Ctl &k = ctl();
+  const int lane = threadIdx.x, n = half ? 8 * k.Gu : 8 * k.Gc;
+  for (int b = lane; b < n; b += 32) {
+    const int e0 = k.nbonds - 2 * k.Eacc[b];
+    if (half) k.E[b + n] += k.E[b] - e0;
+    k.E[b] = e0;
+    k.Eacc[b] = 0;
+  }
+  __syncwarp();
+  // one warp minimum of the key (E + 2^18) 2^8 + slot (|E| <= 3N < 2^18, slot < 2^8)
+  uint32_t key = 0xFFFFFFFFu;
+  int bestb = 0;
+  for (int b = lane; b < 8 * k.Gc; b += 32) {
+    const int lg = b >> 3, lab = lg / k.Gu, r = 8 * (k.g0 + lg - lab * k.Gu) + (b & 7);
+    if (r >= k.T) continue;
+    const uint32_t kb = ((uint32_t)(k.E[b] + (1 << 18)) << 8) | (uint32_t)(r * k.A + lab);
+    if (kb < key) {
+      key = kb;
+      bestb = b;
     }
   }
-  __syncthreads();
-  if (sh.m32[1]) {
-    const int b = sh.m32[7];
-    const int g = b >> 3, i = b & 7;
-    const AptProbDev &P = a.prob[p];
-    int8_t *dst = (k.rank ? a.best_spins2 : a.best_spins) + P.best_off;
-    for (int kk = threadIdx.x; kk < k.geo.N; kk += blockDim.x) {
-      const int c = kk >= k.geo.H ? 1 : 0, j = kk - c * k.geo.H;
-      const uint32_t w = sh.S[(size_t)(2 * g + c) * k.geo.H + j];
-      dst[lin_of(k.geo, c, j)] = ((w >> (4 * i)) & 1u) ? 1 : -1;
+  const uint32_t mn = __reduce_min_sync(0xFFFFFFFFu, key);
+  // the lane holding the minimum (keys are distinct), or lane 0 if no buffer holds a temperature
+  if (mn != 0xFFFFFFFFu ? key == mn : lane == 0) {
+    const int bestE = mn != 0xFFFFFFFFu ? (int)(mn >> 8) - (1 << 18) : 0x7FFFFFFF;
+    int flag = 0;
+    if ((int64_t)bestE < k.m64[0]) {
+      k.m64[0] = bestE;
+      k.m64[1] = sweeps;
+      k.m32[0] = 8 * k.gmap[bestb >> 3] + (bestb & 7);
+      k.m32[7] = bestb;
+      flag = 1;
     }
+    if (k.m64[2] < 0 && k.m64[0] <= k.m64[3]) k.m64[2] = sweeps;
+    k.m32[1] = flag;
   }
-  __syncthreads();
+  __syncwarp();
+}
+
+// The state of a new best replica, in lin order.
+__device__ __noinline__ void copy_best() {
+  Ctl &k = ctl();
+  uint32_t *S = dyn_smem() + k.oS;
+  const int b = k.m32[7], g = b >> 3, i = b & 7;
+  int8_t *dst = k.best_spins;
+  for (int kk = threadIdx.x; kk < k.N; kk += blockDim.x) {
+    const int c = kk >= k.H ? 1 : 0, j = kk - c * k.H;
+    dst[lin_of(k, c, j)] = ((spin_word(k, S, g, kk) >> (4 * i)) & 1u) ? 1 : -1;
+  }
 }
 
 // 32 x 32 bit-matrix transpose across a warp: lane l holds row l on entry
@@ -497,13 +542,14 @@ __device__ __forceinline__ void uf_union(uint32_t *L, uint32_t a, uint32_t b) {
 // clusters, the k-th root, k = floor(x0 n / 2^32), seeds the pair's flood
 // fill.  The labels use the transposed-overlap words, which this rule does
 // not need; R holds one root bit per site.
-__device__ __forceinline__ void icm_cluster_seeds(const Cta &k, const Shared &sh, int nbits, int r0, int P) {
+__device__ __forceinline__ void icm_cluster_seeds(Ctl &k, int nbits, int r0, int P) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const int N = k.geo.N, H = k.geo.H, nchunk = (N + 31) >> 5;
-  uint32_t *V = sh.V, *X = sh.V + N, *Lb = sh.V + 2 * N, *R = sh.V + 2 * N + 32 * nchunk;
+  const int N = k.N, H = k.H, nchunk = (N + 31) >> 5;
+  uint32_t *V = dyn_smem() + k.oV, *X = V + N, *Lb = V + 2 * N, *R = V + 2 * N + 32 * nchunk;
+  const uint32_t *jn = dyn_smem() + k.oJn;
   volatile uint32_t *Lv = Lb;
   for (int pb = 0; pb < nbits; ++pb) {
-    if (r0 + 8 * ((pb >> 3) >> (P - 1)) + (pb & 7) >= k.T || sh.inm[pb] == 0) continue;
+    if (r0 + 8 * ((pb >> 3) >> (P - 1)) + (pb & 7) >= k.T || k.inm[pb] == 0) continue;
     for (int kk = tid; kk < N; kk += nt) Lb[kk] = ((X[kk] >> pb) & 1u) ? (uint32_t)kk : 0xFFFFFFFFu;
     __syncthreads();
     // every bond has one colour-0 end: unite each colour-0 mismatch site
@@ -511,8 +557,8 @@ __device__ __forceinline__ void icm_cluster_seeds(const Cta &k, const Shared &sh
     for (int j = tid; j < H; j += nt) {
       if (!((X[j] >> pb) & 1u)) continue;
       int nb[6];
-      neighbours(k.geo, 0, j, nb);
-      const uint32_t miss = ((uint32_t)sh.jn[j] >> 8) & 0x3Fu;
+      neighbours(k, j, jn[j], nb);
+      const uint32_t miss = (jn[j] >> 8) & 0x3Fu;
 #pragma unroll
       for (int d = 0; d < 6; ++d) {
         const int kk2 = H + nb[d];
@@ -532,7 +578,7 @@ __device__ __forceinline__ void icm_cluster_seeds(const Cta &k, const Shared &sh
       for (int ch = lane; ch < nchunk; ch += 32) tot += __popc(R[ch]);
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xFFFFFFFFu, tot, o);
-      const int kth = (int)(((uint64_t)sh.ikx[pb] * (uint64_t)tot) >> 32);
+      const int kth = (int)(((uint64_t)k.ikx[pb] * (uint64_t)tot) >> 32);
       int base = 0;
       for (int ch0 = 0; ch0 < nchunk; ch0 += 32) {
         const int ch = ch0 + lane;
@@ -577,83 +623,94 @@ __device__ __forceinline__ void icm_cluster_seeds(const Cta &k, const Shared &sh
 // V <- V | (X & OR_nbr V) until no cluster changes.  Clusters larger than
 // N/2 flip one whole replica (x1 bit 0: the pair's first or second label),
 // smaller ones flip in both replicas; then the energies are updated.
-template <bool CSEED>
-__device__ void icm_all(const AptArgs &a, const Cta &k, const Shared &sh, uint32_t t) {
-  long long pt = clock64();
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const int N = k.geo.N, H = k.geo.H;
-  // A labels per temperature form A/2 pairs; label l's groups are
-  // l*Gl .. l*Gl + Gl - 1.  Pair p of temperature r = 8h + i owns bit
-  // 8 (h P + p) + i of the per-site overlap / cluster words.
-  const int A = k.A, P = A >> 1, Gl = k.Gu, nbits = 8 * Gl * P;   // A is 2 or 4
-  const int r0 = 8 * k.g0;   // first temperature held here
-  const uint32_t *S = sh.S;
-  uint32_t *V = sh.V;          // [2][H] cluster bits (one bit per pair)
-  uint32_t *X = sh.V + N;      // [2][H] overlap bits
-  int *match = sh.ibit + 32;   // [32] matching of the labels of each temperature
-  if (tid < nbits) {
-    const int pb = tid, beta = pb >> 3, h = beta >> (P - 1), p = beta - h * P, r = r0 + 8 * h + (pb & 7);
-    if (r < k.T) {
-      const uint4 x = philox((uint32_t)r, t, (uint32_t)p, (k.ent << 8) | TAG_ICM, a.k0, a.k1);
-      sh.ikx[pb] = x.x;
-      sh.ibit[pb] = (int)(x.y & 1u);
-      // Algorithm S2 "randomly partition ICM replicas into pairs": with four
-      // labels, one of the three perfect matchings, floor(3 x2 / 2^32) of
-      // pair 0's draw; two labels always pair (0, 1)
-      if (p == 0) match[r] = A == 4 ? (int)(((uint64_t)x.z * 3u) >> 32) : 0;
+// Overlap bits of one site: the XOR of the two labels' words of each pair,
+// nibbles packed to bits (pair bit 8 (h A/2 + p) + i).  p points at the
+// site's words of quad 0, p1 at those of quad 1.
+template <int A, int GL>
+__device__ __forceinline__ uint32_t site_overlap(const Ctl &k, const uint32_t *p, const uint32_t *p1) {
+  uint32_t xb = 0;
+  if constexpr (A == 2) {
+    constexpr int NW = GL <= 2 ? 2 * GL : GL;   // one quad holds both labels, or each label its own
+    uint32_t w[NW], w1[GL];
+    load_vec<NW>(p, w);
+    if constexpr (GL > 2) load_vec<GL>(p1, w1);
+#pragma unroll
+    for (int h = 0; h < GL; ++h) xb |= nib_to_byte(w[h] ^ (GL > 2 ? w1[h] : w[NW - GL + h])) << (8 * h);
+  } else {
+    // the two labels of pair p depend on each temperature's matching:
+    // select nibbles by the matching masks
+    uint32_t w[4 * GL];
+    {
+      uint32_t t[4];
+      load_vec<4>(p, t);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) w[i] = t[i];
+      if constexpr (GL == 2) {
+        load_vec<4>(p1, t);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[4 * GL - 4 + i] = t[i];
+      }
+    }
+#pragma unroll
+    for (int h = 0; h < GL; ++h) {
+      const uint32_t w0 = w[h], wa = w[GL + h], wb = w[2 * GL + h], wc = w[3 * GL + h];
+      const uint32_t m0 = k.swm[16 + 3 * h], m1 = k.swm[17 + 3 * h], m2 = k.swm[18 + 3 * h];
+      const uint32_t x0 = ((w0 ^ wa) & m0) | ((w0 ^ wb) & m1) | ((w0 ^ wc) & m2);
+      const uint32_t x1 = ((wb ^ wc) & m0) | ((wa ^ wc) & m1) | ((wa ^ wb) & m2);
+      xb |= (nib_to_byte(x0) << (16 * h)) | (nib_to_byte(x1) << (16 * h + 8));
     }
   }
-  if (tid < 24) sh.imask[tid] = 0;
-  if (tid < 64) {
-    sh.isz[tid] = 0;
-    sh.inm[tid] = 0;
-  }
-  __syncthreads();
-  if (A == 4 && tid < 3 * Gl) {
-    // nibble masks of the temperatures of group h that use matching m
-    const int h = tid / 3, m = tid - 3 * h;
-    uint32_t mk = 0;
-    for (int i = 0; i < 8; ++i) {
-      const int r = r0 + 8 * h + i;
-      if (r < k.T && match[r] == m) mk |= 0xFu << (4 * i);
+  return xb;
+}
+
+// The cluster moves of one site: cluster bits v, flip masks imask.
+template <int A, int GL>
+__device__ __forceinline__ void site_flip(const Ctl &k, uint32_t *p, uint32_t *p1, uint32_t v, const uint32_t (&fm)[4 * GL]) {
+  if constexpr (A == 2) {
+    constexpr int NW = GL <= 2 ? 2 * GL : GL;
+    uint32_t w[NW], w1[GL];
+    load_vec<NW>(p, w);
+    if constexpr (GL > 2) load_vec<GL>(p1, w1);
+#pragma unroll
+    for (int h = 0; h < GL; ++h) {
+      const uint32_t vv = byte_to_nib((v >> (8 * h)) & 0xFFu);
+      w[h] ^= (vv & fm[4 * h]) | fm[4 * h + 1];
+      (GL > 2 ? w1[h] : w[NW - GL + h]) ^= (vv & fm[4 * h + 2]) | fm[4 * h + 3];
     }
-    sh.swm[16 + tid] = mk;
+    store_vec<NW>(p, w);
+    if constexpr (GL > 2) store_vec<GL>(p1, w1);
+  } else {
+#pragma unroll
+    for (int q = 0; q < GL; ++q) {
+      uint32_t *pq = q ? p1 : p, w[4];
+      load_vec<4>(pq, w);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int g = 4 * q + u, h = g % GL;   // g = label GL + h
+        const uint32_t n0 = byte_to_nib((v >> (16 * h)) & 0xFFu), n1 = byte_to_nib((v >> (16 * h + 8)) & 0xFFu);
+        w[u] ^= k.imask[16 + g] | (n0 & k.imask[2 * g]) | (n1 & k.imask[2 * g + 1]);
+      }
+      store_vec<4>(pq, w);
+    }
   }
-  __syncthreads();
-  // (A) overlaps.  Warp w takes chunks of 32 sites in canonical order; the
-  // transpose of the chunk's X words gives lane r the chunk's mismatch
-  // bitmask of pair r, kept in Xt[chunk][r].
-  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5, nchunk = (N + 31) >> 5;
-  uint32_t *Xt = sh.V + 2 * N;   // [nchunk][32]
+}
+
+// (A) overlaps.  Warp w takes chunks of 32 sites in canonical order; the
+// transpose of the chunk's X words gives lane r the chunk's mismatch
+// bitmask of pair r, kept in Xt[chunk][r].
+template <int A, int GL>
+__device__ __forceinline__ void icm_overlaps(Ctl &k, int nbits) {
+  constexpr int W = A * GL == 2 ? 2 : 4;   // words per site and quad
+  const int N = k.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, nchunk = (N + 31) >> 5;
+  const uint32_t *S = dyn_smem() + k.oS, *jn = dyn_smem() + k.oJn;
+  uint32_t *V = dyn_smem() + k.oV, *X = V + N, *Xt = V + 2 * N;
   uint32_t nmis = 0;             // lane r: mismatches of pair r in this warp's chunks
   for (int ch = warp; ch < nchunk; ch += nw) {
     const int kk = ch * 32 + lane;
     uint32_t xb = 0;
     if (kk < N) {
-      const int c = kk >= H ? 1 : 0, j = kk - c * H;
-      if (A == 2) {
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          if (h >= Gl) break;
-          const uint32_t x = S[(2 * h + c) * H + j] ^ S[(2 * (h + Gl) + c) * H + j];
-          xb |= nib_to_byte(x) << (8 * h);
-        }
-      } else {
-        // the two labels of pair p depend on each temperature's matching:
-        // select nibbles by the matching masks
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (h >= Gl) break;
-          uint32_t w[4];
-#pragma unroll
-          for (int l = 0; l < 4; ++l) w[l] = S[(2 * (l * Gl + h) + c) * H + j];
-          const uint32_t m0 = sh.swm[16 + 3 * h], m1 = sh.swm[17 + 3 * h], m2 = sh.swm[18 + 3 * h];
-          const uint32_t x0 = ((w[0] ^ w[1]) & m0) | ((w[0] ^ w[2]) & m1) | ((w[0] ^ w[3]) & m2);
-          const uint32_t x1 = ((w[2] ^ w[3]) & m0) | ((w[1] ^ w[3]) & m1) | ((w[1] ^ w[2]) & m2);
-          xb |= (nib_to_byte(x0) << (16 * h)) | (nib_to_byte(x1) << (16 * h + 8));
-        }
-      }
-      if (sh.jn[kk] & 0x8000u) xb = 0;   // a vacancy has no overlap: never a seed or member
+      xb = site_overlap<A, GL>(k, S + kk * W, S + (N + kk) * W);
+      if (jn[kk] & 0x8000u) xb = 0;   // a vacancy has no overlap: never a seed or member
       X[kk] = xb;
       V[kk] = 0u;
     }
@@ -661,18 +718,103 @@ __device__ void icm_all(const AptArgs &a, const Cta &k, const Shared &sh, uint32
     Xt[ch * 32 + lane] = col;
     nmis += __popc(col);
   }
-  if (lane < nbits && nmis) atomicAdd(&sh.inm[lane], (int)nmis);
+  if (lane < nbits && nmis) atomicAdd(&k.inm[lane], (int)nmis);
+}
+
+// (E) flips, the masks read once into registers.
+template <int A, int GL>
+__device__ __forceinline__ void icm_flips(Ctl &k) {
+  constexpr int W = A * GL == 2 ? 2 : 4;   // words per site and quad
+  const int N = k.N;
+  uint32_t *S = dyn_smem() + k.oS;
+  const uint32_t *V = dyn_smem() + k.oV;
+  uint32_t fm[4 * GL];
+  if constexpr (A == 2) {
+#pragma unroll
+    for (int h = 0; h < GL; ++h) {
+      fm[4 * h] = k.imask[h];
+      fm[4 * h + 1] = k.imask[16 + h];
+      fm[4 * h + 2] = k.imask[GL + h];
+      fm[4 * h + 3] = k.imask[16 + GL + h];
+    }
+  }
+  for (int kk = threadIdx.x; kk < N; kk += blockDim.x)
+    site_flip<A, GL>(k, S + kk * W, S + (N + kk) * W, V[kk], fm);
+}
+
+template <bool CSEED>
+__device__ __noinline__ void icm_all(uint32_t t) {
+  Ctl &k = ctl();
+#if PC_APT_PROFILE
+  long long pt = clock64();
+#endif
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int N = k.N, H = k.H;
+  // A labels per temperature form A/2 pairs; label l's groups are
+  // l*Gl .. l*Gl + Gl - 1.  Pair p of temperature r = 8h + i owns bit
+  // 8 (h P + p) + i of the per-site overlap / cluster words.
+  const int A = k.A, P = A >> 1, Gl = k.Gu, nbits = 8 * Gl * P;   // A is 2 or 4
+  const int r0 = 8 * k.g0;   // first temperature held here
+  uint32_t *V = dyn_smem() + k.oV;   // [2][H] cluster bits (one bit per pair)
+  uint32_t *X = V + N;               // [2][H] overlap bits
+  uint32_t *Xt = V + 2 * N;          // [nchunk][32]
+  int *match = k.ibit + 32;          // [32] matching of the labels of each temperature
+  if (tid < nbits) {
+    const int pb = tid, beta = pb >> 3, h = beta >> (P - 1), p = beta - h * P, r = r0 + 8 * h + (pb & 7);
+    if (r < k.T) {
+      const uint4 x = philox((uint32_t)r, t, (uint32_t)p, (k.ent << 8) | TAG_ICM, k.k0, k.k1);
+      k.ikx[pb] = x.x;
+      k.ibit[pb] = (int)(x.y & 1u);
+      // Algorithm S2 "randomly partition ICM replicas into pairs": with four
+      // labels, one of the three perfect matchings, floor(3 x2 / 2^32) of
+      // pair 0's draw; two labels always pair (0, 1)
+      if (p == 0) match[r] = A == 4 ? (int)(((uint64_t)x.z * 3u) >> 32) : 0;
+    }
+  }
+  if (tid < 24) k.imask[tid] = 0;
+  if (tid < 64) {
+    k.isz[tid] = 0;
+    k.inm[tid] = 0;
+  }
+  __syncthreads();
+  if (k.m32[1]) copy_best();
+  if (A == 4) {
+    if (tid < 3 * Gl) {
+      // nibble masks of the temperatures of group h that use matching m
+      const int h = tid / 3, m = tid - 3 * h;
+      uint32_t mk = 0;
+      for (int i = 0; i < 8; ++i) {
+        const int r = r0 + 8 * h + i;
+        if (r < k.T && match[r] == m) mk |= 0xFu << (4 * i);
+      }
+      k.swm[16 + tid] = mk;
+    }
+    __syncthreads();
+  }
+  const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5, nchunk = (N + 31) >> 5;
+  if (A == 2) {
+    switch (Gl) {
+      case 4: icm_overlaps<2, 4>(k, nbits); break;
+      case 3: icm_overlaps<2, 3>(k, nbits); break;
+      case 2: icm_overlaps<2, 2>(k, nbits); break;
+      default: icm_overlaps<2, 1>(k, nbits); break;
+    }
+  } else if (Gl == 2) {
+    icm_overlaps<4, 2>(k, nbits);
+  } else {
+    icm_overlaps<4, 1>(k, nbits);
+  }
   __syncthreads();
   PROF_MARK(4, pt);
   // seeds: warp w finds the k-th mismatch of pairs w, w + nw, ...: chunk
   // counts by popcount, a warp scan over chunks, then the set bit inside
   // the chunk (the cluster-seed rule finds the k-th cluster instead)
-  if (CSEED) icm_cluster_seeds(k, sh, nbits, r0, P);
+  if (CSEED) icm_cluster_seeds(k, nbits, r0, P);
   for (int r = warp; r < nbits && !CSEED; r += nw) {   // r: pair bit
     if (r0 + 8 * ((r >> 3) >> (P - 1)) + (r & 7) >= k.T) continue;
-    const int nm = sh.inm[r];
+    const int nm = k.inm[r];
     if (nm == 0) continue;
-    const int kth = (int)(((uint64_t)sh.ikx[r] * (uint64_t)nm) >> 32);
+    const int kth = (int)(((uint64_t)k.ikx[r] * (uint64_t)nm) >> 32);
     int base = 0;
     for (int ch0 = 0; ch0 < nchunk; ch0 += 32) {
       const int ch = ch0 + lane;
@@ -716,7 +858,7 @@ __device__ void icm_all(const AptArgs &a, const Cta &k, const Shared &sh, uint32
   // growth) and a pass with no change anywhere, started after a barrier,
   // proves the fixed point.
   {
-    const Geo &g = k.geo;
+    const Ctl &g = k;
     const int hx = g.hx, hy = g.Ly >> 1, nblk = N >> 3;
     // plain loads: a pass reads each neighbour word once, after the barrier
     // that ended the previous pass (a compiler fence as well), and a value
@@ -861,7 +1003,7 @@ __device__ void icm_all(const AptArgs &a, const Cta &k, const Shared &sh, uint32
       const int kk = ch * 32 + lane;
       sz += __popc(warp_transpose32(kk < N ? V[kk] : 0u));
     }
-    if (lane < nbits && sz) atomicAdd(&sh.isz[lane], (int)sz);
+    if (lane < nbits && sz) atomicAdd(&k.isz[lane], (int)sz);
   }
   __syncthreads();
   // (D) decisions.  imask[(g P + p)] (g = l Gl + h): nibbles of label l's
@@ -873,144 +1015,117 @@ __device__ void icm_all(const AptArgs &a, const Cta &k, const Shared &sh, uint32
       const int m = match[r];
       const int la = p == 0 ? 0 : (m == 0 ? 2 : 1);
       const int lb = p == 0 ? m + 1 : (m == 2 ? 2 : 3);
-      const int size = sh.isz[pb];
+      const int size = k.isz[pb];
       const uint32_t bit = 1u << (4 * i);
-      if (sh.inm[pb] == 0) {
-        atomicAdd(&sh.m32[2], 1);
-      } else if (a.icm_big && 2 * size > k.nreal) {   // more than half of the spins present
-        atomicOr(&sh.imask[16 + (sh.ibit[pb] ? lb : la) * Gl + h], bit);   // one whole replica
-        atomicAdd(&sh.m32[4], 1);
+      if (k.inm[pb] == 0) {
+        atomicAdd(&k.m32[2], 1);
+      } else if (k.icm_big && 2 * size > k.nreal) {   // more than half of the spins present
+        atomicOr(&k.imask[16 + (k.ibit[pb] ? lb : la) * Gl + h], bit);   // one whole replica
+        atomicAdd(&k.m32[4], 1);
       } else {
-        atomicOr(&sh.imask[(la * Gl + h) * P + p], bit);                  // cluster, both replicas
-        atomicOr(&sh.imask[(lb * Gl + h) * P + p], bit);
-        atomicAdd(&sh.m32[3], 1);
+        atomicOr(&k.imask[(la * Gl + h) * P + p], bit);                  // cluster, both replicas
+        atomicOr(&k.imask[(lb * Gl + h) * P + p], bit);
+        atomicAdd(&k.m32[3], 1);
       }
     }
   }
   __syncthreads();
   PROF_MARK(7, pt);
-  // (E) flips.  With two labels the masks are read once into registers (a
-  // store to S could alias them, so they would be reloaded after every one)
-  uint32_t fm[4][4];
-#pragma unroll
-  for (int h = 0; h < 4; ++h) {
-    const bool on = A == 2 && h < Gl;
-    fm[h][0] = on ? sh.imask[h] : 0u;
-    fm[h][1] = on ? sh.imask[16 + h] : 0u;
-    fm[h][2] = on ? sh.imask[Gl + h] : 0u;
-    fm[h][3] = on ? sh.imask[16 + Gl + h] : 0u;
-  }
-  for (int kk = tid; kk < N; kk += nt) {
-    const int c = kk >= H ? 1 : 0, j = kk - c * H;
-    const uint32_t v = V[kk];
-    if (A == 2) {
-#pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        if (h >= Gl) break;
-        const uint32_t vv = byte_to_nib((v >> (8 * h)) & 0xFFu);
-        uint32_t *p0 = sh.S + (size_t)(2 * h + c) * H + j, *p1 = sh.S + (size_t)(2 * (Gl + h) + c) * H + j;
-        const uint32_t a0 = *p0, a1 = *p1;
-        *p0 = a0 ^ ((vv & fm[h][0]) | fm[h][1]);
-        *p1 = a1 ^ ((vv & fm[h][2]) | fm[h][3]);
-      }
-    } else {
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (h >= Gl) break;
-        const uint32_t n0 = byte_to_nib((v >> (16 * h)) & 0xFFu);
-        const uint32_t n1 = byte_to_nib((v >> (16 * h + 8)) & 0xFFu);
-#pragma unroll
-        for (int l = 0; l < 4; ++l) {
-          const int g = l * Gl + h;
-          sh.S[(2 * g + c) * H + j] ^= sh.imask[16 + g] | (n0 & sh.imask[2 * g]) | (n1 & sh.imask[2 * g + 1]);
-        }
-      }
+  if (A == 2) {
+    switch (Gl) {
+      case 4: icm_flips<2, 4>(k); break;
+      case 3: icm_flips<2, 3>(k); break;
+      case 2: icm_flips<2, 2>(k); break;
+      default: icm_flips<2, 1>(k); break;
     }
+  } else if (Gl == 2) {
+    icm_flips<4, 2>(k);
+  } else {
+    icm_flips<4, 1>(k);
   }
   __syncthreads();
   PROF_MARK(8, pt);
-  // (F) energies after the moves.  A Houdayer move keeps E_a + E_b of its
-  // pair (the cluster's outside neighbours agree in both replicas; a whole
-  // replica flip changes no energy at h = 0), so only label 0 is recounted
-  // and label 1 follows as E_b' = E_a + E_b - E_a'.
-  if (A == 2) {
-    colour_phase<false, true>(a, k, sh, 1, 0u, Gl);
-    __syncthreads();
-    for (int b = tid; b < 8 * Gl; b += nt) {
-      const int e0 = k.nbonds - 2 * sh.Eacc[b];
-      sh.E[b + 8 * Gl] += sh.E[b] - e0;
-      sh.E[b] = e0;
-      sh.Eacc[b] = 0;
-    }
-  } else {
-    // the pairs change with the temperature: recount every label
-    colour_phase<false, true>(a, k, sh, 1, 0u, k.Gc);
-    __syncthreads();
-    finish_energies(k, sh);
-  }
-  __syncthreads();
-  PROF_MARK(9, pt);
 }
 
-// Applies the swap masks of the last attempt (sh.swm) to the words
-// [kb, ke) of every group plane ([0, H): colour 0, [H, 2H): colour 1).  A
-// split problem's boundary swap (bmask: accepted labels) also writes the
-// peer CTA's spins, pushed into `stage`, into this CTA's boundary nibble.
-__device__ void swap_words(const Cta &k, const Shared &sh, int kb, int ke, uint32_t bmask,
-                           const uint32_t *stage) {
-  const int H = k.geo.H, G = k.Gc;
-  // groups touched by the swaps, and the groups g whose nibble 7 pairs with
-  // nibble 0 of g + 1
-  uint32_t touch = 0, cross = 0;
-#pragma unroll
-  for (int g = 0; g < 8; ++g) {
-    if (g < G && sh.swm[g]) touch |= 1u << g;
-    if (g + 1 < G && sh.swm[8 + g]) cross |= 1u << g;
-  }
+
+// Applies the swap masks of the last attempt (Ctl::swm) to the words of
+// colour c.  The groups that exchange nibbles with one another belong to one
+// label, hence to one quad.  A split problem's boundary swap (bmask:
+// accepted labels) also writes the peer CTA's spins, pushed into `stage`,
+// into this CTA's boundary nibble.
+template <int GQ>
+__device__ __forceinline__ void swap_quads(Ctl &k, int c, uint32_t bmask, const uint32_t *stage) {
+  constexpr int W = GQ == 3 ? 4 : GQ;
+  const int H = k.H;
   // rank 0 receives into nibble 7 of each label's last group, rank 1 into
   // nibble 0 of each label's first group
   const int bsh = k.rank == 0 ? 28 : 0, bgoff = k.rank == 0 ? k.Gu - 1 : 0;
-  for (int kk = kb + threadIdx.x; kk < ke; kk += blockDim.x) {
-    uint32_t *col = sh.S + kk;   // word (g, c, j) at col[g * 2H]
+  for (int quad = 0; quad < k.nq; ++quad) {
+    // in-group nibble masks, pairs (u, u + 1) whose nibbles 7 and 0 exchange,
+    // and the labels whose boundary group lies in this quad
+    uint32_t m[GQ], cross = 0, any = 0, bl[GQ];
 #pragma unroll
-    for (int g = 0; g < 8; ++g) {
-      if ((touch >> g) & 1u) {
-        const uint32_t w = col[(size_t)g * 2 * H], m = sh.swm[g];
-        const uint32_t d = (w ^ (w >> 4)) & m;
-        col[(size_t)g * 2 * H] = w ^ (d | (d << 4));
+    for (int u = 0; u < GQ; ++u) {
+      const int g = quad * GQ + u;
+      m[u] = g < k.Gc ? k.swm[g] : 0u;
+      any |= m[u];
+      if (u + 1 < GQ && g + 1 < k.Gc && k.swm[8 + g]) cross |= 1u << u;
+      bl[u] = 0u;
+      if (bmask && g < k.Gc) {
+        const int l = g / k.Gu;
+        if (g - l * k.Gu == bgoff && ((bmask >> l) & 1u)) bl[u] = (uint32_t)(64 * l) + 1u;   // 1 + its stage row
+        any |= bl[u];
       }
     }
+    if (!(any | cross)) continue;
+    uint32_t *Sq = dyn_smem() + k.oS + (2 * quad + c) * H * W;
+    for (int j = threadIdx.x; j < H; j += blockDim.x) {
+      uint32_t w[GQ];
+      load_vec<GQ>(Sq + j * W, w);
 #pragma unroll
-    for (int g = 0; g < 7; ++g) {
-      if ((cross >> g) & 1u) {
-        const uint32_t w0 = col[(size_t)g * 2 * H], w1 = col[(size_t)(g + 1) * 2 * H];
-        const uint32_t d = ((w0 >> 28) ^ w1) & 1u;
-        col[(size_t)g * 2 * H] = w0 ^ (d << 28);
-        col[(size_t)(g + 1) * 2 * H] = w1 ^ d;
+      for (int u = 0; u < GQ; ++u) {
+        const uint32_t d = (w[u] ^ (w[u] >> 4)) & m[u];
+        w[u] ^= d | (d << 4);
       }
-    }
-    if (bmask) {
-      const int e = kk - kb;
-      for (int l = 0; l < k.A; ++l) {
-        if (!((bmask >> l) & 1u)) continue;
-        const uint32_t bit = (stage[64 * l + (e >> 5)] >> (e & 31)) & 1u;
-        uint32_t *wp = col + (size_t)(l * k.Gu + bgoff) * 2 * H;
-        *wp = (*wp & ~(1u << bsh)) | (bit << bsh);
-      }
+#pragma unroll
+      for (int u = 0; u + 1 < GQ; ++u)
+        if ((cross >> u) & 1u) {
+          const uint32_t d = ((w[u] >> 28) ^ w[u + 1]) & 1u;
+          w[u] ^= d << 28;
+          w[u + 1] ^= d;
+        }
+#pragma unroll
+      for (int u = 0; u < GQ; ++u)
+        if (bl[u]) {
+          const uint32_t bit = (stage[bl[u] - 1u + (uint32_t)(j >> 5)] >> (j & 31)) & 1u;
+          w[u] = (w[u] & ~(1u << bsh)) | (bit << bsh);
+        }
+      store_vec<GQ>(Sq + j * W, w);
     }
   }
 }
+__device__ __noinline__ void swap_words(int c, uint32_t bmask, int par) {
+  Ctl &k = ctl();
+  const uint32_t *stage = dyn_smem() + k.oStage + 256 * par;
+  switch (k.gq) {
+    case 4: swap_quads<4>(k, c, bmask, stage); break;
+    case 3: swap_quads<3>(k, c, bmask, stage); break;
+    case 2: swap_quads<2>(k, c, bmask, stage); break;
+    default: swap_quads<1>(k, c, bmask, stage); break;
+  }
+}
 
-// Split problems: writes this CTA's boundary spins of the words
-// [kb, kb + H) (one colour), every label, one bit per site, into the peer
-// CTA's stage[par] (distributed shared memory).  Rank 0 sends the last
-// (coldest) temperature of its half (nibble 7 of each label's last group),
-// rank 1 the first (hottest) of its half (nibble 0 of each label's first
-// group).
-__device__ void push_boundary(const Cta &k, const Shared &sh, int kb, int par, int w0 = 0) {
+// Split problems: writes this CTA's boundary spins of colour c, every
+// label, one bit per site, into the peer CTA's stage[par] (distributed
+// shared memory).  Rank 0 sends the last (coldest) temperature of its half
+// (nibble 7 of each label's last group), rank 1 the first (hottest) of its
+// half (nibble 0 of each label's first group).
+__device__ __noinline__ void push_boundary(int c, int par, int w0) {
   namespace cg = cooperative_groups;
-  const int H = k.geo.H;
-  uint32_t *pstage = cg::this_cluster().map_shared_rank(sh.stage, k.rank ^ 1) + 256 * par;
+  Ctl &k = ctl();
+  const int H = k.H;
+  uint32_t *S = dyn_smem() + k.oS;
+  uint32_t *pstage = cg::this_cluster().map_shared_rank(dyn_smem() + k.oStage, k.rank ^ 1) + 256 * par;
   const int sh_own = k.rank == 0 ? 28 : 0, goff = k.rank == 0 ? k.Gu - 1 : 0;
   // warps w0 .. take part
   const int lane = threadIdx.x & 31, nw = (blockDim.x >> 5) - w0;
@@ -1018,13 +1133,12 @@ __device__ void push_boundary(const Cta &k, const Shared &sh, int kb, int par, i
     const int e = base + lane;
     for (int l = 0; l < k.A; ++l) {
       uint32_t bit = 0;
-      if (e < H) bit = (sh.S[(size_t)(l * k.Gu + goff) * 2 * H + kb + e] >> sh_own) & 1u;
+      if (e < H) bit = (spin_word(k, S, l * k.Gu + goff, c * H + e) >> sh_own) & 1u;
       const uint32_t word = __ballot_sync(0xFFFFFFFFu, bit);
       if (lane == 0) pstage[64 * l + (base >> 5)] = word;
     }
   }
 }
-
 // Replica exchange of attempt t (Sec. "Comparison with Adaptive Parallel
 // Tempering"; Methods): even t pairs (0,1),(2,3)..., odd t (1,2),(3,4)...;
 // each label decides on its own; p_swap = min(1, exp(dbeta dE)).  Accepted
@@ -1035,78 +1149,78 @@ __device__ void push_boundary(const Cta &k, const Shared &sh, int kb, int par, i
 // for the accepted labels.  Buffers alternate with the attempt's parity, so
 // one barrier per attempt orders every exchange.
 template <bool SPLIT>
-__device__ void swap_step(const AptArgs &a, const Cta &k, const Shared &sh, int p, uint32_t t) {
+__device__ __noinline__ void swap_step(uint32_t t) {
+  Ctl &k = ctl();
 #if PC_APT_PROFILE
   long long pt = clock64();
 #endif
-  const AptProbDev &P = a.prob[p];
   const int A = k.A, q = (int)(t & 1u);
   const int r0 = 8 * k.g0, r1 = min(8 * (k.g0 + k.Gu), k.T);   // temperatures held here
   // local buffer of (label l, temperature r): l * 8 Gu + r - r0
   const int lb = 8 * k.Gu;
   auto swap_table = [&](int r, int dE) {
     const int kk = (-dE) >> 1;
-    if (PC_APT_STAGE_SWT && SPLIT && a.stage_swt && kk < kSwtLen) return sh.swt[r * kSwtLen + kk];   // staged at launch
-    const uint32_t off = a.swapidx[P.swapidx_off + 2 * r], len = a.swapidx[P.swapidx_off + 2 * r + 1];
-    return ((uint32_t)kk < len) ? a.swaptab[off + kk] : 0u;
+    if (PC_APT_STAGE_SWT && SPLIT && k.stage_swt && kk < kSwtLen) return dyn_smem()[k.oSwt + r * kSwtLen + kk];   // staged at launch
+    const uint32_t off = k.swapidx[2 * r], len = k.swapidx[2 * r + 1];
+    return ((uint32_t)kk < len) ? k.swaptab[off + kk] : 0u;
   };
   const int par = (int)(t & 1u);
   const int warp = threadIdx.x >> 5;
-  if (k.split) {
+  if (SPLIT) {
     // energies of this side of the boundary pair, and its colour-1 spins
     // (warps 1 ..; warp 0 starts on the decisions meanwhile)
     const int rb_own = k.rank == 0 ? r1 - 1 : r0;
-    int *pe = cooperative_groups::this_cluster().map_shared_rank(sh.xch, k.rank ^ 1) + 4 * par;
-    if (threadIdx.x < A) pe[threadIdx.x] = sh.E[threadIdx.x * lb + rb_own - r0];
-    if (warp >= 1) push_boundary(k, sh, k.geo.H, par, 1);
+    int *pe = cooperative_groups::this_cluster().map_shared_rank(k.xch, k.rank ^ 1) + 4 * par;
+    if (threadIdx.x < A) pe[threadIdx.x] = k.E[threadIdx.x * lb + rb_own - r0];
+    if (warp >= 1) push_boundary(1, par, 1);
     // the boundary pair's draws do not depend on the energies: warp 1 takes
     // them now, before the cluster barrier
     const int rb = k.rank == 0 ? r1 : r0;
     const int lane1 = threadIdx.x - 32;
     if (warp == 1 && lane1 < A && rb < k.T && ((rb - 1) & 1) == q)
-      sh.xch[18 + lane1] =
-          (int)philox((uint32_t)(rb - 1), t, (uint32_t)lane1, (k.ent << 8) | TAG_SWAP, a.k0, a.k1).x;
+      k.xch[18 + lane1] =
+          (int)philox((uint32_t)(rb - 1), t, (uint32_t)lane1, (k.ent << 8) | TAG_SWAP, k.k0, k.k1).x;
   }
   PROF_MARK(12, pt);
   if (threadIdx.x < 32) {
     const int lane = threadIdx.x;
-    if (lane < 16) sh.swm[lane] = 0;
+    if (lane < 16) k.swm[lane] = 0;
     __syncwarp();
     const int first = r0 + q;                          // r0 is even
     const int np = r1 - 1 > first ? (r1 - first) / 2 : 0;   // pairs (r, r + 1), r + 1 < r1
     int any = 0;
     // joint mode (Algorithm S2 read literally): lane idx decides pair idx
     // for all labels at once, with the summed energy difference
-    const int nd = a.joint_swap ? np : np * A;
+    const int nd = k.joint ? np : np * A;
     for (int idx = lane; idx < nd; idx += 32) {
-      const int r = first + 2 * (a.joint_swap ? idx : idx / A), al = a.joint_swap ? 0 : idx % A;
+      const int r = first + 2 * (k.joint ? idx : idx / A), al = k.joint ? 0 : idx % A;
       // the draw first: it does not depend on the energies
-      const uint32_t x0 = philox((uint32_t)r, t, (uint32_t)al, (k.ent << 8) | TAG_SWAP, a.k0, a.k1).x;
+      const uint32_t x0 = philox((uint32_t)r, t, (uint32_t)al, (k.ent << 8) | TAG_SWAP, k.k0, k.k1).x;
       const int bA = al * lb + r - r0, bB = bA + 1;
-      int dE = sh.E[bB] - sh.E[bA];
-      if (a.joint_swap)
-        for (int l = 1; l < A; ++l) dE += sh.E[l * lb + r - r0 + 1] - sh.E[l * lb + r - r0];
+      int dE = k.E[bB] - k.E[bA];
+      if (k.joint)
+        for (int l = 1; l < A; ++l) dE += k.E[l * lb + r - r0 + 1] - k.E[l * lb + r - r0];
       const bool acc = dE >= 0 || x0 < swap_table(r, dE);
-      for (int l = al; l < (a.joint_swap ? A : al + 1); ++l) {
+      for (int l = al; l < (k.joint ? A : al + 1); ++l) {
         const int lA = l * lb + r - r0, lB = lA + 1;
-        sh.satt[r * A + l] += 1;
+        k.satt[r * A + l] += 1;
         if (acc) {
-          sh.sacc[r * A + l] += 1;
-          const int eA = sh.E[lA];
-          sh.E[lA] = sh.E[lB];
-          sh.E[lB] = eA;
-          if ((lA & 7) != 7) atomicOr(&sh.swm[lA >> 3], 1u << (4 * (lA & 7)));
-          else sh.swm[8 + (lA >> 3)] = 1u;
+          k.sacc[r * A + l] += 1;
+          const int eA = k.E[lA];
+          k.E[lA] = k.E[lB];
+          k.E[lB] = eA;
+          if ((lA & 7) != 7) atomicOr(&k.swm[lA >> 3], 1u << (4 * (lA & 7)));
+          else k.swm[8 + (lA >> 3)] = 1u;
           any = 1;
         }
       }
     }
     any = __any_sync(0xFFFFFFFFu, any);
-    if (lane == 0) sh.m32[5] = any;
+    if (lane == 0) k.m32[5] = any;
   }
   PROF_MARK(13, pt);
   uint32_t bmask = 0;
-  if (k.split) {
+  if (SPLIT) {
     cooperative_groups::this_cluster().sync();   // the peer's energies and spins have landed
     // the pair (rb - 1, rb) across the two CTAs, if this attempt's parity
     const int rb = k.rank == 0 ? r1 : r0;
@@ -1114,42 +1228,48 @@ __device__ void swap_step(const AptArgs &a, const Cta &k, const Shared &sh, int 
       uint32_t accm = 0;
       if (rb < k.T && ((rb - 1) & 1) == q) {
         const int rb_own = k.rank == 0 ? r1 - 1 : r0;
-        const int *pe = sh.xch + 4 * par;   // the peer's energies
+        const int *pe = k.xch + 4 * par;   // the peer's energies
         int e_lo[4], e_hi[4];               // energies at rb - 1 (rank 0's) and rb (rank 1's)
         for (int l = 0; l < A; ++l) {
-          const int own = sh.E[l * lb + rb_own - r0];
+          const int own = k.E[l * lb + rb_own - r0];
           e_lo[l] = k.rank == 0 ? own : pe[l];
           e_hi[l] = k.rank == 0 ? pe[l] : own;
         }
-        for (int l = 0; l < (a.joint_swap ? 1 : A); ++l) {
+        for (int l = 0; l < (k.joint ? 1 : A); ++l) {
           int dE = e_hi[l] - e_lo[l];
-          if (a.joint_swap)
+          if (k.joint)
             for (int m = 1; m < A; ++m) dE += e_hi[m] - e_lo[m];
           // the draw taken by warp 1 before the barrier
-          const bool acc = dE >= 0 || (uint32_t)sh.xch[18 + l] < swap_table(rb - 1, dE);
-          if (acc) accm |= a.joint_swap ? (1u << A) - 1u : 1u << l;
+          const bool acc = dE >= 0 || (uint32_t)k.xch[18 + l] < swap_table(rb - 1, dE);
+          if (acc) accm |= k.joint ? (1u << A) - 1u : 1u << l;
         }
         for (int l = 0; l < A; ++l) {
-          if (k.rank == 0) sh.satt[(rb - 1) * A + l] += 1;   // counted once, by rank 0
+          if (k.rank == 0) k.satt[(rb - 1) * A + l] += 1;   // counted once, by rank 0
           if ((accm >> l) & 1u) {
-            if (k.rank == 0) sh.sacc[(rb - 1) * A + l] += 1;
-            sh.E[l * lb + rb_own - r0] = k.rank == 0 ? e_hi[l] : e_lo[l];
+            if (k.rank == 0) k.sacc[(rb - 1) * A + l] += 1;
+            k.E[l * lb + rb_own - r0] = k.rank == 0 ? e_hi[l] : e_lo[l];
           }
         }
       }
-      sh.xch[8] = (int)accm;
+      k.xch[8] = (int)accm;
     }
     __syncthreads();
-    bmask = (uint32_t)sh.xch[8];
+    bmask = (uint32_t)k.xch[8];
   } else {
     __syncthreads();
   }
   PROF_MARK(14, pt);
-  if (!sh.m32[5] && !bmask) return;
+  // the measurement before this step may have found a new best state; its
+  // words have not moved yet
+  if (k.m32[1]) {
+    copy_best();
+    __syncthreads();
+  }
+  if (!k.m32[5] && !bmask) return;
   // colour 0 is rewritten by the next sweep without being read (a Gibbs
   // update depends on the neighbours only), so only colour 1 moves now; the
   // kernel applies the last attempt's swaps to colour 0 before it stores
-  swap_words(k, sh, k.geo.H, 2 * k.geo.H, bmask, sh.stage + 256 * par);
+  swap_words(1, bmask, par);
   PROF_MARK(15, pt);
 }
 
@@ -1157,188 +1277,208 @@ __device__ void swap_step(const AptArgs &a, const Cta &k, const Shared &sh, int 
 // template arguments, so that each kernel carries only its own code (the
 // launcher picks the instantiation from a.mode and a.split).
 template <int MODE, bool SPLIT, bool CSEED>
-__global__ void __launch_bounds__(512) apt_kernel(const AptArgs a) {
-  extern __shared__ __align__(16) uint32_t smem[];
+__global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArgs a) {
+  uint32_t *const smem = dyn_smem();
+  Ctl &k = ctl();
   const int cta = blockIdx.x;
   const int p = a.cta_prob[cta];
   const AptProbDev &P = a.prob[p];
-  Cta k;
-  k.geo.Lx = P.Lx;
-  k.geo.Ly = P.Ly;
-  k.geo.Lz = P.Lz;
-  k.geo.N = P.N;
-  k.geo.H = P.N >> 1;
-  k.geo.hx = P.Lx >> 1;
-  k.geo.mhx = P.mhx;
-  k.geo.mLy = P.mLy;
-  k.geo.mLy2 = P.mLy2;
-  k.nbonds = P.nbonds;
-  k.nreal = P.nreal;
-  k.open = P.open;
-  k.T = P.T;
-  k.Tp = P.Tp;
-  k.A = P.A;
-  k.B = P.B;
-  k.g0 = a.cta_g0[cta];
-  k.Gc = a.cta_gc[cta];
-  k.Bc = min(8 * k.Gc, P.B - 8 * k.g0);
-  k.split = SPLIT;
-  k.rank = SPLIT ? (int)cooperative_groups::this_cluster().block_rank() : 0;
-  if (MODE == pc::APT_MODE_APT || MODE == pc::APT_MODE_ENERGY) {
-    k.Gu = k.Gc / k.A;   // A is 1, 2 or 4
-    k.Glp = k.Tp >> 3;
-  } else {
-    k.Gu = k.Gc;
-    k.Glp = (k.B + 7) >> 3;
-  }
-  k.ent = P.ent;
-  k.nch = a.cta_nch[cta];
-  k.tpc = blockDim.x / k.nch;
-  k.gc = (k.Gc + k.nch - 1) / k.nch;
-  const int N = P.N;
-  // both CTAs of a split problem carve shared memory alike (for the larger
-  // of the two parts), so that distributed-shared-memory addresses correspond
-  const int Gcarve = SPLIT ? k.A * max(k.Gu, k.Glp - k.Gu) : k.Gc, G8 = 8 * Gcarve;
+  const int N = P.N, H = N >> 1;
   const int64_t s0 = a.ctr[0], t0 = a.ctr[1];
   const bool icm = MODE == pc::APT_MODE_APT && a.icm;
-  // carve shared memory
-  Shared sh;
-  uint32_t *cur = smem;
-  sh.S = cur;            cur += (size_t)Gcarve * N;
-  sh.thr = cur;          cur += 16 * G8;
-  // each group's 256-byte block of thrh on a 256-byte boundary of the
-  // shared window (the same padding in both CTAs of a cluster)
-  cur += ((256u - ((uint32_t)__cvta_generic_to_shared(cur) & 255u)) & 255u) >> 2;
-  sh.thrh = reinterpret_cast<uint16_t *>(cur);   cur += 16 * G8;   // uses half of its carve
-  sh.temp_of = reinterpret_cast<int32_t *>(cur);  cur += G8;
-  sh.buf_of = reinterpret_cast<int32_t *>(cur);   cur += G8;
-  sh.E = reinterpret_cast<int32_t *>(cur);        cur += G8;
-  sh.Eacc = reinterpret_cast<int32_t *>(cur);     cur += G8;
-  sh.satt = reinterpret_cast<int32_t *>(cur);     cur += 128;
-  sh.sacc = reinterpret_cast<int32_t *>(cur);     cur += 128;
-  sh.m32 = reinterpret_cast<int32_t *>(cur);      cur += 8;
-  cur += ((uintptr_t)cur & 4) ? 1 : 0;            // 8-byte align
-  sh.m64 = reinterpret_cast<int64_t *>(cur);      cur += 8;
-  sh.sum1 = reinterpret_cast<int64_t *>(cur);     cur += 2 * G8;
-  sh.sum2 = reinterpret_cast<int64_t *>(cur);     cur += 2 * G8;
-  sh.hist = reinterpret_cast<int32_t *>(cur);     cur += MODE == pc::APT_MODE_PILOT ? k.T * a.n_bins : 0;
-  sh.ikx = cur;                                   cur += 64;
-  sh.ibit = reinterpret_cast<int32_t *>(cur);     cur += 64;
-  sh.inm = reinterpret_cast<int32_t *>(cur);      cur += 64;
-  sh.isz = reinterpret_cast<int32_t *>(cur);      cur += 64;
-  sh.imask = cur;                                 cur += 24;
-  sh.swm = cur;                                   cur += 24;
-  sh.gmap = reinterpret_cast<int32_t *>(cur);     cur += 8;
-  sh.xch = reinterpret_cast<int32_t *>(cur);      cur += 24;
-  sh.stage = cur;                                 cur += SPLIT ? 512 : 0;
-  sh.swt = cur;                                   cur += (SPLIT && MODE == pc::APT_MODE_APT && a.stage_swt) ? (size_t)max(k.T - 1, 0) * kSwtLen : 0;
-  sh.V = cur;                                     cur += icm ? (size_t)3 * N + 31 + ((N + 31) >> 5) : 0;   // V, X, Xt, R
-  sh.jn = reinterpret_cast<uint16_t *>(cur);
-
-  // load state: local group u is global group gmap[u]
-  if (threadIdx.x < 8)
-    sh.gmap[threadIdx.x] = (threadIdx.x / max(k.Gu, 1)) * k.Glp + k.g0 + threadIdx.x % max(k.Gu, 1);
-  __syncthreads();
-  for (int i = threadIdx.x; i < k.Gc * N; i += blockDim.x)
-    sh.S[i] = a.spins[P.spin_off + (size_t)sh.gmap[i / N] * N + i % N];
-  for (int i = threadIdx.x; i < N; i += blockDim.x) sh.jn[i] = a.jneg[P.jneg_off + i];
-  for (int b = threadIdx.x; b < 8 * k.Gc; b += blockDim.x) {
-    const int gb = 8 * sh.gmap[b >> 3] + (b & 7);
-    const int tb = (b < k.Bc) ? a.temp_of[P.buf_off + gb] : 0;
-    sh.temp_of[b] = tb;
-    sh.buf_of[b] = (b < k.Bc) ? a.buf_of[P.buf_off + gb] : 0;
-    sh.E[b] = (b < k.Bc) ? a.E[P.buf_off + gb] : 0;
-    sh.Eacc[b] = 0;
-    sh.sum1[b] = 0;
-    sh.sum2[b] = 0;
-    for (int e = 0; e < 16; ++e) {
-      const uint32_t th = a.pbit[P.pbit_off + 16 * tb + e];
-      sh.thr[16 * b + e] = th;
-      sh.thrh[16 * b + e] = (uint16_t)(th >> 16);
-    }
-  }
-  for (int i = threadIdx.x; i < 128; i += blockDim.x) {
-    sh.satt[i] = 0;
-    sh.sacc[i] = 0;
-  }
-  if (threadIdx.x < 24) sh.xch[threadIdx.x] = 0;
-  if (PC_APT_STAGE_SWT && SPLIT && MODE == pc::APT_MODE_APT && a.stage_swt)
-    for (int i = threadIdx.x; i < (k.T - 1) * kSwtLen; i += blockDim.x) {
-      const int r = i / kSwtLen, kk = i - r * kSwtLen;
-      const uint32_t off = a.swapidx[P.swapidx_off + 2 * r], len = a.swapidx[P.swapidx_off + 2 * r + 1];
-      sh.swt[i] = ((uint32_t)kk < len) ? a.swaptab[off + kk] : 0u;
-    }
-  if (MODE == pc::APT_MODE_PILOT)
-    for (int i = threadIdx.x; i < k.T * a.n_bins; i += blockDim.x) sh.hist[i] = 0;
+  const int rank = SPLIT ? (int)cooperative_groups::this_cluster().block_rank() : 0;
   if (threadIdx.x == 0) {
-    sh.m64[0] = a.best_E[p];
-    sh.m64[1] = a.best_sweep[p];
-    sh.m64[2] = a.hit_sweep[p];
-    sh.m64[3] = a.target[p];
-    sh.m32[0] = a.best_buf[p];
-    sh.m32[1] = 0;
-    sh.m32[2] = sh.m32[3] = sh.m32[4] = 0;
-    sh.m32[5] = sh.m32[6] = sh.m32[7] = 0;
+    k.Lx = P.Lx;
+    k.Ly = P.Ly;
+    k.Lz = P.Lz;
+    k.N = N;
+    k.H = H;
+    k.hx = P.Lx >> 1;
+    k.mhx = P.mhx;
+    k.mLy = P.mLy;
+    k.mLy2 = P.mLy2;
+    k.nbonds = P.nbonds;
+    k.nreal = P.nreal;
+    k.open = P.open;
+    k.T = P.T;
+    k.Tp = P.Tp;
+    k.A = P.A;
+    k.B = P.B;
+    k.ent = P.ent;
+    k.g0 = a.cta_g0[cta];
+    k.Gc = a.cta_gc[cta];
+    k.Bc = min(8 * k.Gc, P.B - 8 * k.g0);
+    k.split = SPLIT;
+    k.rank = rank;
+    if (MODE == pc::APT_MODE_APT || MODE == pc::APT_MODE_ENERGY) {
+      k.Gu = k.Gc / k.A;   // A is 1, 2 or 4
+      k.Glp = k.Tp >> 3;
+    } else {
+      k.Gu = k.Gc;
+      k.Glp = (k.B + 7) >> 3;
+    }
+    k.nq = quads_of(k.Gc);
+    k.gq = quad_groups(k.Gc);
+    k.lw = quad_shift(k.Gc);
+    k.nch = a.cta_nch[cta];
+    k.tpc = blockDim.x / k.nch;
+    k.k0 = a.k0;
+    k.k1 = a.k1;
+    k.tag_main = a.tag_main;
+    k.tag_ref = a.tag_ref;
+    k.joint = a.joint_swap;
+    k.icm_big = a.icm_big;
+    k.stage_swt = a.stage_swt;
+    k.swapidx = a.swapidx + P.swapidx_off;
+    k.swaptab = a.swaptab;
+    k.best_spins = (rank ? a.best_spins2 : a.best_spins) + P.best_off;
+    // carve shared memory; both CTAs of a split problem alike (for the
+    // larger of the two parts), so that distributed-shared-memory addresses
+    // correspond
+    const int Gm = SPLIT ? k.A * max(k.Gu, k.Glp - k.Gu) : k.Gc, Gp = quads_of(Gm) * quad_groups(Gm);
+    int o = (int)(sizeof(Ctl) / 4);
+    k.oThr = o;    o += 128 * Gp;
+    // each group's block of thh starts on a 256-byte boundary of the shared window
+    o += (int)((256u - (((uint32_t)__cvta_generic_to_shared(smem) + 4u * (uint32_t)o) & 255u)) & 255u) >> 2;
+    k.oThh = o;    o += 64 * Gp;
+    k.oHist = o;   o += MODE == pc::APT_MODE_PILOT ? (P.T * a.n_bins + 3) & ~3 : 0;
+    k.oStage = o;  o += SPLIT ? 512 : 0;
+    k.oSwt = o;    o += (SPLIT && MODE == pc::APT_MODE_APT && a.stage_swt) ? max(P.T - 1, 0) * kSwtLen : 0;
+    k.oS = o;      o += site_words(Gm) * N;
+    k.oV = o;      o += icm ? 3 * N + 31 + ((N + 31) >> 5) : 0;
+    k.oJn = o;
+    k.m64[0] = a.best_E[p];
+    k.m64[1] = a.best_sweep[p];
+    k.m64[2] = a.hit_sweep[p];
+    k.m64[3] = a.target[p];
+    k.m32[0] = a.best_buf[p];
+    for (int i = 1; i < 8; ++i) k.m32[i] = 0;
+    // local group u is global group gmap[u]
+    for (int g = 0; g < 8; ++g) k.gmap[g] = (g / max(k.Gu, 1)) * k.Glp + k.g0 + g % max(k.Gu, 1);
+  }
+  __syncthreads();
+  // load state
+  {
+    uint32_t *S = smem + k.oS, *jn = smem + k.oJn, *thr = smem + k.oThr;
+    uint16_t *thh = reinterpret_cast<uint16_t *>(smem + k.oThh);
+    for (int i = threadIdx.x; i < k.Gc * N; i += blockDim.x) {
+      const int g = i / N, kk = i - g * N;
+      spin_word(k, S, g, kk) = a.spins[P.spin_off + (size_t)k.gmap[g] * N + kk];
+    }
+    for (int i = threadIdx.x; i < N; i += blockDim.x) {
+      const int c = i >= H ? 1 : 0;
+      jn[i] = (uint32_t)a.jneg[P.jneg_off + i] | place_bits(k, c, i - c * H);
+    }
+    for (int b = threadIdx.x; b < 64; b += blockDim.x) {
+      k.Eacc[b] = 0;
+      if (b >= 8 * k.Gc) continue;
+      const int gb = 8 * k.gmap[b >> 3] + (b & 7);
+      const int tb = (b < k.Bc) ? a.temp_of[P.buf_off + gb] : 0;
+      k.temp_of[b] = tb;
+      k.E[b] = (b < k.Bc) ? a.E[P.buf_off + gb] : 0;
+      k.sum1[b] = 0;
+      k.sum2[b] = 0;
+      for (int e = 0; e < 16; ++e) {
+        const uint32_t th = a.pbit[P.pbit_off + 16 * tb + e];
+        thr[16 * b + e] = th;
+        thh[16 * b + e] = (uint16_t)(th >> 16);
+      }
+    }
+    for (int i = threadIdx.x; i < 128; i += blockDim.x) {
+      k.satt[i] = 0;
+      k.sacc[i] = 0;
+    }
+    if (threadIdx.x < 24) k.xch[threadIdx.x] = 0;
+    if (PC_APT_STAGE_SWT && SPLIT && MODE == pc::APT_MODE_APT && a.stage_swt)
+      for (int i = threadIdx.x; i < (k.T - 1) * kSwtLen; i += blockDim.x) {
+        const int r = i / kSwtLen, kk = i - r * kSwtLen;
+        const uint32_t off = k.swapidx[2 * r], len = k.swapidx[2 * r + 1];
+        smem[k.oSwt + i] = ((uint32_t)kk < len) ? a.swaptab[off + kk] : 0u;
+      }
+    if (MODE == pc::APT_MODE_PILOT)
+      for (int i = threadIdx.x; i < k.T * a.n_bins; i += blockDim.x) smem[k.oHist + i] = 0u;
   }
   __syncthreads();
 
   if (MODE == pc::APT_MODE_ENERGY) {
-    colour_phase<false, true>(a, k, sh, 1, 0u, k.Gc);
+    colour_phase<false, true>(1, 0u);
     __syncthreads();
-    finish_energies(k, sh);
+    for (int b = threadIdx.x; b < 8 * k.Gc; b += blockDim.x) k.E[b] = k.nbonds - 2 * k.Eacc[b];
     __syncthreads();
-  } else {
+  } else if (MODE == pc::APT_MODE_APT) {
+#if PC_APT_PROFILE
     long long pt = clock64();
+#endif
+    const int spp = a.spp;
     for (int it = 0; it < a.n_iter; ++it) {
       const uint32_t t = (uint32_t)(t0 + it);
-      for (int qq = 0; qq < a.spp; ++qq) {
-        const uint32_t s = (uint32_t)(s0 + (int64_t)it * a.spp + qq);
-        colour_phase<true, false>(a, k, sh, 0, s, k.Gc);
+      const uint32_t sf = (uint32_t)(s0 + (int64_t)it * spp);
+      for (int qq = 0; qq < spp; ++qq) {
+        colour_phase<true, false>(0, sf + (uint32_t)qq);
         __syncthreads();
         PROF_MARK(0, pt);
-        if (MODE == pc::APT_MODE_APT && qq + 1 < a.spp) {
-          // the APT mode reads energies only after the attempt's last sweep
-          colour_phase<true, false>(a, k, sh, 1, s, k.Gc);
-          __syncthreads();
-          PROF_MARK(1, pt);
-          continue;
-        }
-        colour_phase<true, true>(a, k, sh, 1, s, k.Gc);
-        __syncthreads();
-        finish_energies(k, sh);
+        // energies are read only after the attempt's last sweep
+        if (qq + 1 < spp)
+          colour_phase<true, false>(1, sf + (uint32_t)qq);
+        else
+          colour_phase<true, true>(1, sf + (uint32_t)qq);
         __syncthreads();
         PROF_MARK(1, pt);
-        if (MODE == pc::APT_MODE_LADDER) {
-          if ((int64_t)it * a.spp + qq >= a.window_from)
-            for (int b = threadIdx.x; b < k.Bc; b += blockDim.x) {
-              const int64_t e = sh.E[b];
-              sh.sum1[b] += e;
-              sh.sum2[b] += e * e;
-            }
-        } else if (MODE == pc::APT_MODE_PILOT) {
-          if ((int64_t)s >= a.window_from)
-            for (int b = threadIdx.x; b < k.Bc; b += blockDim.x) {
-              const int64_t span = 3 * (int64_t)N;
-              const int64_t num = ((int64_t)sh.E[b] + span) * a.n_bins;
-              int64_t bin = num < 0 ? 0 : num / span;
-              if (bin > a.n_bins - 1) bin = a.n_bins - 1;
-              atomicAdd(&sh.hist[sh.temp_of[b] * a.n_bins + (int)bin], 1);
-            }
+      }
+      const int64_t sweeps = s0 + (int64_t)(it + 1) * spp;
+      // warp 0 measures while the others go on to the next barrier
+      if (threadIdx.x < 32) measure(0, sweeps);
+      if (icm) {
+        icm_all<CSEED>(t);
+#if PC_APT_PROFILE
+        pt = clock64();
+#endif
+        if (k.A == 2)
+          label0_energies();
+        else
+          colour_phase<false, true>(1, 0u);   // the pairs change with the temperature
+        __syncthreads();
+        PROF_MARK(9, pt);
+        if (threadIdx.x < 32) {
+          // a flag of the first measurement stands until the copy is made there
+          measure(k.A == 2, sweeps);
         }
       }
-      if (MODE != pc::APT_MODE_APT) continue;
-      const int64_t sweeps = s0 + (int64_t)(it + 1) * a.spp;
-      best_update(a, k, sh, p, sweeps);
-      PROF_MARK(2, pt);
-      if (icm) {
-        icm_all<CSEED>(a, k, sh, t);
-        pt = clock64();
-        best_update(a, k, sh, p, sweeps);
-        PROF_MARK(10, pt);
-      }
-      swap_step<SPLIT>(a, k, sh, p, t);
+      swap_step<SPLIT>(t);
       __syncthreads();
       PROF_MARK(3, pt);
+    }
+  } else {
+    // ladder and pilot chains: energies from window_from on only
+    for (int it = 0; it < a.n_iter; ++it) {
+      const uint32_t s = (uint32_t)(s0 + it);
+      colour_phase<true, false>(0, s);
+      __syncthreads();
+      const bool count = MODE == pc::APT_MODE_LADDER ? (int64_t)it >= a.window_from : (int64_t)s >= a.window_from;
+      if (!count) {
+        colour_phase<true, false>(1, s);
+        __syncthreads();
+        continue;
+      }
+      colour_phase<true, true>(1, s);
+      __syncthreads();
+      // the next energy pass is two barriers away
+      for (int b = threadIdx.x; b < 8 * k.Gc; b += blockDim.x) {
+        const int64_t e = k.nbonds - 2 * k.Eacc[b];
+        k.Eacc[b] = 0;
+        k.E[b] = (int32_t)e;
+        if (b >= k.Bc) continue;
+        if (MODE == pc::APT_MODE_LADDER) {
+          k.sum1[b] += e;
+          k.sum2[b] += e * e;
+        } else {
+          const int64_t span = 3 * (int64_t)N;
+          const int64_t num = (e + span) * a.n_bins;
+          int64_t bin = num < 0 ? 0 : num / span;
+          if (bin > a.n_bins - 1) bin = a.n_bins - 1;
+          atomicAdd(reinterpret_cast<int *>(smem + k.oHist) + k.temp_of[b] * a.n_bins + (int)bin, 1);
+        }
+      }
     }
   }
 
@@ -1348,85 +1488,86 @@ __global__ void __launch_bounds__(512) apt_kernel(const AptArgs a) {
   if (MODE == pc::APT_MODE_APT && a.n_iter > 0) {
     const int lpar = (int)((t0 + a.n_iter - 1) & 1);   // parity of the last attempt
     uint32_t bmask = 0;
-    if (k.split) {
+    if (SPLIT) {
       // colour-0 spins of the last boundary swap, and this rank's best
       // candidate, to the peer (the other parity's buffers are free)
-      push_boundary(k, sh, 0, lpar ^ 1);
+      push_boundary(0, lpar ^ 1, 0);
       if (threadIdx.x == 0) {
-        int *px = cooperative_groups::this_cluster().map_shared_rank(sh.xch, k.rank ^ 1);
-        px[12] = (int)sh.m64[0];
-        px[13] = sh.m32[0];
-        px[14] = (int)(uint32_t)((uint64_t)sh.m64[1] & 0xFFFFFFFFu);
-        px[15] = (int)(uint32_t)((uint64_t)sh.m64[1] >> 32);
-        px[16] = (int)(uint32_t)((uint64_t)sh.m64[2] & 0xFFFFFFFFu);
-        px[17] = (int)(uint32_t)((uint64_t)sh.m64[2] >> 32);
+        int *px = cooperative_groups::this_cluster().map_shared_rank(k.xch, k.rank ^ 1);
+        px[12] = (int)k.m64[0];
+        px[13] = k.m32[0];
+        px[14] = (int)(uint32_t)((uint64_t)k.m64[1] & 0xFFFFFFFFu);
+        px[15] = (int)(uint32_t)((uint64_t)k.m64[1] >> 32);
+        px[16] = (int)(uint32_t)((uint64_t)k.m64[2] & 0xFFFFFFFFu);
+        px[17] = (int)(uint32_t)((uint64_t)k.m64[2] >> 32);
       }
       cooperative_groups::this_cluster().sync();   // last access to the peer's memory
       if (threadIdx.x == 0) {
-        const int64_t pE = sh.xch[12];
-        const int64_t psw = (int64_t)(((uint64_t)(uint32_t)sh.xch[15] << 32) | (uint32_t)sh.xch[14]);
-        const int64_t phit = (int64_t)(((uint64_t)(uint32_t)sh.xch[17] << 32) | (uint32_t)sh.xch[16]);
+        const int64_t pE = k.xch[12];
+        const int64_t psw = (int64_t)(((uint64_t)(uint32_t)k.xch[15] << 32) | (uint32_t)k.xch[14]);
+        const int64_t phit = (int64_t)(((uint64_t)(uint32_t)k.xch[17] << 32) | (uint32_t)k.xch[16]);
         // rank 0's candidate against rank 1's: lower energy, earlier sweep,
         // then rank 0 (its slots are the lower ones)
-        const int64_t E0 = k.rank == 0 ? sh.m64[0] : pE, E1 = k.rank == 0 ? pE : sh.m64[0];
-        const int64_t S0 = k.rank == 0 ? sh.m64[1] : psw, S1 = k.rank == 0 ? psw : sh.m64[1];
+        const int64_t E0 = k.rank == 0 ? k.m64[0] : pE, E1 = k.rank == 0 ? pE : k.m64[0];
+        const int64_t S0 = k.rank == 0 ? k.m64[1] : psw, S1 = k.rank == 0 ? psw : k.m64[1];
         const bool win1 = E1 < E0 || (E1 == E0 && S1 < S0);
         int copy = 0;
         if (k.rank == 0 && win1) {
-          sh.m64[0] = pE;
-          sh.m64[1] = psw;
-          sh.m32[0] = sh.xch[13];
+          k.m64[0] = pE;
+          k.m64[1] = psw;
+          k.m32[0] = k.xch[13];
         }
-        if (k.rank == 1) copy = win1 && sh.m64[0] == E1 && sh.m64[1] == S1 && sh.m64[1] >= s0;
-        const int64_t h = sh.m64[2];
-        sh.m64[2] = h < 0 ? phit : (phit < 0 ? h : min(h, phit));
-        sh.m32[1] = copy;
+        if (k.rank == 1) copy = win1 && k.m64[0] == E1 && k.m64[1] == S1 && k.m64[1] >= s0;
+        const int64_t h = k.m64[2];
+        k.m64[2] = h < 0 ? phit : (phit < 0 ? h : min(h, phit));
+        k.m32[1] = copy;
       }
       __syncthreads();
-      bmask = (uint32_t)sh.xch[8];
-      if (sh.m32[1]) {   // rank 1 found the problem's best: it moves its state
-        const AptProbDev &Pb = a.prob[p];
+      bmask = (uint32_t)k.xch[8];
+      if (k.m32[1]) {   // rank 1 found the problem's best: it moves its state
         for (int i = threadIdx.x; i < N; i += blockDim.x)
-          a.best_spins[Pb.best_off + i] = a.best_spins2[Pb.best_off + i];
+          a.best_spins[P.best_off + i] = a.best_spins2[P.best_off + i];
       }
     }
-    if (sh.m32[5] || bmask) {
-      swap_words(k, sh, 0, k.geo.H, bmask, sh.stage + 256 * (lpar ^ 1));
+    if (k.m32[5] || bmask) {
+      swap_words(0, bmask, lpar ^ 1);
       __syncthreads();
     }
   }
   // store state
-  for (int i = threadIdx.x; i < k.Gc * N; i += blockDim.x)
-    a.spins[P.spin_off + (size_t)sh.gmap[i / N] * N + i % N] = sh.S[i];
+  {
+    uint32_t *S = smem + k.oS;
+    for (int i = threadIdx.x; i < k.Gc * N; i += blockDim.x) {
+      const int g = i / N, kk = i - g * N;
+      a.spins[P.spin_off + (size_t)k.gmap[g] * N + kk] = spin_word(k, S, g, kk);
+    }
+  }
   for (int b = threadIdx.x; b < k.Bc; b += blockDim.x) {
-    const int gb = 8 * sh.gmap[b >> 3] + (b & 7);
-    a.temp_of[P.buf_off + gb] = sh.temp_of[b];
-    a.buf_of[P.buf_off + gb] = sh.buf_of[b];
-    a.E[P.buf_off + gb] = sh.E[b];
+    const int gb = 8 * k.gmap[b >> 3] + (b & 7);
+    a.E[P.buf_off + gb] = k.E[b];
     if (MODE == pc::APT_MODE_LADDER) {
-      a.sum1[P.buf_off + gb] = sh.sum1[b];
-      a.sum2[P.buf_off + gb] = sh.sum2[b];
+      a.sum1[P.buf_off + gb] = k.sum1[b];
+      a.sum2[P.buf_off + gb] = k.sum2[b];
     }
   }
   if (MODE == pc::APT_MODE_PILOT)
     for (int i = threadIdx.x; i < k.T * a.n_bins; i += blockDim.x)
-      atomicAdd(reinterpret_cast<unsigned long long *>(&a.hist[P.hist_off + i]),
-                (unsigned long long)sh.hist[i]);
+      atomicAdd(reinterpret_cast<unsigned long long *>(&a.hist[P.hist_off + i]), (unsigned long long)smem[k.oHist + i]);
   if (MODE == pc::APT_MODE_APT) {
     // statistics: both CTAs of a split problem add theirs
     unsigned long long *st = reinterpret_cast<unsigned long long *>(a.stats + P.stat_off);
     const int npair = (k.T - 1) * k.A;
     for (int i = threadIdx.x; i < npair; i += blockDim.x) {
-      if (sh.satt[i]) atomicAdd(st + i, (unsigned long long)sh.satt[i]);
-      if (sh.sacc[i]) atomicAdd(st + npair + i, (unsigned long long)sh.sacc[i]);
+      if (k.satt[i]) atomicAdd(st + i, (unsigned long long)k.satt[i]);
+      if (k.sacc[i]) atomicAdd(st + npair + i, (unsigned long long)k.sacc[i]);
     }
-    if (threadIdx.x < 3 && sh.m32[2 + threadIdx.x])
-      atomicAdd(st + 2 * npair + threadIdx.x, (unsigned long long)sh.m32[2 + threadIdx.x]);
+    if (threadIdx.x < 3 && k.m32[2 + threadIdx.x])
+      atomicAdd(st + 2 * npair + threadIdx.x, (unsigned long long)k.m32[2 + threadIdx.x]);
     if (threadIdx.x == 0 && k.rank == 0) {
-      a.best_E[p] = sh.m64[0];
-      a.best_sweep[p] = sh.m64[1];
-      a.hit_sweep[p] = sh.m64[2];
-      a.best_buf[p] = sh.m32[0];
+      a.best_E[p] = k.m64[0];
+      a.best_sweep[p] = k.m64[1];
+      a.hit_sweep[p] = k.m64[2];
+      a.best_buf[p] = k.m32[0];
     }
   }
 }
@@ -1459,14 +1600,14 @@ __global__ void apt_init_kernel(const AptArgs a, int n_prob) {
 namespace pc {
 
 size_t apt_smem_bytes(int N, int Gc, int nwarps, int mode, int icm, int T, int n_bins, int stage_swt) {
-  const size_t G8 = 8 * (size_t)Gc;
-  size_t words = (size_t)Gc * N + 32 * G8 + 4 * G8 + 128 + 8 + 1 + 16 + 8 * G8;
-  words += 4 * 64 + 24 + 24 + 128 + 8 + 24 + 512;   // + larger swap stats, group map, exchange, stage
-  if (mode == APT_MODE_PILOT) words += (size_t)T * n_bins;
+  const int Gp = quads_of(Gc) * quad_groups(Gc);
+  size_t words = sizeof(Ctl) / 4 + 192 * (size_t)Gp + 64 + 512;   // thr, thh and its alignment, stage
+  if (mode == APT_MODE_PILOT) words += ((size_t)T * n_bins + 3) & ~(size_t)3;
   if (mode == APT_MODE_APT && stage_swt) words += (size_t)(T > 1 ? T - 1 : 0) * kSwtLen;   // staged swap tables
+  words += (size_t)site_words(Gc) * N;
   // V, X, the transposed X (or the cluster labels) and the root masks
   if (mode == APT_MODE_APT && icm) words += (size_t)3 * N + 31 + (size_t)((N + 31) >> 5);
-  return words * 4 + (size_t)N * 2 + 16 + 256;   // + the threshold table's alignment
+  return (words + (size_t)N) * 4;
 }
 
 template <int MODE, bool CSEED>

@@ -55,19 +55,18 @@ struct Batch {
   std::vector<uint32_t> h_pbit, h_swaptab, h_swapidx;
 };
 
-// Split of a CTA's threads into nch chunks of tpb/nch threads, each chunk
-// sweeping ceil(Gc/nch) groups of every site: `pref` where it fits (tpb a
-// multiple of 32 nch, nch <= Gc, at most 4 groups per thread), else the
-// choice that minimises the longest thread's work (site rounds x groups).
+// Split of a CTA's threads into nch chunks of tpb/nch threads, chunk q
+// sweeping the quads (up to four replica groups) q, q + nch, .. of every
+// site: `pref` where it fits (tpb a multiple of 32 nch, nch <= quads), else
+// the choice that minimises the longest thread's work (site rounds x quads).
 int choose_nch(int H, int Gc, int tpb, int pref) {
-  if (pref > 0 && tpb % (32 * pref) == 0 && pref <= Gc && (Gc + pref - 1) / pref <= 4) return pref;
+  const int nq = (Gc + 3) / 4;
+  if (pref > 0 && tpb % (32 * pref) == 0 && pref <= nq) return pref;
   int best = 1, best_cost = INT_MAX;
-  for (int nch = 1; nch <= 8; nch *= 2) {
+  for (int nch = 1; nch <= nq; nch *= 2) {
     if (tpb % (32 * nch)) continue;
-    const int gc = (Gc + nch - 1) / nch;
-    if (gc > 4) continue;
     const int tpc = tpb / nch;
-    const int cost = ((H + tpc - 1) / tpc) * gc;
+    const int cost = ((H + tpc - 1) / tpc) * ((nq + nch - 1) / nch);
     if (cost < best_cost) {
       best_cost = cost;
       best = nch;
