@@ -278,15 +278,19 @@ int pc_sqa_setup_bc(pc_ctx *c, const int32_t *dims, const uint8_t *periodic, con
   q.jq.resize((size_t)n_sweeps);
   q.table.assign((size_t)(n_sweeps > 0 ? n_sweeps : 1) * kSqaTab, 0u);
   const double beta_eff = 1.0 / ((double)P * T);
+  int nreal = 0;
+  std::vector<uint16_t> jn = pack_jn16(lat, per, present, J, &q.nbonds, &nreal);
+  // in-slice fields I = -6..6; with every bond present only the even ones
+  // occur, and a row needs 21 exponentials instead of 39
+  const int de = q.nbonds == 3 * lat.N ? 2 : 1;
   // every sweep's row is independent: long schedules are built by several
   // host threads (the rows do not depend on how they are split)
   auto rows = [&](int s0, int s1) {
     for (int s = s0; s < s1; ++s) {
       const int32_t jq = pc_jperp_q(gamma[s], P, T);
       q.jq[(size_t)s] = jq;
-      // every in-slice field I = -6..6 (odd at open faces) and time count m
       for (int m = 0; m < 3; ++m)
-        for (int e = 0; e < 13; ++e)
+        for (int e = 0; e < 13; e += de)
           q.table[(size_t)s * kSqaTab + e + 13 * m] = sqa_threshold(beta_eff, e - 6, jq, 2 * m - 2);
     }
   };
@@ -312,8 +316,6 @@ int pc_sqa_setup_bc(pc_ctx *c, const int32_t *dims, const uint8_t *periodic, con
     for (int i = made; i < nth; ++i) rows(lo(i), lo(i + 1));
     for (auto &t : pool) t.join();
   }
-  int nreal = 0;
-  std::vector<uint16_t> jn = pack_jn16(lat, per, present, J, &q.nbonds, &nreal);
   if (q.d_jneg.n < jn.size() && (rc = q.d_jneg.alloc(jn.size()))) return rc;
   if (q.d_table.n < q.table.size() && (rc = q.d_table.alloc(q.table.size()))) return rc;
   // stage through pinned memory: one copy of each array
@@ -374,10 +376,21 @@ static int sqa_enqueue(pc_ctx *c, int R, uint32_t run0, int32_t *E_dev, int32_t 
   a.n_items = R;
   a.first_item = 0;
   a.wait_ns = wait_ns;
-  if (a.S > 0) {
-    // persistent time-sliced schedule: about 32 (run, chunk) items per SM
+  c->sqa.last_err = nullptr;
+  // Persistent time-sliced schedule: about 32 (run, chunk) items per SM, so
+  // that a number of runs that is no multiple of the SMs keeps all of them
+  // busy.  With at most one run per SM there is nothing to level and a run is
+  // one item; slicing it only adds hand-offs through global memory (8 runs of
+  // 1024 spins, 100 sweeps: 100 slices of one sweep, 0.45 ms; whole runs
+  // 0.19 ms).  Else an item holds at least 2^19 spin updates (about 50 us of an
+  // SM), far above a hand-off's few microseconds.  Runs of one item that are
+  // short skip the queue as well.
+  const int64_t upd = (int64_t)a.N * a.P * a.S;
+  const bool level = R > c->sms || first_chunk > 0;
+  if (a.S > 0 && (level || upd > (1 << 22))) {
     SqaState &q = c->sqa;
-    int nch = (32 * c->sms + R - 1) / R;
+    int nch = level ? (32 * c->sms + R - 1) / R : 1;
+    if (first_chunk == 0) nch = (int)std::min<int64_t>(nch, upd >> 19);
     if (nch > a.S) nch = a.S;
     if (nch < 1) nch = 1;
     a.K = (a.S + nch - 1) / nch;

@@ -209,3 +209,25 @@ def test_bounded_wait_reports_timeout_and_context_survives(pc, orc):
     E = pc.pc_sqa_run(ctx.h, 3, 0, P, 64)
     assert np.array_equal(E, orc.sqa_anneal(dims, J, P, 0.05, gamma, 3, seed=5))
     ctx.close()
+
+
+@pytest.mark.parametrize("P,R,S,spins", [
+    (16, 152, 40, True),     # one run per SM: whole anneals, one CTA each
+    (16, 153, 1025, False),  # one more: items of 2^19 updates, two slices
+    (32, 160, 40, True),     # time-sliced schedule with one slice
+])
+def test_sqa_schedule_follows_the_number_of_runs(pc, orc, P, R, S, spins):
+    """Anneals with at most one run per SM take one CTA per run, more runs the
+    time-sliced queue; both equal the oracle bit for bit."""
+    dims, seed = (4, 4, 4), 23
+    J = W.ea_couplings(dims, W.SEED_INSTANCES, seed)
+    gamma = W.linear_gamma_schedule(S)
+    ctx = pc.Context(0, seed)
+    pc.pc_sqa_setup(ctx.h, dims, J, P, 0.05, gamma)
+    got = pc.pc_sqa_run(ctx.h, R, 5, P, 64, want_spins=spins)
+    ctx.close()
+    want = orc.sqa_anneal(dims, J, P, 0.05, gamma, R, run0=5, seed=seed, want_spins=spins)
+    if spins:
+        assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
+    else:
+        assert np.array_equal(got, want)
