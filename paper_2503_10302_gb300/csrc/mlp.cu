@@ -5,9 +5,9 @@
 // Algorithm S2 by a network reading cheap instance features and short pilot
 // histograms, on the grounds that ladders of one size are nearly identical
 // across instances (Fig. S12).  These are tiny dense layers, so they run as
-// plain SIMT kernels: a 64x64-tiled GEMM with bias / ReLU / ReLU-mask
-// epilogues, a warp-per-sample head (scan and reverse scan over the 32
-// outputs), column sums for bias gradients, and an elementwise Adam step.
+// plain SIMT kernels: a 32x32-tiled product with bias / ReLU / ReLU-mask
+// epilogues and row sums for bias gradients, a warp-per-sample head (scan and
+// reverse scan over the 32 outputs), and an elementwise Adam step.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -24,60 +24,133 @@ namespace {
 constexpr int kIn = 259, kHid = 256, kOut = 32, kLayers = 4;
 constexpr int kDims[kLayers + 1] = {kIn, kHid, kHid, kHid, kOut};
 
-// C[m][n] (ldc) = epi( sum_k A(m,k) B(k,n) ) with A(m,k) = A[m*sam + k*sak],
-// B(k,n) = B[k*sbk + n*sbn].  Epilogues: + bias[n]; ReLU; multiply by
-// (mask[m*ldmask + n] > 0).
-template <bool BIAS, bool RELU, bool MASK>
-__global__ void __launch_bounds__(256) gemm_kernel(int M, int N, int K, const float *__restrict__ A,
-                                                   int sam, int sak, const float *__restrict__ B,
-                                                   int sbk, int sbn, float *__restrict__ C, int ldc,
-                                                   const float *__restrict__ bias,
-                                                   const float *__restrict__ mask, int ldmask) {
-  __shared__ float As[16][64 + 1];
-  __shared__ float Bs[16][64 + 1];
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
-  float acc[4][4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-#pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
-  for (int k0 = 0; k0 < K; k0 += 16) {
-    for (int e = threadIdx.x; e < 16 * 64; e += 256) {
-      const int kk = e >> 6, mm = e & 63;
-      const int m = m0 + mm, k = k0 + kk;
-      As[kk][mm] = (m < M && k < K) ? A[(size_t)m * sam + (size_t)k * sak] : 0.f;
-      const int n = n0 + mm;
-      Bs[kk][mm] = (n < N && k < K) ? B[(size_t)k * sbk + (size_t)n * sbn] : 0.f;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < 16; ++kk) {
-      float a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[kk][ty + 16 * i];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) b[j] = Bs[kk][tx + 16 * j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
+// One product C[m][n] = epi( sum_k A(m,k) B(k,n) ) with A(m,k) = A[m*sam +
+// k*sak], B(k,n) = B[k*sbk + n*sbn].  Epilogue: + bias[n]; ReLU; times
+// (mask[m*ldc + n] > 0).  `rowsum`, if given, receives sum_k A(m,k) (the
+// bias gradient) as one more column, B(k, N) = 1.
+struct Product {
+  int M, N, K;
+  const float *A, *B;
+  int sam, sak, sbk, sbn;
+  float *C;
+  int ldc, relu;
+  const float *bias, *mask;
+  float *rowsum;
+  int tn, tiles;    // tiles along n, and in all (0: no product)
+};
+
+// A layer's independent products (dW and dZ of the layer below) and, in one
+// more block, the loss sum go out in one launch.
+struct Products {
+  Product p[2];
+  int loss_n;              // samples of the loss sum (0: none)
+  const float *loss_s;
+  float *loss, *loss2;     // loss2: a second destination or NULL
+};
+
+// A 32 x 32 tile per block of 128 threads, 2 x 4 outputs per thread, K in
+// steps of 32 whose global loads are issued one step ahead.  What bounds
+// these layers (256 x 256 x 259 and below) is not arithmetic but how many
+// SMs take part and the latency of each K step: a 64 x 64 tile put 256 x 256
+// on 16 SMs and waited for every load (48 us per product).  With 64 blocks,
+// the loads ahead and 11 instead of 19 launches a training step of 256
+// samples went from 0.40 to 0.11 ms.  Every output is one fmaf chain over k
+// in order.
+constexpr int kTile = 32, kGemmThreads = 128;
+
+__device__ __forceinline__ void loss_sum(int B, const float *loss_s, float *loss, float *loss2, float *part) {
+  // 256 partial sums in fixed order, two per thread
+  for (int t = threadIdx.x; t < 256; t += kGemmThreads) {
+    float s = 0.f;
+    for (int i = t; i < B; i += 256) s += loss_s[i];
+    part[t] = s;
+  }
+  __syncthreads();
+  for (int w = 128; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
     __syncthreads();
   }
+  if (threadIdx.x == 0) {
+    const float l = part[0] / (float)(B * kOut);
+    *loss = l;
+    if (loss2) *loss2 = l;
+  }
+}
+
+__global__ void __launch_bounds__(kGemmThreads) gemm_kernel(const __grid_constant__ Products P) {
+  __shared__ __align__(16) float As[kTile][kTile + 2];   // rows 8-byte aligned (float2 reads)
+  __shared__ __align__(16) float Bs[kTile][kTile + 4];   // rows 16-byte aligned (float4 reads)
+  int tile = (int)blockIdx.x;
+  if (P.loss_n) {
+    if (tile == 0) {
+      loss_sum(P.loss_n, P.loss_s, P.loss, P.loss2, &As[0][0]);
+      return;
+    }
+    --tile;
+  }
+  const bool second = tile >= P.p[0].tiles;
+  const Product &g = P.p[second ? 1 : 0];
+  if (second) tile -= P.p[0].tiles;
+  const int M = g.M, N = g.N, K = g.K;
+  const int m0 = (tile / g.tn) * kTile, n0 = (tile % g.tn) * kTile;
+  const int tid = threadIdx.x, r = tid & 31, w = tid >> 5;
+  // element e = w + 4 q of a tile: lanes run along the contiguous index
+  const bool ak = g.sak == 1, bk = g.sbk == 1;
+  float ra[8], rb[8];
+  auto load = [&](int k0) {
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int m = m0 + ty + 16 * i;
+    for (int q = 0; q < 8; ++q) {
+      const int e = w + 4 * q;
+      const int ma = m0 + (ak ? e : r), ka = k0 + (ak ? r : e);
+      ra[q] = (ma < M && ka < K) ? g.A[(size_t)ma * g.sam + (size_t)ka * g.sak] : 0.f;
+      const int nb = n0 + (bk ? e : r), kb = k0 + (bk ? r : e);
+      rb[q] = (nb < N && kb < K) ? g.B[(size_t)kb * g.sbk + (size_t)nb * g.sbn] : (nb == N && kb < K ? 1.f : 0.f);
+    }
+  };
+  const int tx = tid & 7, ty = tid >> 3;   // outputs m0 + 2 ty + i, n0 + 4 tx + j
+  float acc[2][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.f;
+  load(0);
+  for (int k0 = 0; k0 < K; k0 += kTile) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const int e = w + 4 * q;
+      if (ak) As[r][e] = ra[q]; else As[e][r] = ra[q];
+      if (bk) Bs[r][e] = rb[q]; else Bs[e][r] = rb[q];
+    }
+    __syncthreads();
+    if (k0 + kTile < K) load(k0 + kTile);
+#pragma unroll
+    for (int kk = 0; kk < kTile; ++kk) {
+      const float2 a = *reinterpret_cast<const float2 *>(&As[kk][2 * ty]);
+      const float4 b = *reinterpret_cast<const float4 *>(&Bs[kk][4 * tx]);
+      const float av[2] = {a.x, a.y}, bv[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(av[i], bv[j], acc[i][j]);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int m = m0 + 2 * ty + i;
     if (m >= M) continue;
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      const int n = n0 + tx + 16 * j;
-      if (n >= N) continue;
+      const int n = n0 + 4 * tx + j;
       float v = acc[i][j];
-      if (BIAS) v += bias[n];
-      if (RELU) v = fmaxf(v, 0.f);
-      if (MASK) v = (mask[(size_t)m * ldmask + n] > 0.f) ? v : 0.f;
-      C[(size_t)m * ldc + n] = v;
+      if (n < N) {
+        if (g.bias) v += g.bias[n];
+        if (g.relu) v = fmaxf(v, 0.f);
+        if (g.mask) v = (g.mask[(size_t)m * g.ldc + n] > 0.f) ? v : 0.f;
+        g.C[(size_t)m * g.ldc + n] = v;
+      } else if (n == N && g.rowsum) {
+        g.rowsum[m] = v;
+      }
     }
   }
 }
@@ -134,29 +207,6 @@ __global__ void head_kernel(int B, const float *O, const float *Y, float beta_mi
   dO[(size_t)warp * kOut + lane] = dov;
 }
 
-// out[n] = sum_m X[m][n] (bias gradients), one thread per column.
-__global__ void colsum_kernel(int M, int N, const float *X, float *out) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  if (n >= N) return;
-  float s = 0.f;
-  for (int m = 0; m < M; ++m) s += X[(size_t)m * N + n];
-  out[n] = s;
-}
-
-// loss = sum_s loss_s / (B * 32), one block, fixed reduction order.
-__global__ void loss_kernel(int B, const float *loss_s, float *loss) {
-  __shared__ float part[256];
-  float s = 0.f;
-  for (int i = threadIdx.x; i < B; i += 256) s += loss_s[i];
-  part[threadIdx.x] = s;
-  __syncthreads();
-  for (int w = 128; w > 0; w >>= 1) {
-    if (threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) *loss = part[0] / (float)(B * kOut);
-}
-
 // Adam (Kingma & Ba): m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
 // p -= lr * (m / c1) / (sqrt(v / c2) + eps) with c1 = 1 - b1^t, c2 = 1 - b2^t.
 __global__ void adam_kernel(int n, float *p, const float *g, float *m, float *v, float lr, float b1,
@@ -201,12 +251,15 @@ using namespace pc;
 
 namespace {
 
-template <bool BIAS, bool RELU, bool MASK>
-int gemm(cudaStream_t st, int M, int N, int K, const float *A, int sam, int sak, const float *B, int sbk,
-         int sbn, float *C, int ldc, const float *bias, const float *mask, int ldmask) {
-  dim3 grid((unsigned)((N + 63) / 64), (unsigned)((M + 63) / 64));
-  gemm_kernel<BIAS, RELU, MASK><<<grid, 256, 0, st>>>(M, N, K, A, sam, sak, B, sbk, sbn, C, ldc, bias, mask,
-                                                       ldmask);
+Product product(int M, int N, int K, const float *A, int sam, int sak, const float *B, int sbk, int sbn, float *C,
+                int ldc, const float *bias, int relu, const float *mask, float *rowsum) {
+  const int tn = (N + (rowsum ? 1 : 0) + kTile - 1) / kTile;
+  return {M, N, K, A, B, sam, sak, sbk, sbn, C, ldc, relu, bias, mask, rowsum, tn, tn * ((M + kTile - 1) / kTile)};
+}
+
+int gemm(cudaStream_t st, const Products &P) {
+  const int blocks = P.p[0].tiles + P.p[1].tiles + (P.loss_n ? 1 : 0);
+  gemm_kernel<<<blocks, kGemmThreads, 0, st>>>(P);
   PC_CUDA_TRY(cudaGetLastError());
   return PC_OK;
 }
@@ -232,15 +285,14 @@ int forward(pc_mlp *mm, int batch, const float *X, float *beta_dev) {
   const float *p = mm->params.p;
   const float *in = X;
   int rc;
-  for (int l = 0; l < 3; ++l) {
-    if ((rc = gemm<true, true, false>(st, batch, kDims[l + 1], kDims[l], in, kDims[l], 1, p + mm->w_off[l], 1,
-                                      kDims[l], mm->H[l].p, kDims[l + 1], p + mm->b_off[l], nullptr, 0)))
-      return rc;
-    in = mm->H[l].p;
+  for (int l = 0; l < kLayers; ++l) {
+    Products P = {};
+    float *out = l < 3 ? mm->H[l].p : mm->O.p;
+    P.p[0] = product(batch, kDims[l + 1], kDims[l], in, kDims[l], 1, p + mm->w_off[l], 1, kDims[l], out, kDims[l + 1],
+                     p + mm->b_off[l], l < 3, nullptr, nullptr);
+    if ((rc = gemm(st, P))) return rc;
+    in = out;
   }
-  if ((rc = gemm<true, false, false>(st, batch, kOut, kHid, in, kHid, 1, p + mm->w_off[3], 1, kHid, mm->O.p,
-                                     kOut, p + mm->b_off[3], nullptr, 0)))
-    return rc;
   if (beta_dev) {
     head_kernel<<<(batch * 32 + 255) / 256, 256, 0, st>>>(batch, mm->O.p, nullptr, mm->beta_min, 0.f, beta_dev,
                                                           nullptr, nullptr);
@@ -249,15 +301,14 @@ int forward(pc_mlp *mm, int batch, const float *X, float *beta_dev) {
   return PC_OK;
 }
 
-// Loss and gradients into mm->grads for X, Y on the device.
-int backward(pc_mlp *mm, int batch, const float *X, const float *Y) {
+// Loss (also to loss2_dev, if given) and gradients into mm->grads for X, Y
+// on the device.
+int backward(pc_mlp *mm, int batch, const float *X, const float *Y, float *loss2_dev = nullptr) {
   cudaStream_t st = mm->ctx->stream;
   int rc = forward(mm, batch, X, nullptr);
   if (rc) return rc;
   head_kernel<<<(batch * 32 + 255) / 256, 256, 0, st>>>(batch, mm->O.p, Y, mm->beta_min, mm->gap_weight,
                                                         mm->beta.p, mm->dO.p, mm->loss_s.p);
-  PC_CUDA_TRY(cudaGetLastError());
-  loss_kernel<<<1, 256, 0, st>>>(batch, mm->loss_s.p, mm->loss.p);
   PC_CUDA_TRY(cudaGetLastError());
   const float *p = mm->params.p;
   float *g = mm->grads.p;
@@ -265,19 +316,22 @@ int backward(pc_mlp *mm, int batch, const float *X, const float *Y) {
   for (int l = kLayers - 1; l >= 0; --l) {
     const int out = kDims[l + 1], in = kDims[l];
     const float *Hin = (l == 0) ? X : mm->H[l - 1].p;
-    // dW[out][in] = sum_b dZ[b][out] Hin[b][in]
-    if ((rc = gemm<false, false, false>(st, out, in, batch, dZ, 1, out, Hin, in, 1, g + mm->w_off[l], in,
-                                        nullptr, nullptr, 0)))
-      return rc;
-    colsum_kernel<<<(out + 127) / 128, 128, 0, st>>>(batch, out, dZ, g + mm->b_off[l]);
-    PC_CUDA_TRY(cudaGetLastError());
-    if (l > 0) {
-      // dZ_{l-1}[b][in] = (sum_o dZ[b][o] W[o][in]) * (H_{l-1} > 0)
-      if ((rc = gemm<false, false, true>(st, batch, in, out, dZ, out, 1, p + mm->w_off[l], in, 1,
-                                         mm->dH[l - 1].p, in, nullptr, mm->H[l - 1].p, in)))
-        return rc;
-      dZ = mm->dH[l - 1].p;
+    Products P = {};
+    // dW[out][in] = sum_b dZ[b][out] Hin[b][in], db[out] = sum_b dZ[b][out]
+    P.p[0] = product(out, in, batch, dZ, 1, out, Hin, in, 1, g + mm->w_off[l], in, nullptr, 0, nullptr,
+                     g + mm->b_off[l]);
+    // dZ_{l-1}[b][in] = (sum_o dZ[b][o] W[o][in]) * (H_{l-1} > 0)
+    if (l > 0)
+      P.p[1] = product(batch, in, out, dZ, out, 1, p + mm->w_off[l], in, 1, mm->dH[l - 1].p, in, nullptr, 0,
+                       mm->H[l - 1].p, nullptr);
+    if (l == kLayers - 1) {
+      P.loss_n = batch;
+      P.loss_s = mm->loss_s.p;
+      P.loss = mm->loss.p;
+      P.loss2 = loss2_dev;
     }
+    if ((rc = gemm(st, P))) return rc;
+    if (l > 0) dZ = mm->dH[l - 1].p;
   }
   return PC_OK;
 }
@@ -425,9 +479,7 @@ int pc_mlp_train_step_dev(pc_mlp *mm, int batch, const float *X_dev, const float
   PC_CUDA_TRY(cudaSetDevice(mm->ctx->device));
   int rc = ensure_batch(mm, batch);
   if (rc) return rc;
-  if ((rc = backward(mm, batch, X_dev, Y_dev))) return rc;
-  if (loss_dev)
-    PC_CUDA_TRY(cudaMemcpyAsync(loss_dev, mm->loss.p, 4, cudaMemcpyDeviceToDevice, mm->ctx->stream));
+  if ((rc = backward(mm, batch, X_dev, Y_dev, loss_dev))) return rc;
   return adam(mm, lr);
 } catch (...) {
   return pc::fail_exception();
