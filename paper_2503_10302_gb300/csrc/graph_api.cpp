@@ -303,6 +303,8 @@ int gload(pc_ctx *c, GImpl *im, int n_prob, const int32_t *n_vert, const int32_t
     P.A = n_labels;
     P.Imax = g.Imax;
     P.m = (int)g.adj.size();
+    P.deg8 = 1;
+    for (const int2 &v : g.vinfo) P.deg8 = P.deg8 && (v.y & 1023) <= 8;
     P.ent = entry0 + (uint32_t)i;
     P.vbase = (uint32_t)vinfo.size();
     P.abase = (uint32_t)adj.size();

@@ -34,6 +34,7 @@ constexpr int kGWarps = kGThreads / 32;
 
 struct GProbDev {
   int n, C, T, A, Imax, m;
+  int deg8;                     // every vertex has at most 8 neighbours
   uint32_t ent;                 // problem entry of the counters
   uint32_t vbase;               // first vertex in vinfo / spins ([n][A] words from vbase * A)
   uint32_t abase;               // first adjacency entry

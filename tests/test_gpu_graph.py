@@ -269,3 +269,31 @@ def test_gapt_fuzz_shapes(pc, orc):
         _compare(pc, ctx, o, [g], betas, A)
         ctx.close()
         assert deg.max(initial=0) <= 200
+
+
+@pytest.mark.parametrize("dims,deg", [((8, 8, 8), 6), ((8, 16, 8), 6), ((5, 5, 41), 6), ((16, 16, 12), 6),
+                                      ((7, 439, 1), 6), ((10, 10, 10), 9)])
+def test_gapt_cluster_fill_sizes(pc, orc, dims, deg):
+    """ICM's flood fill keeps up to 2 or 6 vertices per thread with at most 8
+    neighbours in registers (512, 1024 | 1025, 3072 | 3073 vertices, and a
+    vertex with 9 neighbours): all equal the oracle bit for bit."""
+    n = int(np.prod(dims))
+    J = W.ea_couplings(dims, 1000, n)
+    if deg == 6:
+        g = W.lattice_graph(dims, (1, 1, 0 if dims[2] == 1 else 1), J)[0]
+    else:
+        e = W.lattice_graph(dims, (1, 1, 1), J)[0].edges()
+        have = {(u, v) for u, v, _ in e}
+        e += [(0, v, 1) for v in (555, 777, 999) if (0, v) not in have]   # vertex 0: 9 neighbours
+        g = W.csr_from_edges(n, [(u, v) for u, v, _ in e], [w for _, _, w in e])
+        assert int(np.diff(g.rp).max()) == 9
+    betas = [W.geometric_ladder(6, 0.3, 1.5)]
+    ctx = pc.Context(0, 5)
+    pc.pc_gapt_load(ctx.h, [(g.rp, g.col, g.w)], betas, 2, 0)
+    pc.pc_gapt_run(ctx.h, 4, 1, True)
+    got = pc.pc_gapt_get_spins(ctx.h, 0, 6, 2, g.n), pc.pc_gapt_get_energies(ctx.h, 0, 6, 2)
+    ctx.close()
+    ref = orc.GApt([(g.rp, g.col, g.w)], betas, n_labels=2, seed=5)
+    ref.run(4)
+    s, e, _ = ref.state(0)
+    assert np.array_equal(got[0], s) and np.array_equal(got[1], e)
