@@ -34,15 +34,9 @@
 #ifndef PC_APT_PROFILE
 #define PC_APT_PROFILE 0
 #endif
-// The flood fill keeps a block's overlap words in registers across passes
-// (build-time knob; 0 reloads them every pass).
-#ifndef PC_APT_FILL_XREG
-#define PC_APT_FILL_XREG 1
-#endif
-// Split problems keep the first entries of their swap tables in shared
-// memory (build-time knob).
-#ifndef PC_APT_STAGE_SWT
-#define PC_APT_STAGE_SWT 1
+// Rounds of spreading inside a block per flood-fill pass (build-time knob).
+#ifndef PC_APT_FILL_ROUNDS
+#define PC_APT_FILL_ROUNDS 1
 #endif
 #if PC_APT_PROFILE
 __device__ unsigned long long g_apt_prof[32];
@@ -62,6 +56,57 @@ namespace {
 using namespace pcdev;
 using pc::AptArgs;
 using pc::AptProbDev;
+
+// The first two rounds of philox(c0, c1, c2, c3) taken apart, for draws that
+// pair many (c0, c3) with many (c1, c2).  Round 1 turns c0 and c2 into
+// products that do not meet before round 2, whose product of the c2 lane
+// depends on (c0, c3) alone and whose product of the c0 lane depends on
+// (c1, c2) alone: a site's part is shared by its replica groups, a group's
+// part by the sites, and a draw starts at round 3 after two XORs (saves 4 of
+// 20 wide products, the half-rate instructions, and 2 of 20 XORs).
+struct PhiloxA { uint32_t lo0, b_lo, b_hi; };   // of (c0, c3)
+struct PhiloxB { uint32_t x0, x2, lo; };        // of (c1, c2), round-2 keys folded in
+
+__device__ __forceinline__ PhiloxA philox_a(uint32_t c0, uint32_t c3, uint32_t k1) {
+  PhiloxA p;
+  p.lo0 = 0xD2511F53u * c0;
+  const uint32_t n2 = __umulhi(0xD2511F53u, c0) ^ c3 ^ k1;
+  p.b_lo = 0xCD9E8D57u * n2;
+  p.b_hi = __umulhi(0xCD9E8D57u, n2);
+  return p;
+}
+__device__ __forceinline__ PhiloxB philox_b(uint32_t c1, uint32_t c2, uint32_t k0, uint32_t k1) {
+  PhiloxB p;
+  const uint32_t n0 = __umulhi(0xCD9E8D57u, c2) ^ c1 ^ k0;
+  p.x0 = (0xCD9E8D57u * c2) ^ (k0 + 0x9E3779B9u);
+  p.x2 = __umulhi(0xD2511F53u, n0) ^ (k1 + 0xBB67AE85u);
+  p.lo = 0xD2511F53u * n0;
+  return p;
+}
+__device__ __forceinline__ uint4 philox_ab(const PhiloxA &a, const PhiloxB &b, uint32_t k0, uint32_t k1) {
+  uint32_t c0 = a.b_hi ^ b.x0, c1 = a.b_lo, c2 = b.x2 ^ a.lo0, c3 = b.lo;
+  k0 += 2u * 0x9E3779B9u;
+  k1 += 2u * 0xBB67AE85u;
+#pragma unroll
+  for (int r = 2; r < 10; ++r) {
+    const uint32_t lo0 = 0xD2511F53u * c0, hi0 = __umulhi(0xD2511F53u, c0);
+    const uint32_t lo1 = 0xCD9E8D57u * c2, hi1 = __umulhi(0xCD9E8D57u, c2);
+    c0 = hi1 ^ c1 ^ k0;
+    c2 = hi0 ^ c3 ^ k1;
+    c1 = lo1;
+    c3 = lo0;
+    k0 += 0x9E3779B9u;
+    k1 += 0xBB67AE85u;
+  }
+  return make_uint4(c0, c1, c2, c3);
+}
+
+// The 16-bit word at a shared-window address.
+__device__ __forceinline__ uint32_t lds_u16(uint32_t addr) {
+  uint32_t v;
+  asm("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
 
 // Everything a phase of the kernel needs to know about its CTA, at the start
 // of dynamic shared memory.  The phases are functions of their own that read
@@ -86,8 +131,9 @@ struct __align__(16) Ctl {
   // words apart; the threads in nch chunks of tpc, chunk q sweeping quads q, q + nch, ..
   int nq, gq, lw, nch, tpc;
   uint32_t k0, k1, tag_main, tag_ref;
-  int joint, icm_big, stage_swt;
-  int oThr, oThh, oHist, oS, oV, oJn, oStage, oSwt;   // word offsets of the arrays below
+  int joint, icm_big;
+  int swt_len;       // entries of each pair's swap table in shared memory
+  int oThr, oThh, oHist, oS, oV, oJn, oPos, oStage, oSwt;   // word offsets of the arrays below
   const uint32_t *swapidx, *swaptab;   // the problem's swap tables in global memory
   int8_t *best_spins;                  // where this CTA's best state goes
   int64_t m64[4];      // best E, best sweep, hit sweep, target
@@ -97,8 +143,8 @@ struct __align__(16) Ctl {
   int32_t satt[128], sacc[128];   // swap attempts / accepts of this launch
   uint32_t ikx[64];    // per pair: Philox word 0
   int32_t ibit[64];    // per pair: replica choice bit; [32 ..]: 4-label matching per temperature
-  int32_t inm[64];     // per pair: mismatch count
-  int32_t isz[64];     // per pair: cluster size
+  int32_t inm[32];     // per pair: mismatch count
+  int32_t isz[32];     // per pair: cluster size
   uint32_t imask[24];  // [3][8] per group: cluster-flip masks, whole flips
   uint32_t swm[24];    // [8] per group: in-group swap nibble mask; [8] cross-group flags;
                        // [6] ICM matching nibble masks (4 labels)
@@ -112,17 +158,29 @@ struct __align__(16) Ctl {
 //   thh  [64][16]    their top halves, 16-bit, each group's 256 bytes on a 256-byte boundary
 //   hist [T][n_bins] pilot histogram
 //   stage [2][4][64] peer boundary spins by attempt parity, one bit per site (split)
-//   swt  [T-1][kSwtLen] first entries of each pair's swap table (split)
+//   swt  [T-1][swt_len] first entries (|dE| = 0, 2, ..) of each pair's swap table; larger |dE| read
+//                    the table in global memory, two dependent loads on the deciding warp's path
 //   S    [nq][2][H][W]  spin words: group q gq + u, colour c, site j at ((2 q + c) H + j) W + u, so
 //                    the words of a site's groups move as one vector access
-//   V    ICM cluster bits [2][H], overlap bits [2][H], transposed overlaps [N/32][32], root masks
+//   V    ICM cluster bits and overlap bits, block-major (below), transposed overlaps
+//        [N/32][33], root masks
+//   pos  [2][H] 16-bit: a site's place in the block-major arrays
 //   jn   [2][H]      coupling signs (bits 0-5), missing bonds (8-13), vacancy (15) and, from bit
 //                    16, the site's place: x odd in its row pair, wraps of +x -x +y -y +z -z
 
-// Entries of each pair's swap table (|dE| = 0, 2, .., 2 (kSwtLen - 1)) that a
-// split problem's CTAs keep in shared memory; larger |dE| read the table in
-// global memory.
-constexpr int kSwtLen = 256;
+// The cluster and overlap words of ICM are kept by 2 x 2 x 2 block: site
+// i = dx + 2 dy + 4 dz of block b at i kBlk + b (at most 512 blocks).  The
+// constant stride makes every access of the flood fill a block index plus an
+// immediate, and block kBlk - 1 of the cluster words stays 0, so that an
+// absent outside neighbour (open axis) needs no mask.
+constexpr int kBlk = 513;
+constexpr int kFillRounds = PC_APT_FILL_ROUNDS;
+constexpr int kXtStride = 33;   // a lane per chunk or a lane per pair: no bank conflict either way
+// words from V on: V, X, the transposed X (or the cluster labels), root masks
+__host__ __device__ inline int icm_words(int N) {
+  const int nchunk = (N + 31) >> 5;
+  return 16 * kBlk + kXtStride * nchunk + nchunk;
+}
 
 extern __shared__ __align__(16) uint32_t smem_words[];
 __device__ __forceinline__ uint32_t *dyn_smem() { return smem_words; }
@@ -145,6 +203,11 @@ __device__ __forceinline__ int group_off(const Ctl &k, int g) {
 }
 __device__ __forceinline__ uint32_t &spin_word(const Ctl &k, uint32_t *S, int g, int kk) {
   return S[group_off(k, g) + (kk << k.lw)];
+}
+
+// Label of local group g (at most four labels of Gu groups each).
+__device__ __forceinline__ int label_of(const Ctl &k, int g) {
+  return (g >= k.Gu ? 1 : 0) + (g >= 2 * k.Gu ? 1 : 0) + (g >= 3 * k.Gu ? 1 : 0);
 }
 
 // Neighbours (other colour, colour-local index) of site (c, j) with packed
@@ -368,7 +431,7 @@ __device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int qu
 
 template <bool UPDATE, bool ENERGY, bool OPEN>
 __device__ __forceinline__ void colour_phase_t(Ctl &k, int c, uint32_t sweep) {
-  const int q = (int)threadIdx.x / k.tpc, lt = (int)threadIdx.x - q * k.tpc;
+  const int q = (int)threadIdx.x >= k.tpc ? 1 : 0, lt = (int)threadIdx.x - q * k.tpc;   // nch is 1 or 2
   for (int quad = q; quad < k.nq; quad += k.nch) {
     switch (k.gq) {
       case 4: quad_sites<4, 4, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc); break;
@@ -439,7 +502,7 @@ __device__ __noinline__ void measure(int half, int64_t sweeps) {
   uint32_t key = 0xFFFFFFFFu;
   int bestb = 0;
   for (int b = lane; b < 8 * k.Gc; b += 32) {
-    const int lg = b >> 3, lab = lg / k.Gu, r = 8 * (k.g0 + lg - lab * k.Gu) + (b & 7);
+    const int lg = b >> 3, lab = label_of(k, lg), r = 8 * (k.g0 + lg - lab * k.Gu) + (b & 7);
     if (r >= k.T) continue;
     const uint32_t kb = ((uint32_t)(k.E[b] + (1 << 18)) << 8) | (uint32_t)(r * k.A + lab);
     if (kb < key) {
@@ -492,17 +555,24 @@ __device__ __forceinline__ uint32_t warp_transpose32(uint32_t x) {
   return x;
 }
 
-// Nibble mask (bit 4i) <-> byte (bit i) of eight pairs.
-__device__ __forceinline__ uint32_t nib_to_byte(uint32_t z) {
-  uint32_t t = z & 0x11111111u;
-  t = (t | (t >> 3)) & 0x03030303u;
-  t = (t | (t >> 6)) & 0x000F000Fu;
-  return (t | (t >> 12)) & 0xFFu;
+// Pair p of temperature r = r0 + 8h + i owns bit 4i + b, b = h P + p < 4, of
+// the per-site overlap and cluster words (A labels form P = A/2 pairs): eight
+// pairs' nibble bits enter with one shift and leave with one.  Temperature
+// of pair bit pb, or T and more where the bit has no pair.
+__device__ __forceinline__ int pair_temp(const Ctl &k, int pb) {
+  const int P = k.A >> 1, b = pb & 3;
+  return b < k.Gu * P ? 8 * (k.g0 + (b >> (P - 1))) + (pb >> 2) : k.T;
 }
-__device__ __forceinline__ uint32_t byte_to_nib(uint32_t b) {
-  uint32_t t = (b | (b << 12)) & 0x000F000Fu;
-  t = (t | (t << 6)) & 0x03030303u;
-  return (t | (t << 3)) & 0x11111111u;
+
+// Place of canonical site kk = c H + j in the block-major arrays.
+__device__ __forceinline__ int block_pos(const Ctl &k, int kk) {
+  const int c = kk >= k.H ? 1 : 0, j = kk - c * k.H;
+  const int row = (int)fdiv((uint32_t)j, k.mhx);   // j / hx
+  const int bx = j - row * k.hx;
+  const int z = (int)fdiv((uint32_t)row, k.mLy);   // row / Ly
+  const int y = row - z * k.Ly;
+  const int i = ((y + z + c) & 1) + 2 * (y & 1) + 4 * (z & 1);
+  return i * kBlk + bx + k.hx * ((y >> 1) + (k.Ly >> 1) * (z >> 1));
 }
 
 // Union-find over 32-bit parent words in shared memory, every parent no
@@ -542,33 +612,34 @@ __device__ __forceinline__ void uf_union(uint32_t *L, uint32_t a, uint32_t b) {
 // clusters, the k-th root, k = floor(x0 n / 2^32), seeds the pair's flood
 // fill.  The labels use the transposed-overlap words, which this rule does
 // not need; R holds one root bit per site.
-__device__ __forceinline__ void icm_cluster_seeds(Ctl &k, int nbits, int r0, int P) {
+__device__ __forceinline__ void icm_cluster_seeds(Ctl &k) {
   const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int N = k.N, H = k.H, nchunk = (N + 31) >> 5;
-  uint32_t *V = dyn_smem() + k.oV, *X = V + N, *Lb = V + 2 * N, *R = V + 2 * N + 32 * nchunk;
+  uint32_t *V = dyn_smem() + k.oV, *X = V + 8 * kBlk, *Lb = V + 16 * kBlk, *R = Lb + kXtStride * nchunk;
   const uint32_t *jn = dyn_smem() + k.oJn;
+  const uint16_t *pos = reinterpret_cast<const uint16_t *>(dyn_smem() + k.oPos);
   volatile uint32_t *Lv = Lb;
-  for (int pb = 0; pb < nbits; ++pb) {
-    if (r0 + 8 * ((pb >> 3) >> (P - 1)) + (pb & 7) >= k.T || k.inm[pb] == 0) continue;
-    for (int kk = tid; kk < N; kk += nt) Lb[kk] = ((X[kk] >> pb) & 1u) ? (uint32_t)kk : 0xFFFFFFFFu;
+  for (int pb = 0; pb < 32; ++pb) {
+    if (pair_temp(k, pb) >= k.T || k.inm[pb] == 0) continue;
+    for (int kk = tid; kk < N; kk += nt) Lb[kk] = ((X[pos[kk]] >> pb) & 1u) ? (uint32_t)kk : 0xFFFFFFFFu;
     __syncthreads();
     // every bond has one colour-0 end: unite each colour-0 mismatch site
     // with its mismatched neighbours over the bonds present
     for (int j = tid; j < H; j += nt) {
-      if (!((X[j] >> pb) & 1u)) continue;
+      if (!((X[pos[j]] >> pb) & 1u)) continue;
       int nb[6];
       neighbours(k, j, jn[j], nb);
       const uint32_t miss = (jn[j] >> 8) & 0x3Fu;
 #pragma unroll
       for (int d = 0; d < 6; ++d) {
         const int kk2 = H + nb[d];
-        if (((miss >> d) & 1u) == 0u && ((X[kk2] >> pb) & 1u)) uf_union(Lb, (uint32_t)j, (uint32_t)kk2);
+        if (((miss >> d) & 1u) == 0u && ((X[pos[kk2]] >> pb) & 1u)) uf_union(Lb, (uint32_t)j, (uint32_t)kk2);
       }
     }
     __syncthreads();
     for (int ch = warp; ch < nchunk; ch += (nt >> 5)) {
       const int kk = ch * 32 + lane;
-      const bool root = kk < N && ((X[kk] >> pb) & 1u) && uf_find(Lv, (uint32_t)kk) == (uint32_t)kk;
+      const bool root = kk < N && ((X[pos[kk]] >> pb) & 1u) && uf_find(Lv, (uint32_t)kk) == (uint32_t)kk;
       const uint32_t m = __ballot_sync(0xFFFFFFFFu, root);
       if (lane == 0) R[ch] = m;
     }
@@ -593,17 +664,17 @@ __device__ __forceinline__ void icm_cluster_seeds(Ctl &k, int nbits, int r0, int
         const int ex = base + inc - cn;
         const bool hit = kth >= ex && kth < ex + cn;
         if (hit) {
-          int q = kth - ex, pos = 0;
+          int q = kth - ex, at = 0;
 #pragma unroll
           for (int h = 16; h >= 1; h >>= 1) {
             const int cl = __popc(w & ((1u << h) - 1u));
             if (q >= cl) {
               q -= cl;
               w >>= h;
-              pos += h;
+              at += h;
             }
           }
-          V[ch * 32 + pos] |= 1u << pb;
+          V[pos[ch * 32 + at]] |= 1u << pb;
         }
         if (__any_sync(0xFFFFFFFFu, hit)) break;
         base += __shfl_sync(0xFFFFFFFFu, inc, 31);
@@ -616,7 +687,7 @@ __device__ __forceinline__ void icm_cluster_seeds(Ctl &k, int nbits, int r0, int
 // ICMop of Algorithm S2 for every temperature at once.  With A labels per
 // temperature (2 or 4) the labels of temperature r = 8h + i sit in nibble i
 // of groups l*Gl + h, and pair p of the temperature's random matching owns
-// bit 8 (h A/2 + p) + i of the per-site overlap word X, so the overlaps of
+// bit 4i + h A/2 + p of the per-site overlap word X, so the overlaps of
 // eight pairs come from one XOR (two labels) or three masked XORs (four).
 // The seed of a pair is the k-th site (canonical order c*H + j) with its
 // bit set, k = floor(x0 n_minus / 2^32); its cluster grows by a flood fill
@@ -624,7 +695,7 @@ __device__ __forceinline__ void icm_cluster_seeds(Ctl &k, int nbits, int r0, int
 // N/2 flip one whole replica (x1 bit 0: the pair's first or second label),
 // smaller ones flip in both replicas; then the energies are updated.
 // Overlap bits of one site: the XOR of the two labels' words of each pair,
-// nibbles packed to bits (pair bit 8 (h A/2 + p) + i).  p points at the
+// pair bit 4i + h A/2 + p for nibble i of group h.  p points at the
 // site's words of quad 0, p1 at those of quad 1.
 template <int A, int GL>
 __device__ __forceinline__ uint32_t site_overlap(const Ctl &k, const uint32_t *p, const uint32_t *p1) {
@@ -635,7 +706,7 @@ __device__ __forceinline__ uint32_t site_overlap(const Ctl &k, const uint32_t *p
     load_vec<NW>(p, w);
     if constexpr (GL > 2) load_vec<GL>(p1, w1);
 #pragma unroll
-    for (int h = 0; h < GL; ++h) xb |= nib_to_byte(w[h] ^ (GL > 2 ? w1[h] : w[NW - GL + h])) << (8 * h);
+    for (int h = 0; h < GL; ++h) xb |= (w[h] ^ (GL > 2 ? w1[h] : w[NW - GL + h])) << h;
   } else {
     // the two labels of pair p depend on each temperature's matching:
     // select nibbles by the matching masks
@@ -657,7 +728,7 @@ __device__ __forceinline__ uint32_t site_overlap(const Ctl &k, const uint32_t *p
       const uint32_t m0 = k.swm[16 + 3 * h], m1 = k.swm[17 + 3 * h], m2 = k.swm[18 + 3 * h];
       const uint32_t x0 = ((w0 ^ wa) & m0) | ((w0 ^ wb) & m1) | ((w0 ^ wc) & m2);
       const uint32_t x1 = ((wb ^ wc) & m0) | ((wa ^ wc) & m1) | ((wa ^ wb) & m2);
-      xb |= (nib_to_byte(x0) << (16 * h)) | (nib_to_byte(x1) << (16 * h + 8));
+      xb |= (x0 << (2 * h)) | (x1 << (2 * h + 1));
     }
   }
   return xb;
@@ -673,7 +744,7 @@ __device__ __forceinline__ void site_flip(const Ctl &k, uint32_t *p, uint32_t *p
     if constexpr (GL > 2) load_vec<GL>(p1, w1);
 #pragma unroll
     for (int h = 0; h < GL; ++h) {
-      const uint32_t vv = byte_to_nib((v >> (8 * h)) & 0xFFu);
+      const uint32_t vv = v >> h;   // the masks keep every fourth bit
       w[h] ^= (vv & fm[4 * h]) | fm[4 * h + 1];
       (GL > 2 ? w1[h] : w[NW - GL + h]) ^= (vv & fm[4 * h + 2]) | fm[4 * h + 3];
     }
@@ -687,7 +758,7 @@ __device__ __forceinline__ void site_flip(const Ctl &k, uint32_t *p, uint32_t *p
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int g = 4 * q + u, h = g % GL;   // g = label GL + h
-        const uint32_t n0 = byte_to_nib((v >> (16 * h)) & 0xFFu), n1 = byte_to_nib((v >> (16 * h + 8)) & 0xFFu);
+        const uint32_t n0 = v >> (2 * h), n1 = v >> (2 * h + 1);
         w[u] ^= k.imask[16 + g] | (n0 & k.imask[2 * g]) | (n1 & k.imask[2 * g + 1]);
       }
       store_vec<4>(pq, w);
@@ -699,26 +770,29 @@ __device__ __forceinline__ void site_flip(const Ctl &k, uint32_t *p, uint32_t *p
 // transpose of the chunk's X words gives lane r the chunk's mismatch
 // bitmask of pair r, kept in Xt[chunk][r].
 template <int A, int GL>
-__device__ __forceinline__ void icm_overlaps(Ctl &k, int nbits) {
+__device__ __forceinline__ void icm_overlaps(Ctl &k) {
   constexpr int W = A * GL == 2 ? 2 : 4;   // words per site and quad
   const int N = k.N, lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5, nchunk = (N + 31) >> 5;
   const uint32_t *S = dyn_smem() + k.oS, *jn = dyn_smem() + k.oJn;
-  uint32_t *V = dyn_smem() + k.oV, *X = V + N, *Xt = V + 2 * N;
+  uint32_t *V = dyn_smem() + k.oV, *X = V + 8 * kBlk, *Xt = V + 16 * kBlk;
+  const uint16_t *pos = reinterpret_cast<const uint16_t *>(dyn_smem() + k.oPos);
   uint32_t nmis = 0;             // lane r: mismatches of pair r in this warp's chunks
+#pragma unroll 2
   for (int ch = warp; ch < nchunk; ch += nw) {
     const int kk = ch * 32 + lane;
     uint32_t xb = 0;
     if (kk < N) {
       xb = site_overlap<A, GL>(k, S + kk * W, S + (N + kk) * W);
       if (jn[kk] & 0x8000u) xb = 0;   // a vacancy has no overlap: never a seed or member
-      X[kk] = xb;
-      V[kk] = 0u;
+      const int q = pos[kk];
+      X[q] = xb;
+      V[q] = 0u;
     }
     const uint32_t col = warp_transpose32(xb);
-    Xt[ch * 32 + lane] = col;
+    Xt[ch * kXtStride + lane] = col;
     nmis += __popc(col);
   }
-  if (lane < nbits && nmis) atomicAdd(&k.inm[lane], (int)nmis);
+  if (nmis) atomicAdd(&k.inm[lane], (int)nmis);
 }
 
 // (E) flips, the masks read once into registers.
@@ -728,6 +802,7 @@ __device__ __forceinline__ void icm_flips(Ctl &k) {
   const int N = k.N;
   uint32_t *S = dyn_smem() + k.oS;
   const uint32_t *V = dyn_smem() + k.oV;
+  const uint16_t *pos = reinterpret_cast<const uint16_t *>(dyn_smem() + k.oPos);
   uint32_t fm[4 * GL];
   if constexpr (A == 2) {
 #pragma unroll
@@ -739,7 +814,7 @@ __device__ __forceinline__ void icm_flips(Ctl &k) {
     }
   }
   for (int kk = threadIdx.x; kk < N; kk += blockDim.x)
-    site_flip<A, GL>(k, S + kk * W, S + (N + kk) * W, V[kk], fm);
+    site_flip<A, GL>(k, S + kk * W, S + (N + kk) * W, V[pos[kk]], fm);
 }
 
 template <bool CSEED>
@@ -750,17 +825,17 @@ __device__ __noinline__ void icm_all(uint32_t t) {
 #endif
   const int tid = threadIdx.x, nt = blockDim.x;
   const int N = k.N, H = k.H;
-  // A labels per temperature form A/2 pairs; label l's groups are
-  // l*Gl .. l*Gl + Gl - 1.  Pair p of temperature r = 8h + i owns bit
-  // 8 (h P + p) + i of the per-site overlap / cluster words.
-  const int A = k.A, P = A >> 1, Gl = k.Gu, nbits = 8 * Gl * P;   // A is 2 or 4
+  // label l's groups are l*Gl .. l*Gl + Gl - 1; A is 2 or 4
+  const int A = k.A, P = A >> 1, Gl = k.Gu;
   const int r0 = 8 * k.g0;   // first temperature held here
-  uint32_t *V = dyn_smem() + k.oV;   // [2][H] cluster bits (one bit per pair)
-  uint32_t *X = V + N;               // [2][H] overlap bits
-  uint32_t *Xt = V + 2 * N;          // [nchunk][32]
+  uint32_t *V = dyn_smem() + k.oV;   // cluster bits (one bit per pair), block-major
+  uint32_t *X = V + 8 * kBlk;        // overlap bits, block-major
+  uint32_t *Xt = V + 16 * kBlk;      // [nchunk][kXtStride]
+  const uint16_t *pos = reinterpret_cast<const uint16_t *>(dyn_smem() + k.oPos);
   int *match = k.ibit + 32;          // [32] matching of the labels of each temperature
-  if (tid < nbits) {
-    const int pb = tid, beta = pb >> 3, h = beta >> (P - 1), p = beta - h * P, r = r0 + 8 * h + (pb & 7);
+  // the draws, on warp 1 (warp 0 may still be measuring)
+  if (tid >= 32 && tid < 64) {
+    const int pb = tid - 32, p = pb & (P - 1), r = pair_temp(k, pb);   // b = h P + p, P is 1 or 2
     if (r < k.T) {
       const uint4 x = philox((uint32_t)r, t, (uint32_t)p, (k.ent << 8) | TAG_ICM, k.k0, k.k1);
       k.ikx[pb] = x.x;
@@ -771,10 +846,9 @@ __device__ __noinline__ void icm_all(uint32_t t) {
       if (p == 0) match[r] = A == 4 ? (int)(((uint64_t)x.z * 3u) >> 32) : 0;
     }
   }
-  if (tid < 24) k.imask[tid] = 0;
-  if (tid < 64) {
-    k.isz[tid] = 0;
-    k.inm[tid] = 0;
+  if (tid >= 32 && tid < 64) {
+    k.isz[tid - 32] = 0;
+    k.inm[tid - 32] = 0;
   }
   __syncthreads();
   if (k.m32[1]) copy_best();
@@ -794,177 +868,200 @@ __device__ __noinline__ void icm_all(uint32_t t) {
   const int lane = tid & 31, warp = tid >> 5, nw = nt >> 5, nchunk = (N + 31) >> 5;
   if (A == 2) {
     switch (Gl) {
-      case 4: icm_overlaps<2, 4>(k, nbits); break;
-      case 3: icm_overlaps<2, 3>(k, nbits); break;
-      case 2: icm_overlaps<2, 2>(k, nbits); break;
-      default: icm_overlaps<2, 1>(k, nbits); break;
+      case 4: icm_overlaps<2, 4>(k); break;
+      case 3: icm_overlaps<2, 3>(k); break;
+      case 2: icm_overlaps<2, 2>(k); break;
+      default: icm_overlaps<2, 1>(k); break;
     }
   } else if (Gl == 2) {
-    icm_overlaps<4, 2>(k, nbits);
+    icm_overlaps<4, 2>(k);
   } else {
-    icm_overlaps<4, 1>(k, nbits);
+    icm_overlaps<4, 1>(k);
   }
   __syncthreads();
   PROF_MARK(4, pt);
   // seeds: warp w finds the k-th mismatch of pairs w, w + nw, ...: chunk
   // counts by popcount, a warp scan over chunks, then the set bit inside
   // the chunk (the cluster-seed rule finds the k-th cluster instead)
-  if (CSEED) icm_cluster_seeds(k, nbits, r0, P);
-  for (int r = warp; r < nbits && !CSEED; r += nw) {   // r: pair bit
-    if (r0 + 8 * ((r >> 3) >> (P - 1)) + (r & 7) >= k.T) continue;
-    const int nm = k.inm[r];
-    if (nm == 0) continue;
-    const int kth = (int)(((uint64_t)k.ikx[r] * (uint64_t)nm) >> 32);
-    int base = 0;
-    for (int ch0 = 0; ch0 < nchunk; ch0 += 32) {
-      const int ch = ch0 + lane;
-      uint32_t w = ch < nchunk ? Xt[ch * 32 + r] : 0u;
+  if (CSEED) icm_cluster_seeds(k);
+  if (!CSEED && nchunk <= 8 && warp == 0) {
+    // few chunks: a lane per pair walks them
+    const int r = lane, nm = pair_temp(k, r) < k.T ? k.inm[r] : 0;
+    int q = (int)(((uint64_t)k.ikx[r] * (uint64_t)nm) >> 32);
+    bool find = nm > 0;
+    for (int ch = 0; ch < nchunk && find; ++ch) {
+      uint32_t w = Xt[ch * kXtStride + r];
       const int cn = __popc(w);
-      int inc = cn;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
-        if (lane >= o) inc += y;
-      }
-      const int ex = base + inc - cn;
-      const bool hit = kth >= ex && kth < ex + cn;
-      if (hit) {
-        // position of set bit number q (from 0) of w: binary search on
-        // popcounts of the low half of the remaining window
-        int q = kth - ex, pos = 0;
+      if (q < cn) {
+        int at = 0;
 #pragma unroll
         for (int h = 16; h >= 1; h >>= 1) {
           const int cl = __popc(w & ((1u << h) - 1u));
           if (q >= cl) {
             q -= cl;
             w >>= h;
-            pos += h;
+            at += h;
           }
         }
-        atomicOr(&V[ch * 32 + pos], 1u << r);
+        atomicOr(&V[pos[ch * 32 + at]], 1u << r);
+        find = false;
       }
-      if (__any_sync(0xFFFFFFFFu, hit)) break;
-      base += __shfl_sync(0xFFFFFFFFu, inc, 31);
+      q -= cn;
+    }
+  }
+  const int nb = Gl * P;   // pairs per nibble, 1 .. 4
+  for (int v = warp; v < 8 * nb && !CSEED && nchunk > 8; v += nw) {
+    const int vi = nb == 4 ? v >> 2 : nb == 3 ? (v * 43) >> 7 : v >> (nb - 1);   // v / nb, v < 32
+    const int r = 4 * vi + v - nb * vi;                                           // pair bit
+    if (pair_temp(k, r) >= k.T) continue;
+    const int nm = k.inm[r];
+    if (nm == 0) continue;
+    int kth = (int)(((uint64_t)k.ikx[r] * (uint64_t)nm) >> 32);
+    // lane l takes chunks [l cl, (l + 1) cl): its count, one scan over the
+    // lanes, and the lane that holds the kth mismatch walks its chunks
+    const int cl = (nchunk + 31) >> 5, c0 = lane * cl, c1 = min(nchunk, c0 + cl);
+    int cn = 0;
+#pragma unroll 4
+    for (int ch = c0; ch < c1; ++ch) cn += __popc(Xt[ch * kXtStride + r]);
+    int inc = cn;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xFFFFFFFFu, inc, o);
+      if (lane >= o) inc += y;
+    }
+    kth -= inc - cn;
+    if (kth >= 0 && kth < cn) {
+      for (int ch = c0; ch < c1; ++ch) {
+        uint32_t w = Xt[ch * kXtStride + r];
+        const int n1 = __popc(w);
+        if (kth < n1) {
+          // set bit number kth of w: binary search on popcounts of the low
+          // half of the remaining window
+          int at = 0;
+#pragma unroll
+          for (int h = 16; h >= 1; h >>= 1) {
+            const int lo = __popc(w & ((1u << h) - 1u));
+            if (kth >= lo) {
+              kth -= lo;
+              w >>= h;
+              at += h;
+            }
+          }
+          atomicOr(&V[pos[ch * 32 + at]], 1u << r);
+          break;
+        }
+        kth -= n1;
+      }
     }
   }
   __syncthreads();
   PROF_MARK(5, pt);
   // (B) flood fill.  The cluster is the least fixed point of the monotone
-  // update V <- V | (X & OR_nbr V).  A thread owns 2x2x2 blocks of sites
-  // (bx, by, bz): per pass it reads the 24 outside neighbours of a block and
-  // closes the block internally (the cube has diameter 3), so a pass moves
-  // a cluster front by up to three sites.  Each site word has one writer,
-  // so passes run without inner barriers (a stale neighbour read only delays
-  // growth) and a pass with no change anywhere, started after a barrier,
-  // proves the fixed point.
+  // update V <- V | (X & OR_nbr V).  A thread owns 2x2x2 blocks of sites: per
+  // pass it reads the 24 outside neighbours of a block (each the opposite
+  // site's word of an adjacent block), then spreads inside the cube axis by
+  // axis, kFillRounds times.  Each site word has one writer, so passes run
+  // without inner barriers (a stale neighbour read only delays growth), and a
+  // pass with no change anywhere, started after a barrier, proves the fixed
+  // point: it ORs in every neighbour of every site.  A pass is a chain of
+  // dependent loads and logic on few warps (216 blocks at L = 12), so what
+  // counts is its length: 64 x L = 12, 14 passes, 15.1k cycles with 24
+  // computed addresses and masks and three rounds of all six directions,
+  // 10.5k so (two rounds per pass 11.0k, three 11.6k: fewer passes do not
+  // pay for longer ones).
   {
-    const Ctl &g = k;
-    const int hx = g.hx, hy = g.Ly >> 1, nblk = N >> 3;
-    // plain loads: a pass reads each neighbour word once, after the barrier
-    // that ended the previous pass (a compiler fence as well), and a value
-    // another thread writes during the pass is only seen one pass later
-    const uint32_t *Vv = V;
-    // block geometry: site i = dx + 2 dy + 4 dz of block (bx, by, bz) has
-    // colour (dx+dy+dz)&1 and index bx + hx (y0 + dy + Ly (z0 + dz)) inside
-    // its colour; an outside neighbour is the opposite corner's word of the
-    // adjacent block, i.e. a site of this block shifted by one block step
-    struct Blk {
-      int kk[8];
-      uint32_t dx2, dy2, dz2;   // (minus, plus) block steps as two int16 each
-      uint32_t ok;              // bits -x,+x,-y,+y,-z,+z: outside neighbour present
-    };
-    auto make_blk = [&](int blk) {
-      Blk B;
-      const int rest = (int)fdiv((uint32_t)blk, g.mhx);           // blk / hx
+    const int hx = k.hx, hy = k.Ly >> 1, hz = k.Lz >> 1, nblk = N >> 3;
+    constexpr int kZero = kBlk - 1;   // the block of zeros
+    // indices of the six adjacent blocks, -x +x -y +y -z +z; an open axis has
+    // no bond across its ends
+    auto adjacent = [&](int blk, int (&nb)[6]) {
+      const int rest = (int)fdiv((uint32_t)blk, k.mhx);           // blk / hx
       const int bx = blk - rest * hx;
-      const int bz = (int)fdiv((uint32_t)rest, g.mLy2);           // rest / (Ly/2)
+      const int bz = (int)fdiv((uint32_t)rest, k.mLy2);           // rest / (Ly/2)
       const int by = rest - bz * hy;
-      const int y0 = 2 * by, z0 = 2 * bz;
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int dx = i & 1, dy = (i >> 1) & 1, dz = i >> 2;
-        B.kk[i] = ((dx + dy + dz) & 1) * H + bx + hx * (y0 + dy + g.Ly * (z0 + dz));
-      }
-      const int LyHx = g.Ly * hx;
-      auto pack = [](int m, int p) { return ((uint32_t)m & 0xFFFFu) | ((uint32_t)p << 16); };
-      B.dx2 = pack(bx == 0 ? hx - 1 : -1, bx + 1 == hx ? 1 - hx : 1);
-      B.dy2 = pack(hx * (y0 == 0 ? g.Ly - 2 : -2), hx * (y0 + 2 == g.Ly ? 2 - g.Ly : 2));
-      B.dz2 = pack(LyHx * (z0 == 0 ? g.Lz - 2 : -2), LyHx * (z0 + 2 == g.Lz ? 2 - g.Lz : 2));
-      // an open axis has no bond across its ends
-      B.ok = 0x3Fu;
-      if (k.open & 1u) B.ok &= ~((bx == 0 ? 1u : 0u) | (bx + 1 == hx ? 2u : 0u));
-      if (k.open & 2u) B.ok &= ~((y0 == 0 ? 4u : 0u) | (y0 + 2 == g.Ly ? 8u : 0u));
-      if (k.open & 4u) B.ok &= ~((z0 == 0 ? 16u : 0u) | (z0 + 2 == g.Lz ? 32u : 0u));
-      return B;
+      const int sy = hx, sz = hx * hy;
+      nb[0] = bx > 0 ? blk - 1 : ((k.open & 1u) ? kZero : blk + hx - 1);
+      nb[1] = bx + 1 < hx ? blk + 1 : ((k.open & 1u) ? kZero : blk - (hx - 1));
+      nb[2] = by > 0 ? blk - sy : ((k.open & 2u) ? kZero : blk + sz - sy);
+      nb[3] = by + 1 < hy ? blk + sy : ((k.open & 2u) ? kZero : blk - (sz - sy));
+      nb[4] = bz > 0 ? blk - sz : ((k.open & 4u) ? kZero : blk + sz * (hz - 1));
+      nb[5] = bz + 1 < hz ? blk + sz : ((k.open & 4u) ? kZero : blk - sz * (hz - 1));
     };
-    // one relaxation of a block: outside neighbours, then the internal
-    // closure (three rounds reach across the cube); writes changed words
-    auto relax = [&](const Blk &B, const uint32_t (&x)[8], uint32_t (&v)[8]) {
+    // one relaxation of a block; writes its words if any changed
+    auto relax = [&](int blk, const int (&nb)[6], const uint32_t (&x)[8], uint32_t (&v)[8]) {
       uint32_t nv[8];
-      const int dxm = (int16_t)(B.dx2 & 0xFFFFu), dxp = (int16_t)(B.dx2 >> 16);
-      const int dym = (int16_t)(B.dy2 & 0xFFFFu), dyp = (int16_t)(B.dy2 >> 16);
-      const int dzm = (int16_t)(B.dz2 & 0xFFFFu), dzp = (int16_t)(B.dz2 >> 16);
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
-        const int dx = i & 1, dy = (i >> 1) & 1, dz = i >> 2;
-        const uint32_t mx = ((B.ok >> dx) & 1u) ? ~0u : 0u;
-        const uint32_t my = ((B.ok >> (2 + dy)) & 1u) ? ~0u : 0u;
-        const uint32_t mz = ((B.ok >> (4 + dz)) & 1u) ? ~0u : 0u;
-        const uint32_t ox = Vv[B.kk[i ^ 1] + (dx ? dxp : dxm)] & mx;
-        const uint32_t oy = Vv[B.kk[i ^ 2] + (dy ? dyp : dym)] & my;
-        const uint32_t oz = Vv[B.kk[i ^ 4] + (dz ? dzp : dzm)] & mz;
+        const uint32_t ox = V[(i ^ 1) * kBlk + nb[i & 1]];
+        const uint32_t oy = V[(i ^ 2) * kBlk + nb[2 + ((i >> 1) & 1)]];
+        const uint32_t oz = V[(i ^ 4) * kBlk + nb[4 + (i >> 2)]];
         nv[i] = v[i] | (x[i] & (ox | oy | oz));
       }
 #pragma unroll
-      for (int round = 0; round < 3; ++round) {
+      for (int round = 0; round < kFillRounds; ++round) {
 #pragma unroll
-        for (int i = 0; i < 8; ++i) nv[i] |= x[i] & (nv[i ^ 1] | nv[i ^ 2] | nv[i ^ 4]);
-      }
-      int ch = 0;
+        for (int ax = 1; ax <= 4; ax <<= 1) {
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        if (nv[i] != v[i]) {
-          V[B.kk[i]] = nv[i];
-          v[i] = nv[i];
-          ch = 1;
+          for (int i = 0; i < 8; ++i)
+            if (!(i & ax)) {
+              const uint32_t a0 = nv[i], a1 = nv[i ^ ax];
+              nv[i] = a0 | (x[i] & a1);
+              nv[i ^ ax] = a1 | (x[i ^ ax] & a0);
+            }
         }
       }
-      return ch;
+      uint32_t d = 0;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) d |= nv[i] ^ v[i];
+      if (d) {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          V[i * kBlk + blk] = nv[i];
+          v[i] = nv[i];
+        }
+      }
+      return d != 0u;
     };
-    if (nblk <= nt) {
-      // one block per thread: its geometry and cluster words stay in
-      // registers across passes (the thread is their only writer)
-      Blk B;
-      uint32_t v[8];
-#if PC_APT_FILL_XREG
-      uint32_t x[8];   // the block's overlap words do not change during the fill
-#endif
+    if (nblk <= 32) {
+      // small lattices: one warp, passes end with a vote instead of a barrier
+      if (warp == 0) {
+        int nb[6];
+        uint32_t v[8], x[8];
+        if (lane < nblk) adjacent(lane, nb);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          v[i] = lane < nblk ? V[i * kBlk + lane] : 0u;
+          x[i] = lane < nblk ? X[i * kBlk + lane] : 0u;
+        }
+        for (int it = 0; it < N; ++it) {
+          const bool changed = lane < nblk && relax(lane, nb, x, v);
+          __syncwarp();
+          if (!__any_sync(0xFFFFFFFFu, changed)) break;
+        }
+      }
+      __syncthreads();
+    } else if (nblk <= nt) {
+      // one block per thread: its neighbours, cluster and overlap words stay
+      // in registers across passes (the thread is their only writer)
+      int nb[6];
+      uint32_t v[8], x[8];
       bool open = false;
       if (tid < nblk) {
-        B = make_blk(tid);
+        adjacent(tid, nb);
         uint32_t o = 0;
 #pragma unroll
         for (int i = 0; i < 8; ++i) {
-          v[i] = V[B.kk[i]];
-#if PC_APT_FILL_XREG
-          x[i] = X[B.kk[i]];
+          v[i] = V[i * kBlk + tid];
+          x[i] = X[i * kBlk + tid];
           o |= x[i] & ~v[i];
-#else
-          o |= X[B.kk[i]] & ~v[i];
-#endif
         }
         open = o != 0;
       }
       for (int it = 0; it < N; ++it) {
         int changed = 0;
         if (open) {
+          changed = relax(tid, nb, x, v);
           uint32_t o = 0;
-#if !PC_APT_FILL_XREG
-          uint32_t x[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) x[i] = X[B.kk[i]];
-#endif
-          changed = relax(B, x, v);
 #pragma unroll
           for (int i = 0; i < 8; ++i) o |= x[i] & ~v[i];
           open = o != 0;
@@ -980,53 +1077,82 @@ __device__ __noinline__ void icm_all(uint32_t t) {
       for (int it = 0; it < N; ++it) {
         int changed = 0;
         for (int blk = tid; blk < nblk; blk += nt) {
-          const Blk B = make_blk(blk);
           uint32_t x[8], v[8];
           uint32_t open = 0;
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            x[i] = X[B.kk[i]];
-            v[i] = Vv[B.kk[i]];
+            x[i] = X[i * kBlk + blk];
+            v[i] = V[i * kBlk + blk];
             open |= x[i] & ~v[i];
           }
-          if (open) changed |= relax(B, x, v);
+          if (open) {
+            int nb[6];
+            adjacent(blk, nb);
+            changed |= relax(blk, nb, x, v);
+          }
         }
         if (!__syncthreads_or(changed)) break;
       }
     }
   }
   PROF_MARK(6, pt);
-  // (C) cluster sizes: per chunk, lane r counts pair r's cluster sites
+  // (C) cluster sizes.  A lane adds the eight words of its block into four
+  // bit planes (counts 0 .. 8 of every pair); the transposes of a warp's
+  // planes give lane r pair r's counts over 32 blocks.
   {
+    const int nblk = N >> 3;
     uint32_t sz = 0;
-    for (int ch = warp; ch < nchunk; ch += nw) {
-      const int kk = ch * 32 + lane;
-      sz += __popc(warp_transpose32(kk < N ? V[kk] : 0u));
+    for (int b0 = 32 * warp; b0 < nblk; b0 += nt) {
+      const int b = b0 + lane;
+      uint32_t w[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) w[i] = b < nblk ? V[i * kBlk + b] : 0u;
+      auto add3 = [](uint32_t x, uint32_t y, uint32_t z, uint32_t &cy) {
+        cy = (x & y) | (x & z) | (y & z);
+        return x ^ y ^ z;
+      };
+      uint32_t c0, c1, c2, c3, c4, c5;
+      const uint32_t s0 = add3(w[0], w[1], w[2], c0), s1 = add3(w[3], w[4], w[5], c1);
+      const uint32_t s2 = add3(s0, s1, w[6], c2), p0 = s2 ^ w[7];
+      c3 = s2 & w[7];
+      const uint32_t t = add3(c0, c1, c2, c4), p1 = t ^ c3;
+      c5 = t & c3;
+      sz += (uint32_t)__popc(warp_transpose32(p0)) + 2u * (uint32_t)__popc(warp_transpose32(p1)) +
+            4u * (uint32_t)__popc(warp_transpose32(c4 ^ c5)) + 8u * (uint32_t)__popc(warp_transpose32(c4 & c5));
     }
-    if (lane < nbits && sz) atomicAdd(&k.isz[lane], (int)sz);
+    if (sz) atomicAdd(&k.isz[lane], (int)sz);
   }
   __syncthreads();
-  // (D) decisions.  imask[(g P + p)] (g = l Gl + h): nibbles of label l's
-  // group h flipped by pair p's cluster; imask[16 + g]: whole-replica flips.
-  if (tid < nbits) {
-    const int pb = tid, beta = pb >> 3, h = beta >> (P - 1), p = beta - h * P, i = pb & 7,
-              r = r0 + 8 * h + i;
-    if (r < k.T) {
-      const int m = match[r];
-      const int la = p == 0 ? 0 : (m == 0 ? 2 : 1);
-      const int lb = p == 0 ? m + 1 : (m == 2 ? 2 : 3);
-      const int size = k.isz[pb];
-      const uint32_t bit = 1u << (4 * i);
-      if (k.inm[pb] == 0) {
-        atomicAdd(&k.m32[2], 1);
-      } else if (k.icm_big && 2 * size > k.nreal) {   // more than half of the spins present
-        atomicOr(&k.imask[16 + (k.ibit[pb] ? lb : la) * Gl + h], bit);   // one whole replica
-        atomicAdd(&k.m32[4], 1);
-      } else {
-        atomicOr(&k.imask[(la * Gl + h) * P + p], bit);                  // cluster, both replicas
-        atomicOr(&k.imask[(lb * Gl + h) * P + p], bit);
-        atomicAdd(&k.m32[3], 1);
+  // (D) decisions, warp 0, a lane per pair.  imask[(g P + p)] (g = l Gl + h):
+  // nibbles of label l's group h flipped by pair p's cluster; imask[16 + g]:
+  // whole-replica flips.  The lanes' bits reach the masks as ballots: pair
+  // bits h P + p, h P + p + 4, .. are the nibbles of group h.
+  if (warp == 0) {
+    const int pb = lane, p = pb & (P - 1), r = pair_temp(k, pb);
+    const bool valid = r < k.T;
+    const int m = valid ? match[r] : 0;
+    const int la = p == 0 ? 0 : (m == 0 ? 2 : 1);
+    const int lb = p == 0 ? m + 1 : (m == 2 ? 2 : 3);
+    const bool none = valid && k.inm[pb] == 0;
+    const bool big = valid && !none && k.icm_big && 2 * k.isz[pb] > k.nreal;   // more than half of the spins present
+    const bool small = valid && !none && !big;
+    const int whole = big ? (k.ibit[pb] ? lb : la) : -1;   // the replica that flips whole
+    const uint32_t mn = __ballot_sync(0xFFFFFFFFu, none), ms = __ballot_sync(0xFFFFFFFFu, small),
+                   mb = __ballot_sync(0xFFFFFFFFu, big);
+    for (int l = 0; l < A; ++l) {
+      const uint32_t fl = __ballot_sync(0xFFFFFFFFu, small && (la == l || lb == l));
+      const uint32_t wh = __ballot_sync(0xFFFFFFFFu, whole == l);
+      if (lane < Gl * P) k.imask[l * Gl * P + lane] = (fl >> lane) & 0x11111111u;
+      if (lane < Gl) {
+        uint32_t w = 0u;
+        for (int q = 0; q < P; ++q) w |= (wh >> (lane * P + q)) & 0x11111111u;
+        k.imask[16 + l * Gl + lane] = w;
       }
+    }
+    if (lane == 0) {
+      k.m32[2] += __popc(mn);
+      k.m32[3] += __popc(ms);
+      k.m32[4] += __popc(mb);
     }
   }
   __syncthreads();
@@ -1072,7 +1198,7 @@ __device__ __forceinline__ void swap_quads(Ctl &k, int c, uint32_t bmask, const 
       if (u + 1 < GQ && g + 1 < k.Gc && k.swm[8 + g]) cross |= 1u << u;
       bl[u] = 0u;
       if (bmask && g < k.Gc) {
-        const int l = g / k.Gu;
+        const int l = label_of(k, g);
         if (g - l * k.Gu == bgoff && ((bmask >> l) & 1u)) bl[u] = (uint32_t)(64 * l) + 1u;   // 1 + its stage row
         any |= bl[u];
       }
@@ -1154,13 +1280,13 @@ __device__ __noinline__ void swap_step(uint32_t t) {
 #if PC_APT_PROFILE
   long long pt = clock64();
 #endif
-  const int A = k.A, q = (int)(t & 1u);
+  const int A = k.A, lA2 = A >> 1, q = (int)(t & 1u);   // A = 1 << lA2 (1, 2 or 4)
   const int r0 = 8 * k.g0, r1 = min(8 * (k.g0 + k.Gu), k.T);   // temperatures held here
   // local buffer of (label l, temperature r): l * 8 Gu + r - r0
   const int lb = 8 * k.Gu;
   auto swap_table = [&](int r, int dE) {
     const int kk = (-dE) >> 1;
-    if (PC_APT_STAGE_SWT && SPLIT && k.stage_swt && kk < kSwtLen) return dyn_smem()[k.oSwt + r * kSwtLen + kk];   // staged at launch
+    if (kk < k.swt_len) return dyn_smem()[k.oSwt + r * k.swt_len + kk];   // staged at launch
     const uint32_t off = k.swapidx[2 * r], len = k.swapidx[2 * r + 1];
     return ((uint32_t)kk < len) ? k.swaptab[off + kk] : 0u;
   };
@@ -1193,7 +1319,7 @@ __device__ __noinline__ void swap_step(uint32_t t) {
     // for all labels at once, with the summed energy difference
     const int nd = k.joint ? np : np * A;
     for (int idx = lane; idx < nd; idx += 32) {
-      const int r = first + 2 * (k.joint ? idx : idx / A), al = k.joint ? 0 : idx % A;
+      const int r = first + 2 * (k.joint ? idx : idx >> lA2), al = k.joint ? 0 : idx & (A - 1);
       // the draw first: it does not depend on the energies
       const uint32_t x0 = philox((uint32_t)r, t, (uint32_t)al, (k.ent << 8) | TAG_SWAP, k.k0, k.k1).x;
       const int bA = al * lb + r - r0, bB = bA + 1;
@@ -1224,34 +1350,30 @@ __device__ __noinline__ void swap_step(uint32_t t) {
     cooperative_groups::this_cluster().sync();   // the peer's energies and spins have landed
     // the pair (rb - 1, rb) across the two CTAs, if this attempt's parity
     const int rb = k.rank == 0 ? r1 : r0;
-    if (threadIdx.x == 0) {
-      uint32_t accm = 0;
-      if (rb < k.T && ((rb - 1) & 1) == q) {
-        const int rb_own = k.rank == 0 ? r1 - 1 : r0;
-        const int *pe = k.xch + 4 * par;   // the peer's energies
-        int e_lo[4], e_hi[4];               // energies at rb - 1 (rank 0's) and rb (rank 1's)
-        for (int l = 0; l < A; ++l) {
-          const int own = k.E[l * lb + rb_own - r0];
-          e_lo[l] = k.rank == 0 ? own : pe[l];
-          e_hi[l] = k.rank == 0 ? pe[l] : own;
-        }
-        for (int l = 0; l < (k.joint ? 1 : A); ++l) {
-          int dE = e_hi[l] - e_lo[l];
-          if (k.joint)
-            for (int m = 1; m < A; ++m) dE += e_hi[m] - e_lo[m];
-          // the draw taken by warp 1 before the barrier
-          const bool acc = dE >= 0 || (uint32_t)k.xch[18 + l] < swap_table(rb - 1, dE);
-          if (acc) accm |= k.joint ? (1u << A) - 1u : 1u << l;
-        }
-        for (int l = 0; l < A; ++l) {
-          if (k.rank == 0) k.satt[(rb - 1) * A + l] += 1;   // counted once, by rank 0
-          if ((accm >> l) & 1u) {
-            if (k.rank == 0) k.sacc[(rb - 1) * A + l] += 1;
-            k.E[l * lb + rb_own - r0] = k.rank == 0 ? e_hi[l] : e_lo[l];
-          }
-        }
+    if (threadIdx.x < 32) {
+      // a lane per label
+      const int l = threadIdx.x, rb_own = k.rank == 0 ? r1 - 1 : r0;
+      const bool on = l < A && rb < k.T && ((rb - 1) & 1) == q;
+      int e_lo = 0, e_hi = 0;               // energies at rb - 1 (rank 0's) and rb (rank 1's)
+      if (on) {
+        const int own = k.E[l * lb + rb_own - r0], peer = k.xch[4 * par + l];
+        e_lo = k.rank == 0 ? own : peer;
+        e_hi = k.rank == 0 ? peer : own;
       }
-      k.xch[8] = (int)accm;
+      const int sum = (int)__reduce_add_sync(0xFFFFFFFFu, (unsigned)(e_hi - e_lo));
+      bool acc = false;
+      if (on) {
+        const int dE = k.joint ? sum : e_hi - e_lo;
+        // the draw taken by warp 1 before the barrier
+        acc = dE >= 0 || (uint32_t)k.xch[18 + (k.joint ? 0 : l)] < swap_table(rb - 1, dE);
+        if (k.rank == 0) {   // counted once, by rank 0
+          k.satt[(rb - 1) * A + l] += 1;
+          if (acc) k.sacc[(rb - 1) * A + l] += 1;
+        }
+        if (acc) k.E[l * lb + rb_own - r0] = k.rank == 0 ? e_hi : e_lo;
+      }
+      const uint32_t accm = __ballot_sync(0xFFFFFFFFu, acc);
+      if (l == 0) k.xch[8] = (int)accm;
     }
     __syncthreads();
     bmask = (uint32_t)k.xch[8];
@@ -1328,7 +1450,7 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     k.tag_ref = a.tag_ref;
     k.joint = a.joint_swap;
     k.icm_big = a.icm_big;
-    k.stage_swt = a.stage_swt;
+    k.swt_len = MODE == pc::APT_MODE_APT ? a.swt_len : 0;
     k.swapidx = a.swapidx + P.swapidx_off;
     k.swaptab = a.swaptab;
     k.best_spins = (rank ? a.best_spins2 : a.best_spins) + P.best_off;
@@ -1343,10 +1465,11 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     k.oThh = o;    o += 64 * Gp;
     k.oHist = o;   o += MODE == pc::APT_MODE_PILOT ? (P.T * a.n_bins + 3) & ~3 : 0;
     k.oStage = o;  o += SPLIT ? 512 : 0;
-    k.oSwt = o;    o += (SPLIT && MODE == pc::APT_MODE_APT && a.stage_swt) ? max(P.T - 1, 0) * kSwtLen : 0;
+    k.oSwt = o;    o += (max(P.T - 1, 0) * k.swt_len + 3) & ~3;
     k.oS = o;      o += site_words(Gm) * N;
-    k.oV = o;      o += icm ? 3 * N + 31 + ((N + 31) >> 5) : 0;
-    k.oJn = o;
+    k.oV = o;      o += icm ? icm_words(N) : 0;
+    k.oJn = o;     o += N;
+    k.oPos = o;
     k.m64[0] = a.best_E[p];
     k.m64[1] = a.best_sweep[p];
     k.m64[2] = a.hit_sweep[p];
@@ -1368,7 +1491,9 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
       const int c = i >= H ? 1 : 0;
       jn[i] = (uint32_t)a.jneg[P.jneg_off + i] | place_bits(k, c, i - c * H);
+      if (icm) reinterpret_cast<uint16_t *>(smem + k.oPos)[i] = (uint16_t)block_pos(k, i);
     }
+    if (icm && threadIdx.x < 8) smem[k.oV + threadIdx.x * kBlk + kBlk - 1] = 0u;
     for (int b = threadIdx.x; b < 64; b += blockDim.x) {
       k.Eacc[b] = 0;
       if (b >= 8 * k.Gc) continue;
@@ -1389,12 +1514,11 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
       k.sacc[i] = 0;
     }
     if (threadIdx.x < 24) k.xch[threadIdx.x] = 0;
-    if (PC_APT_STAGE_SWT && SPLIT && MODE == pc::APT_MODE_APT && a.stage_swt)
-      for (int i = threadIdx.x; i < (k.T - 1) * kSwtLen; i += blockDim.x) {
-        const int r = i / kSwtLen, kk = i - r * kSwtLen;
-        const uint32_t off = k.swapidx[2 * r], len = k.swapidx[2 * r + 1];
-        smem[k.oSwt + i] = ((uint32_t)kk < len) ? a.swaptab[off + kk] : 0u;
-      }
+    for (int i = threadIdx.x; i < (k.T - 1) * k.swt_len; i += blockDim.x) {
+      const int r = i / k.swt_len, kk = i - r * k.swt_len;
+      const uint32_t off = k.swapidx[2 * r], len = k.swapidx[2 * r + 1];
+      smem[k.oSwt + i] = ((uint32_t)kk < len) ? a.swaptab[off + kk] : 0u;
+    }
     if (MODE == pc::APT_MODE_PILOT)
       for (int i = threadIdx.x; i < k.T * a.n_bins; i += blockDim.x) smem[k.oHist + i] = 0u;
   }
@@ -1599,14 +1723,13 @@ __global__ void apt_init_kernel(const AptArgs a, int n_prob) {
 
 namespace pc {
 
-size_t apt_smem_bytes(int N, int Gc, int nwarps, int mode, int icm, int T, int n_bins, int stage_swt) {
+size_t apt_smem_bytes(int N, int Gc, int mode, int icm, int T, int n_bins, int swt_len) {
   const int Gp = quads_of(Gc) * quad_groups(Gc);
   size_t words = sizeof(Ctl) / 4 + 192 * (size_t)Gp + 64 + 512;   // thr, thh and its alignment, stage
   if (mode == APT_MODE_PILOT) words += ((size_t)T * n_bins + 3) & ~(size_t)3;
-  if (mode == APT_MODE_APT && stage_swt) words += (size_t)(T > 1 ? T - 1 : 0) * kSwtLen;   // staged swap tables
+  if (mode == APT_MODE_APT) words += ((size_t)(T > 1 ? T - 1 : 0) * swt_len + 3) & ~(size_t)3;   // staged swap tables
   words += (size_t)site_words(Gc) * N;
-  // V, X, the transposed X (or the cluster labels) and the root masks
-  if (mode == APT_MODE_APT && icm) words += (size_t)3 * N + 31 + (size_t)((N + 31) >> 5);
+  if (mode == APT_MODE_APT && icm) words += (size_t)icm_words(N) + (size_t)(N + 1) / 2;   // and the sites' places
   return (words + (size_t)N) * 4;
 }
 

@@ -51,7 +51,7 @@ struct Batch {
   int split_h = 0;       // split problems: temperature groups per label on rank 0 (0: half)
   size_t smem = 0;       // max of the two parts
   size_t smem_u = 0, smem_s = 0;
-  int stage_swt = 1;     // the split part stages swap tables (when its CTAs still fit)
+  int swt_u = 0, swt_s = 0;   // swap-table entries per pair in shared memory, by part
   std::vector<uint32_t> h_pbit, h_swaptab, h_swapidx;
 };
 
@@ -266,7 +266,7 @@ AptArgs base_args(pc_ctx *c, Batch &bt) {
   a.spp = 1;
   a.icm_big = 1;
   a.icm_seed = 0;
-  a.stage_swt = bt.stage_swt;
+  a.swt_len = bt.split ? bt.swt_s : bt.swt_u;
   return a;
 }
 
@@ -326,7 +326,11 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
   }
   // [0]: one-CTA part, [1]: two-CTA-cluster part
   std::vector<int> cp[2], cg0[2], cgc[2], cnch[2];
-  size_t smem[2] = {0, 0}, smem_ns = 0;   // smem_ns: the split part without staged swap tables
+  // swap-table entries per pair in shared memory: the most that fit (energy
+  // gaps up to 510, 126; none where a part is too large: 32 temperatures x 4
+  // labels on 16^3)
+  constexpr int kSwtLens[3] = {256, 64, 0};
+  size_t smem[2][3] = {};
   for (int i : order) {
     const AptProbDev &P = bt.prob[(size_t)i];
     const int G = bt.G[(size_t)i];
@@ -345,8 +349,8 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
         cnch[1].push_back(choose_nch(P.N / 2, P.A * gu, bt.tpb, bt.nch_pref));
       }
       const int gmx = P.A * std::max(h1, Glp - h1);
-      smem[1] = std::max(smem[1], apt_smem_bytes(P.N, gmx, bt.tpb / 32, mode, icm, P.T, n_bins, 1));
-      smem_ns = std::max(smem_ns, apt_smem_bytes(P.N, gmx, bt.tpb / 32, mode, icm, P.T, n_bins, 0));
+      for (int q = 0; q < 3; ++q)
+        smem[1][q] = std::max(smem[1][q], apt_smem_bytes(P.N, gmx, mode, icm, P.T, n_bins, kSwtLens[q]));
       continue;
     }
     // equal chunks of at most gmax groups
@@ -357,19 +361,23 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
       cg0[0].push_back(g0);
       cgc[0].push_back(gc);
       cnch[0].push_back(choose_nch(P.N / 2, gc, bt.tpb, bt.nch_pref));
-      smem[0] = std::max(smem[0], apt_smem_bytes(P.N, gc, bt.tpb / 32, mode, icm, P.T, n_bins, 0));
+      for (int q = 0; q < 3; ++q)
+        smem[0][q] = std::max(smem[0][q], apt_smem_bytes(P.N, gc, mode, icm, P.T, n_bins, kSwtLens[q]));
     }
   }
-  // the split part stages its swap tables only where its CTAs still fit
-  bt.stage_swt = smem[1] <= (size_t)c->smem_optin;
-  if (!bt.stage_swt) smem[1] = smem_ns;
+  int fit[2] = {2, 2};
+  for (int part = 0; part < 2; ++part)
+    for (int q = 2; q >= 0; --q)
+      if (smem[part][q] <= (size_t)c->smem_optin) fit[part] = q;
   bt.n_u = (int)cp[0].size();
   bt.n_s = (int)cp[1].size();
   bt.split = bt.n_s > 0 && bt.n_u == 0;
   bt.hybrid = bt.n_s > 0 && bt.n_u > 0;
-  bt.smem_u = smem[0];
-  bt.smem_s = smem[1];
-  const size_t smem_max = std::max(smem[0], smem[1]);
+  bt.swt_u = kSwtLens[fit[0]];
+  bt.swt_s = kSwtLens[fit[1]];
+  bt.smem_u = smem[0][fit[0]];
+  bt.smem_s = smem[1][fit[1]];
+  const size_t smem_max = std::max(bt.smem_u, bt.smem_s);
   bt.n_cta = bt.n_u + bt.n_s;
   for (int part = 0; part < 2; ++part)
     for (int g : cgc[part])
@@ -443,6 +451,8 @@ int launch_parts(Batch &bt, AptArgs a, cudaStream_t st, Fork &f) {
   PC_CUDA_TRY(cudaDeviceGetStreamPriorityRange(&least, &greatest));
   as.split = 1;
   as.prio = greatest;
+  as.swt_len = bt.swt_s;
+  au.swt_len = bt.swt_u;
   as.cta_prob = ts;
   as.cta_g0 = ts + bt.n_s;
   as.cta_gc = ts + 2 * bt.n_s;

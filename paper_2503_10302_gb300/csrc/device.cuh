@@ -36,57 +36,6 @@ __device__ __forceinline__ uint32_t word_of(const uint4 &x, int w) {
   return w == 0 ? x.x : (w == 1 ? x.y : (w == 2 ? x.z : x.w));
 }
 
-// The first two rounds of philox(c0, c1, c2, c3) taken apart, for draws that
-// pair many (c0, c3) with many (c1, c2).  Round 1 turns c0 and c2 into
-// products that do not meet before round 2, whose product of the c2 lane
-// depends on (c0, c3) alone and whose product of the c0 lane depends on
-// (c1, c2) alone: a site's part is shared by its replica groups, a group's
-// part by the sites, and a draw starts at round 3 after two XORs (saves 4 of
-// 20 wide products, the half-rate instructions, and 2 of 20 XORs).
-struct PhiloxA { uint32_t lo0, b_lo, b_hi; };   // of (c0, c3)
-struct PhiloxB { uint32_t x0, x2, lo; };        // of (c1, c2), round-2 keys folded in
-
-__device__ __forceinline__ PhiloxA philox_a(uint32_t c0, uint32_t c3, uint32_t k1) {
-  PhiloxA p;
-  p.lo0 = 0xD2511F53u * c0;
-  const uint32_t n2 = __umulhi(0xD2511F53u, c0) ^ c3 ^ k1;
-  p.b_lo = 0xCD9E8D57u * n2;
-  p.b_hi = __umulhi(0xCD9E8D57u, n2);
-  return p;
-}
-__device__ __forceinline__ PhiloxB philox_b(uint32_t c1, uint32_t c2, uint32_t k0, uint32_t k1) {
-  PhiloxB p;
-  const uint32_t n0 = __umulhi(0xCD9E8D57u, c2) ^ c1 ^ k0;
-  p.x0 = (0xCD9E8D57u * c2) ^ (k0 + 0x9E3779B9u);
-  p.x2 = __umulhi(0xD2511F53u, n0) ^ (k1 + 0xBB67AE85u);
-  p.lo = 0xD2511F53u * n0;
-  return p;
-}
-__device__ __forceinline__ uint4 philox_ab(const PhiloxA &a, const PhiloxB &b, uint32_t k0, uint32_t k1) {
-  uint32_t c0 = a.b_hi ^ b.x0, c1 = a.b_lo, c2 = b.x2 ^ a.lo0, c3 = b.lo;
-  k0 += 2u * 0x9E3779B9u;
-  k1 += 2u * 0xBB67AE85u;
-#pragma unroll
-  for (int r = 2; r < 10; ++r) {
-    const uint32_t lo0 = 0xD2511F53u * c0, hi0 = __umulhi(0xD2511F53u, c0);
-    const uint32_t lo1 = 0xCD9E8D57u * c2, hi1 = __umulhi(0xCD9E8D57u, c2);
-    c0 = hi1 ^ c1 ^ k0;
-    c2 = hi0 ^ c3 ^ k1;
-    c1 = lo1;
-    c3 = lo0;
-    k0 += 0x9E3779B9u;
-    k1 += 0xBB67AE85u;
-  }
-  return make_uint4(c0, c1, c2, c3);
-}
-
-// The 16-bit word at a shared-window address.
-__device__ __forceinline__ uint32_t lds_u16(uint32_t addr) {
-  uint32_t v;
-  asm("ld.shared.u16 %0, [%1];" : "=r"(v) : "r"(addr));
-  return v;
-}
-
 // Half-word i of a Philox block placed in the high 16 bits (low bits 0).
 __device__ __forceinline__ uint32_t half_hi(const uint4 &x, int i) {
   const uint32_t w = word_of(x, i >> 1);
