@@ -14,6 +14,8 @@
 // (slice, vertex) entry of the replicated network, in the same way.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+#include <atomic>
 #include <climits>
 #include <cooperative_groups.h>
 #include <cstdint>
@@ -843,8 +845,8 @@ int gapt_launch_t(const GAptArgs &a, int n_prob, size_t smem, bool init, cudaStr
 }
 
 // DT-SQA on the replicated network of a graph (Eq. S.3, Algorithm S1),
-// multi-spin coded: a CTA anneals 32 runs, whose spins of one (slice,
-// vertex) share a word, and a thread owns one entry (slice k, vertex p) of
+// multi-spin coded: a CTA anneals 8 G8 runs (32, or 16 where 32 would leave
+// SMs without work), whose spins of one (slice, vertex) share a word, and a thread owns one entry (slice k, vertex p) of
 // the colour class being swept.  The in-slice field is summed bit-sliced
 // over the neighbour words (NP planes); the two time neighbours' words give
 // each run's count of +1 neighbours in imaginary time.  Run q takes half
@@ -861,7 +863,7 @@ int gapt_launch_t(const GAptArgs &a, int n_prob, size_t smem, bool init, cudaStr
 // shared memory, and every colour phase ends with a cluster barrier.
 // SMG: the vertex table and adjacency are staged in shared memory (else
 // they are read through the L1 cache).
-template <int NP, bool REP, bool CL, bool SMG>
+template <int NP, bool REP, bool CL, bool SMG, int G8>
 __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
   namespace cg = cooperative_groups;
   extern __shared__ __align__(16) uint32_t dyn[];
@@ -869,7 +871,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
   const int nt = 2 * a.Imax + 1, ntab = 3 * nt, TB = REP ? 32 * ntab : ntab;
   const int n = a.n, P = a.P;
   const int CS = CL ? a.CS : 1, rank = CL ? (int)cg::this_cluster().block_rank() : 0;
-  const int grp = (int)blockIdx.x / CS;                       // run group (32 runs)
+  const int grp = (int)blockIdx.x / CS;                       // run group (8 G8 runs)
   const int kb = rank * P / CS, ke = (rank + 1) * P / CS;     // own slices [kb, ke)
   const int nkmax = (P + CS - 1) / CS;                        // equal carve in every CTA
   uint32_t *tab = dyn;                       // [2][TB]
@@ -894,7 +896,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
     Wl = cg::this_cluster().map_shared_rank(W, rl) + (size_t)((rl + 1) * P / CS - rl * P / CS - 1) * n;
     Wr = cg::this_cluster().map_shared_rank(W, rr);
   }
-  const uint32_t g0 = (a.run0 >> 3) + 4u * (uint32_t)grp;   // run group of bit 0 (run0 % 8 == 0)
+  const uint32_t g0 = (a.run0 >> 3) + (uint32_t)(G8 * grp);   // run group of bit 0 (run0 % 8 == 0)
   // this CTA's part of colour class c: entries [o0 + lo, o0 + hi) of the class list
   auto part = [&](int c, int &o0, int &lo, int &hi) {
     o0 = a.cls_off[c];
@@ -909,7 +911,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
       const uint32_t e = __ldg(a.cls + o0 + j);
       uint32_t word = 0u;
 #pragma unroll
-      for (int g = 0; g < 4; ++g) {
+      for (int g = 0; g < G8; ++g) {
         const uint4 x = philox((uint32_t)j, 0u, (uint32_t)c, ((g0 + g) << 8) | TAG_GS_INIT, a.k0, a.k1);
 #pragma unroll
         for (int i = 0; i < 8; ++i)
@@ -943,7 +945,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
         // decisions and the exact settlement of possible ties as in g_sweep
         uint32_t word = 0u, gmask = 0u;
 #pragma unroll
-        for (int g = 3; g >= 0; --g) {
+        for (int g = G8 - 1; g >= 0; --g) {
           const uint4 x = philox((uint32_t)j, (uint32_t)s, (uint32_t)c, ((g0 + g) << 8) | TAG_GS_SWEEP, a.k0, a.k1);
           uint32_t tp = 1u;
           // three planes (Imax <= 7): the group's table indices
@@ -973,7 +975,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
         }
         if (gmask) {
 #pragma unroll 1
-          for (int g = 0; g < 4; ++g) {
+          for (int g = 0; g < G8; ++g) {
             if (!((gmask >> g) & 1u)) continue;
             const uint32_t gq = (g0 + (uint32_t)g) << 8;
             const uint4 x = philox((uint32_t)j, (uint32_t)s, (uint32_t)c, gq | TAG_GS_SWEEP, a.k0, a.k1);
@@ -1007,7 +1009,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
   // of higher base colour, biases included), bit-sliced as in the APT
   // energy pass: e_v = W_l + |h| - 2 U per run, U counted per run by warp
   // transposes over blocks of 32 vertices
-  const int runs_here = min(32, a.R - 32 * grp);
+  const int runs_here = min(8 * G8, a.R - 8 * G8 * grp);
   const int nb32 = (n + 31) / 32;
   for (int it0 = 32 * warp; it0 < 32 * (ke - kb) * nb32; it0 += kGThreads) {
     const int blk = it0 >> 5, k = kb + blk / nb32, v = 32 * (blk % nb32) + lane;
@@ -1040,7 +1042,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gsqa_kernel(GSqaArgs a) {
     for (int q = 0; q < NP; ++q) cnt += __popc(transpose32(U[q], lane)) << q;
     const long long ek = (long long)__reduce_add_sync(0xFFFFFFFFu, (unsigned)K) - 2LL * cnt;
     if (lane < runs_here)
-      atomicAdd(reinterpret_cast<unsigned long long *>(&a.E[(size_t)(32 * grp + lane) * P + k]),
+      atomicAdd(reinterpret_cast<unsigned long long *>(&a.E[(size_t)(8 * G8 * grp + lane) * P + k]),
                 (unsigned long long)ek);
   }
   if (a.spins)
@@ -1056,14 +1058,81 @@ size_t gsqa_smem_bytes(int n, int P, int Imax, int m, int CS) {
   return sizeof(uint32_t) * (((base + 1) & ~(size_t)1) + 2 * (size_t)n + (size_t)m);
 }
 
-template <int NP, bool REP, bool CL, bool SMG>
+namespace {
+
+// Clusters of cs CTAs with an SM each that the device holds at a time (0:
+// none), asked once per device and size.
+__global__ void __launch_bounds__(kGThreads, 1) cluster_probe_kernel() {}
+int exclusive_clusters(int cs) {
+  static std::atomic<int> known[64][17];   // 1 + the answer
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64 || cs < 1 || cs > 16) return 0;
+  const int k = known[dev][cs].load();
+  if (k) return k - 1;
+  int n = 0;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)cs);
+  cfg.blockDim = dim3((unsigned)kGThreads);
+  cfg.dynamicSmemBytes = kGSqaAloneBytes;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = (unsigned)cs;
+  attr[0].val.clusterDim.y = 1;
+  attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  if (cudaFuncSetAttribute(cluster_probe_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGSqaAloneBytes) !=
+          cudaSuccess ||
+      cudaFuncSetAttribute(cluster_probe_kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, cluster_probe_kernel, &cfg) != cudaSuccess) {
+    cudaGetLastError();
+    n = 0;
+  }
+  known[dev][cs].store(n + 1);
+  return n;
+}
+
+}  // namespace
+
+// A colour phase of a CTA takes about 7.8k cycles per 512 words of 32 runs
+// (one per thread), 0.6 of that with 16 runs, not below 3.5k and 2.1k (one
+// warp's chain of decisions), and a barrier, about 0.1k cycles in a CTA and
+// 0.6k in a cluster.  More CTAs per run group, and 16 instead of 32 runs in a
+// group, pay while every CTA still has an SM to itself (5400 p-bits, 64
+// slices, 256 runs, 200 sweeps: 8 groups x 8 CTAs on 64 SMs 48.8 ms,
+// x 11 CTAs on 88 SMs 38.9 ms).
+GSqaShape gsqa_shape(int cs_min, int n, int P, int C, int R, int sms) {
+  GSqaShape best = {cs_min, 32, false};
+  double best_t = 1e300;
+  for (int rw = 32; rw >= 16; rw /= 2) {
+    const int groups = (R + rw - 1) / rw;
+    const double f = rw == 32 ? 1.0 : 0.6;
+    for (int cs = cs_min; cs <= 16 && cs <= P; ++cs) {
+      const bool base = cs == cs_min && rw == 32;
+      const bool alone = groups * cs <= sms && exclusive_clusters(cs) >= groups;
+      if (!alone && !base) continue;
+      const int waves = alone ? 1 : std::max(1, (groups * cs + sms - 1) / sms);
+      const double words = (double)n * ((P + cs - 1) / cs) / C;
+      const double t = waves * (f * std::max(3500.0, 7800.0 * words / 512.0) + (cs > 1 ? 600.0 : 100.0));
+      if (t < 0.95 * best_t) {   // a larger shape has to gain
+        best_t = t;
+        best = {cs, rw, alone && !base};
+      }
+    }
+  }
+  return best;
+}
+
+template <int NP, bool REP, bool CL, bool SMG, int G8>
 int gsqa_launch_t(const GSqaArgs &a, size_t smem, cudaStream_t st) {
-  auto kern = gsqa_kernel<NP, REP, CL, SMG>;
+  auto kern = gsqa_kernel<NP, REP, CL, SMG, G8>;
   PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  const unsigned grid = (unsigned)(((a.R + 31) / 32) * (CL ? a.CS : 1));
+  const unsigned grid = (unsigned)(((a.R + 8 * G8 - 1) / (8 * G8)) * (CL ? a.CS : 1));
   if (!CL) {
     kern<<<grid, kGThreads, smem, st>>>(a);
   } else {
+    // above the portable 8 CTAs the cluster size has to be allowed
+    if (a.CS > 8) PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3((unsigned)kGThreads);
@@ -1082,18 +1151,23 @@ int gsqa_launch_t(const GSqaArgs &a, size_t smem, cudaStream_t st) {
   return PC_OK;
 }
 
-int gsqa_launch(const GSqaArgs &a, bool staged, size_t smem, cudaStream_t st) {
+template <int G8>
+int gsqa_launch_g(const GSqaArgs &a, bool staged, size_t smem, cudaStream_t st) {
   const int sel = (a.Imax <= 7 ? 4 : 0) + (a.CS > 1 ? 2 : 0) + (staged ? 1 : 0);
   switch (sel) {
-    case 0: return gsqa_launch_t<7, false, false, false>(a, smem, st);
-    case 1: return gsqa_launch_t<7, false, false, true>(a, smem, st);
-    case 2: return gsqa_launch_t<7, false, true, false>(a, smem, st);
-    case 3: return gsqa_launch_t<7, false, true, true>(a, smem, st);
-    case 4: return gsqa_launch_t<3, true, false, false>(a, smem, st);
-    case 5: return gsqa_launch_t<3, true, false, true>(a, smem, st);
-    case 6: return gsqa_launch_t<3, true, true, false>(a, smem, st);
-    default: return gsqa_launch_t<3, true, true, true>(a, smem, st);
+    case 0: return gsqa_launch_t<7, false, false, false, G8>(a, smem, st);
+    case 1: return gsqa_launch_t<7, false, false, true, G8>(a, smem, st);
+    case 2: return gsqa_launch_t<7, false, true, false, G8>(a, smem, st);
+    case 3: return gsqa_launch_t<7, false, true, true, G8>(a, smem, st);
+    case 4: return gsqa_launch_t<3, true, false, false, G8>(a, smem, st);
+    case 5: return gsqa_launch_t<3, true, false, true, G8>(a, smem, st);
+    case 6: return gsqa_launch_t<3, true, true, false, G8>(a, smem, st);
+    default: return gsqa_launch_t<3, true, true, true, G8>(a, smem, st);
   }
+}
+
+int gsqa_launch(const GSqaArgs &a, int rw, bool staged, size_t smem, cudaStream_t st) {
+  return rw == 16 ? gsqa_launch_g<2>(a, staged, smem, st) : gsqa_launch_g<4>(a, staged, smem, st);
 }
 
 size_t gapt_smem_bytes(int n, int A, int Imax, int m) {

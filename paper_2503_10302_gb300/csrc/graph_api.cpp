@@ -577,10 +577,18 @@ int pc_gsqa_anneal(pc_ctx *c, int n, const int32_t *row_ptr, const int32_t *col,
     CS = 1;
     while (!fits(CS, false) && CS < 8 && 2 * CS <= P) CS *= 2;
   }
-  const size_t smem = gsqa_smem_bytes(n, P, g.Imax, staged ? (int)g.adj.size() : -1, CS);
+  // and to a larger one, or to groups of 16 instead of 32 runs, when the run
+  // groups leave SMs idle
+  const int Cp = std::max(g.C, (P & 1) ? 3 : 2);
+  PC_CUDA_TRY(cudaSetDevice(c->device));
+  const GSqaShape shape = gsqa_shape(CS, n, P, Cp, R, c->sms);
+  CS = shape.CS;
+  staged = fits(CS, true);
+  size_t smem = gsqa_smem_bytes(n, P, g.Imax, staged ? (int)g.adj.size() : -1, CS);
+  if (shape.alone) smem = std::max(smem, std::min(budget, kGSqaAloneBytes));
+  const int rw = shape.runs, groups = (R + rw - 1) / rw;
   if ((rc = static_smem_guard(c, smem))) return rc;
   // colour classes of the replicated network, each ordered by slice, then vertex
-  const int Cp = std::max(g.C, (P & 1) ? 3 : 2);
   std::vector<uint32_t> cls;
   std::vector<int> cls_off(Cp + 1, 0);
   for (int cp = 0; cp < Cp; ++cp) {
@@ -611,7 +619,6 @@ int pc_gsqa_anneal(pc_ctx *c, int n, const int32_t *row_ptr, const int32_t *col,
       for (int I = -g.Imax; I <= g.Imax; ++I)
         table[((size_t)s * 3 + nup) * nt + (I + g.Imax)] = sqa_threshold(beta_eff, I, jq, 2 * nup - 2);
   }
-  PC_CUDA_TRY(cudaSetDevice(c->device));
   cudaStream_t st = c->stream;
   DevBuf<int2> d_vinfo;
   DevBuf<uint32_t> d_adj, d_cls, d_table, d_spins;
@@ -619,7 +626,6 @@ int pc_gsqa_anneal(pc_ctx *c, int n, const int32_t *row_ptr, const int32_t *col,
   DevBuf<long long> d_E;
   std::vector<uint32_t> adj = g.adj;
   if (adj.empty()) adj.push_back(0u);
-  const int groups = (R + 31) / 32;
   if ((rc = upload(d_vinfo, g.vinfo, st)) || (rc = upload(d_adj, adj, st)) || (rc = upload(d_cls, cls, st)) ||
       (rc = upload(d_off, cls_off, st)) || (rc = upload(d_table, table, st)) ||
       (rc = upload(d_rank, cls_rank, st)) ||
@@ -646,7 +652,7 @@ int pc_gsqa_anneal(pc_ctx *c, int n, const int32_t *row_ptr, const int32_t *col,
   a.spins = spins_out ? d_spins.p : nullptr;
   a.CS = CS;
   a.cls_rank = d_rank.p;
-  if ((rc = gsqa_launch(a, staged, smem, st))) return rc;
+  if ((rc = gsqa_launch(a, rw, staged, smem, st))) return rc;
   std::vector<long long> E((size_t)R * P);
   PC_CUDA_TRY(cudaMemcpyAsync(E.data(), d_E.p, E.size() * 8, cudaMemcpyDeviceToHost, st));
   std::vector<uint32_t> wd;
@@ -661,7 +667,7 @@ int pc_gsqa_anneal(pc_ctx *c, int n, const int32_t *row_ptr, const int32_t *col,
       for (int k = 0; k < P; ++k)
         for (int v = 0; v < n; ++v)
           spins_out[((size_t)r * P + k) * n + v] =
-              ((wd[((size_t)(r >> 5) * P + k) * n + g.newid[v]] >> (r & 31)) & 1u) ? 1 : -1;
+              ((wd[((size_t)(r / rw) * P + k) * n + g.newid[v]] >> (r % rw)) & 1u) ? 1 : -1;
   return PC_OK;
 } catch (...) {
   return pc::fail_exception();

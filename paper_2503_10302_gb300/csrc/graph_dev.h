@@ -92,7 +92,16 @@ size_t gapt_smem_bytes(int n, int A, int Imax, int m);
 int gapt_launch(const GAptArgs &a, int n_prob, int A, int Imax, bool staged, size_t smem, bool init,
                 cudaStream_t st);
 size_t gsqa_smem_bytes(int n, int P, int Imax, int m, int CS);
+// How an anneal of R runs is cut: clusters of CS CTAs per group of `runs` (32
+// or 16) runs; alone: every CTA is to have an SM to itself.
+struct GSqaShape {
+  int CS, runs;
+  bool alone;
+};
+// n vertices, P slices, C colour classes; cs_min: the cluster the words need.
+GSqaShape gsqa_shape(int cs_min, int n, int P, int C, int R, int sms);
+constexpr size_t kGSqaAloneBytes = 116 * 1024;   // shared memory of a CTA that leaves no room for a second one
 // staged: vertex table and adjacency in shared memory (m >= 0 in gsqa_smem_bytes)
-int gsqa_launch(const GSqaArgs &a, bool staged, size_t smem, cudaStream_t st);
+int gsqa_launch(const GSqaArgs &a, int runs, bool staged, size_t smem, cudaStream_t st);
 
 }  // namespace pc

@@ -297,3 +297,16 @@ def test_gapt_cluster_fill_sizes(pc, orc, dims, deg):
     ref.run(4)
     s, e, _ = ref.state(0)
     assert np.array_equal(got[0], s) and np.array_equal(got[1], e)
+
+
+@pytest.mark.parametrize("P,R", [(13, 8), (64, 16), (33, 40)])
+def test_gsqa_run_groups_and_clusters_fill_the_gpu(pc, orc, P, R):
+    """Few runs: groups of 16 runs and larger clusters, of sizes that do not
+    divide the slices; every shape equals the oracle bit for bit."""
+    g = W.dimer_embedding((3, 4, 3), W.ea_couplings((3, 4, 3), 1000, 21))
+    gamma = W.linear_gamma_schedule(9, 2.0, 0.2)
+    ctx = pc.Context(0, 17)
+    E1, s1 = pc.pc_gsqa_anneal(ctx.h, g.rp, g.col, g.w, P, 0.2, gamma, R, run0=8, want_spins=True)
+    ctx.close()
+    E2, s2 = orc.gsqa_anneal(g.rp, g.col, g.w, P, 0.2, gamma, R, run0=8, seed=17, want_spins=True)
+    assert np.array_equal(s1, s2) and np.array_equal(E1, E2)
