@@ -57,11 +57,14 @@ struct GShared {
   uint32_t att[128], acc[128];   // swap counters [r * A + a]
   unsigned long long icm[3];
   long long bestE, bestSweep, bestSlot, hit, target;
+  int bestPhase;                 // 0: measured after the sweeps, 1: after the cluster moves
+  int fresh;                     // the best state was found in this launch
   int copy_slot;
 };
 
 struct GCta {
   int n, C, T, Imax, tid, lane, warp, deg8;
+  int lab0;                      // first label this CTA sweeps (a split problem: its only one)
   int ths;                       // row length of the [temperature][field] table
   int ushift;                    // (entry >> 8) - ubase >> ushift = neighbour index
   uint32_t ubase;                // byte offset of the spin words from the dynamic base
@@ -231,16 +234,18 @@ __device__ void g_init(const GCta &k, GShared &sh) {
 // every (vertex, label) of the class in parallel.  Replica b = 32 a + r
 // takes half b & 7 of P(j, s, (c << 16) | (b >> 3), (e << 8) | TAG), so one
 // Philox call serves 8 replicas of the vertex.
-template <int A, int NP, bool SM>
+// The AL labels from k.lab0 on are swept.
+template <int A, int NP, bool SM, int AL>
 __device__ void g_sweep(const GCta &k, GShared &sh, uint32_t s) {
   const uint32_t c3m = (k.ent << 8) | k.tag_sweep;
   const uint32_t c3r = (k.ent << 8) | k.tag_refine;
   for (int c = 0; c < k.C; ++c) {
     const int o0 = sh.off[c], nc = sh.off[c + 1] - o0;
-    const int nitems = 32 * A * ((nc + 31) / 32);
+    const int nitems = 32 * AL * ((nc + 31) / 32);
     for (int it = k.tid; it < nitems; it += kGThreads) {
       int j, a;
-      item_of<A>(it, j, a);
+      item_of<AL>(it, j, a);
+      a += k.lab0;
       if (j >= nc) continue;
       const int p = o0 + j;
       const int2 vi = ld_vi<SM>(k.vinfo, p);
@@ -326,16 +331,18 @@ __device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
 //   e_v = W_l + |h| - 2 U,   U = (s_v = +1 ? Cl : W_l - Cl) + |h| y.
 // U is formed bit-sliced (U <= Imax < 2^NP); each warp (one label, 32
 // vertices) transposes the planes and counts bits per replica.
-// AL: only the first AL labels are counted (their rows of E are rewritten).
+// AL: only the AL labels from k.lab0 on are counted (their rows of E are
+// rewritten).
 template <int A, int NP, bool SM, int AL = A>
 __device__ void g_energy(const GCta &k, GShared &sh) {
-  if (k.tid < 32 * AL) sh.E[k.tid >> 5][k.tid & 31] = 0;
+  if (k.tid < 32 * AL) sh.E[k.lab0 + (k.tid >> 5)][k.tid & 31] = 0;
   __syncthreads();
-  int eacc = 0, a_w = 0;
+  int eacc = 0, a_w = k.lab0;
   const int nitems = 32 * AL * ((k.n + 31) / 32);
   for (int it0 = 32 * k.warp; it0 < nitems; it0 += kGThreads) {
     int v, a;
     item_of<AL>(it0 + k.lane, v, a);
+    a += k.lab0;
     a_w = a;
     uint32_t U[NP];
 #pragma unroll
@@ -370,13 +377,14 @@ __device__ void g_energy(const GCta &k, GShared &sh) {
 }
 
 // Minimum-energy tracking: lowest slot r*A + a on ties, strict improvement;
-// an improvement copies that replica's state into the best-state bits.
-template <int A>
-__device__ void g_best(const GCta &k, GShared &sh, long long sweeps) {
+// an improvement copies that replica's state into the best-state bits.  A
+// split problem's CTAs track their own label's best and combine at the end.
+template <int A, int AL>
+__device__ void g_best(const GCta &k, GShared &sh, long long sweeps, int phase) {
   if (k.warp == 0) {
     int bE = INT_MAX, bB = INT_MAX;
     if (k.lane < k.T)
-      for (int aa = 0; aa < A; ++aa) {
+      for (int aa = k.lab0; aa < k.lab0 + AL; ++aa) {
         const int e = sh.E[aa][k.lane];
         if (e < bE) { bE = e; bB = k.lane * A + aa; }
       }
@@ -390,6 +398,8 @@ __device__ void g_best(const GCta &k, GShared &sh, long long sweeps) {
         sh.bestE = bE;
         sh.bestSweep = sweeps;
         sh.bestSlot = bB;
+        sh.bestPhase = phase;
+        sh.fresh = 1;
         sh.copy_slot = bB;
       }
       if (sh.hit < 0 && sh.bestE <= sh.target) sh.hit = sweeps;
@@ -413,7 +423,7 @@ __device__ void g_best(const GCta &k, GShared &sh, long long sweeps) {
 // ...; per label (or jointly over labels) accept with min(1, exp(dbeta dE))
 // through the pair's table by |dE|.  Accepted pairs exchange their states
 // (bit r and r+1 of every word of the label) and energies.
-template <int A>
+template <int A, int AL>
 __device__ void g_swap(const GCta &k, GShared &sh, uint32_t t, int joint, const uint32_t *swaptab,
                        const uint32_t *swapidx) {
   if (k.tid < 4) sh.swmask[k.tid] = 0u;
@@ -439,8 +449,8 @@ __device__ void g_swap(const GCta &k, GShared &sh, uint32_t t, int joint, const 
         }
       }
     }
-  } else if (k.tid < npairs * A) {
-    const int r = r0 + 2 * (k.tid / A), aa = k.tid % A;
+  } else if (k.tid < npairs * AL) {
+    const int r = r0 + 2 * (k.tid / AL), aa = k.lab0 + k.tid % AL;
     const long long dE = (long long)sh.E[aa][r + 1] - sh.E[aa][r];
     const uint32_t x = philox((uint32_t)r, t, (uint32_t)aa, c3, k.k0, k.k1).x;
     bool acc = dE >= 0;
@@ -455,21 +465,24 @@ __device__ void g_swap(const GCta &k, GShared &sh, uint32_t t, int joint, const 
     }
   }
   __syncthreads();
-  for (int i = k.tid; i < k.n * A; i += kGThreads) {
-    const uint32_t M = sh.swmask[i % A];
+  for (int i = k.tid; i < k.n * AL; i += kGThreads) {
+    const int a = k.lab0 + i % AL;
+    const uint32_t M = sh.swmask[a];
     if (M) {
-      const uint32_t w = k.S[i], d = (w ^ (w >> 1)) & M;
-      k.S[i] = w ^ d ^ (d << 1);
+      uint32_t &word = k.S[i / AL * A + a];
+      const uint32_t w = word, d = (w ^ (w >> 1)) & M;
+      word = w ^ d ^ (d << 1);
     }
   }
-  if (k.warp < A) {
-    const uint32_t M = sh.swmask[k.warp];
-    const int e = sh.E[k.warp][k.lane];
+  if (k.warp < AL) {
+    const int a = k.lab0 + k.warp;
+    const uint32_t M = sh.swmask[a];
+    const int e = sh.E[a][k.lane];
     int src = k.lane;
     if ((M >> k.lane) & 1u) src = k.lane + 1;
     else if (k.lane > 0 && ((M >> (k.lane - 1)) & 1u)) src = k.lane - 1;
     const int o = __shfl_sync(0xFFFFFFFFu, e, src);
-    sh.E[k.warp][k.lane] = o;
+    sh.E[a][k.lane] = o;
   }
   __syncthreads();
 }
@@ -712,13 +725,25 @@ __device__ void g_icm(const GCta &k, GShared &sh, uint32_t t) {
 // NP: bit planes of the field counts (2^NP > Imax).  SM: the problem's
 // vertex table and adjacency are staged in shared memory (when they fit)
 // instead of being read through the L1 cache.
-template <int A, int NP, bool SM>
+// CL (two labels): a problem runs as a cluster of two CTAs, each sweeping,
+// measuring and swapping one label.  Before the cluster moves each CTA reads
+// the other label's words through distributed shared memory (one cluster
+// barrier when both have swept, one when both have read); both then make the
+// same moves on their copies, of which the own label's count.  The best
+// states combine at the end of the launch: the lower energy, then the earlier
+// measurement, then the lower slot, as one CTA's tracking would have it.
+template <int A, int NP, bool SM, bool CL>
 __global__ void __launch_bounds__(kGThreads, 1) gapt_kernel(GAptArgs a, int init) {
+  namespace cg = cooperative_groups;
+  constexpr int AL = CL ? 1 : A;
   extern __shared__ __align__(16) uint32_t dyn[];
   __shared__ GShared sh;
-  if (a.active && !a.active[blockIdx.x]) return;   // converged ladder problem
-  const GProbDev &P = a.prob[blockIdx.x];
+  const int rank = CL ? (int)cg::this_cluster().block_rank() : 0;
+  const size_t prob = CL ? blockIdx.x >> 1 : blockIdx.x;
+  if (a.active && !a.active[prob]) return;   // converged ladder problem
+  const GProbDev &P = a.prob[prob];
   GCta k;
+  k.lab0 = rank;
   k.n = P.n;
   k.C = P.C;
   k.T = P.T;
@@ -756,11 +781,11 @@ __global__ void __launch_bounds__(kGThreads, 1) gapt_kernel(GAptArgs a, int init
     k.vinfo = a.vinfo + P.vbase;
     k.adj = a.adj + P.abase;
   }
-  k.best_bits = a.best_bits + P.bestbase;
+  k.best_bits = (rank ? a.best_bits2 : a.best_bits) + P.bestbase;
   uint32_t *gS = a.spins + (size_t)P.vbase * A;
   if (k.tid <= k.C) sh.off[k.tid] = P.off[k.tid];
   for (int i = k.tid; i < nth; i += kGThreads) Th[i] = a.pbit[P.thbase + i];
-  const long long *gb = a.best + 4 * (size_t)blockIdx.x;
+  const long long *gb = a.best + 4 * prob;
   if (init) {
     __syncthreads();
     g_init<A>(k, sh);
@@ -768,7 +793,7 @@ __global__ void __launch_bounds__(kGThreads, 1) gapt_kernel(GAptArgs a, int init
   } else {
     for (int i = k.tid; i < P.n * A; i += kGThreads) k.S[i] = gS[i];
     if (k.tid < 128) {
-      sh.E[k.tid >> 5][k.tid & 31] = a.E[128 * (size_t)blockIdx.x + k.tid];
+      sh.E[k.tid >> 5][k.tid & 31] = a.E[128 * prob + k.tid];
       sh.att[k.tid] = 0u;
       sh.acc[k.tid] = 0u;
     }
@@ -777,29 +802,39 @@ __global__ void __launch_bounds__(kGThreads, 1) gapt_kernel(GAptArgs a, int init
       sh.bestSweep = gb[1];
       sh.bestSlot = gb[2];
       sh.hit = gb[3];
-      sh.target = a.target[blockIdx.x];
+      sh.target = a.target[prob];
       sh.icm[0] = sh.icm[1] = sh.icm[2] = 0ull;
+      sh.bestPhase = 0;
+      sh.fresh = 0;
     }
     __syncthreads();
     const uint32_t *swidx = a.swapidx + P.swbase;
     for (int t = 0; t < a.n_swaps; ++t) {
       const uint32_t tt = a.swap0 + (uint32_t)t;
-      for (int q = 0; q < a.spp; ++q) g_sweep<A, NP, SM>(k, sh, a.sweep0 + (uint32_t)(t * a.spp + q));
-      g_energy<A, NP, SM>(k, sh);
+      for (int q = 0; q < a.spp; ++q) g_sweep<A, NP, SM, AL>(k, sh, a.sweep0 + (uint32_t)(t * a.spp + q));
+      g_energy<A, NP, SM, AL>(k, sh);
       if (a.ladder) {
         // thread tid reads (and next zeroes) only its own slot's energy
         if (t >= a.window_from && k.tid < 32 * A) {
           const long long e = sh.E[k.tid >> 5][k.tid & 31];
-          a.sum1[128 * (size_t)blockIdx.x + k.tid] += e;
-          a.sum2[128 * (size_t)blockIdx.x + k.tid] += e * e;
+          a.sum1[128 * prob + k.tid] += e;
+          a.sum2[128 * prob + k.tid] += e * e;
         }
         continue;
       }
       const long long done = (long long)a.sweep0 + (long long)(t + 1) * a.spp;
-      g_best<A>(k, sh, done);
+      g_best<A, AL>(k, sh, done, 0);
       if (A >= 2 && a.icm) {
+        if (CL) {
+          cg::this_cluster().sync();
+          const uint32_t *peer = cg::this_cluster().map_shared_rank(k.S, rank ^ 1);
+          for (int i = k.tid; i < k.n; i += kGThreads) k.S[2 * i + (rank ^ 1)] = peer[2 * i + (rank ^ 1)];
+          cg::this_cluster().sync();
+        }
         g_icm<A, SM>(k, sh, tt);
-        if (A == 2) {
+        if (CL) {
+          g_energy<A, NP, SM, AL>(k, sh);
+        } else if (A == 2) {
           // a cluster move keeps each pair's E_0 + E_1 and a whole-replica
           // flip keeps both (h = 0): recount label 0, label 1 follows
           int keep = 0;
@@ -810,36 +845,75 @@ __global__ void __launch_bounds__(kGThreads, 1) gapt_kernel(GAptArgs a, int init
         } else {
           g_energy<A, NP, SM>(k, sh);
         }
-        g_best<A>(k, sh, done);
+        g_best<A, AL>(k, sh, done, 1);
       }
-      g_swap<A>(k, sh, tt, a.joint, a.swaptab, swidx);
+      g_swap<A, AL>(k, sh, tt, a.joint, a.swaptab, swidx);
     }
     unsigned long long *st = a.stats + P.statbase;
     const int np = (P.T > 1 ? P.T - 1 : 0) * A;
     for (int i = k.tid; i < np; i += kGThreads) {
+      if (CL && i % A != rank) continue;   // the other CTA's label
       st[i] += sh.att[i];
       st[np + i] += sh.acc[i];
     }
-    if (k.tid == 0) {
+    bool mine = rank == 0;   // this CTA's best stands
+    if (CL) {
+      cg::this_cluster().sync();
+      const GShared *o = cg::this_cluster().map_shared_rank(&sh, rank ^ 1);
+      const long long oE = o->bestE, oS = o->bestSweep, oH = o->hit, oB = o->bestSlot;
+      const int oP = o->bestPhase, oF = o->fresh;
+      cg::this_cluster().sync();   // last access to the peer's memory
+      if (sh.fresh || oF) {
+        const long long dE = sh.bestE - oE, dS = sh.bestSweep - oS, dB = sh.bestSlot - oB;
+        const int dP = sh.bestPhase - oP;
+        mine = dE ? dE < 0 : dS ? dS < 0 : dP ? dP < 0 : dB < 0;
+      }
+      __syncthreads();
+      if (k.tid == 0) sh.hit = sh.hit < 0 ? oH : (oH < 0 ? sh.hit : min(sh.hit, oH));
+      if (mine && rank == 1)   // rank 1 found the best: it moves its state
+        for (int i = k.tid; i < (k.n + 31) / 32; i += kGThreads) a.best_bits[P.bestbase + i] = k.best_bits[i];
+    }
+    if (k.tid == 0 && rank == 0) {
       st[2 * np] += sh.icm[0];
       st[2 * np + 1] += sh.icm[1];
       st[2 * np + 2] += sh.icm[2];
-      long long *b = a.best + 4 * (size_t)blockIdx.x;
+    }
+    if (k.tid == 0 && mine) {
+      long long *b = a.best + 4 * prob;
       b[0] = sh.bestE;
       b[1] = sh.bestSweep;
       b[2] = sh.bestSlot;
       b[3] = sh.hit;
     }
   }
-  for (int i = k.tid; i < P.n * A; i += kGThreads) gS[i] = k.S[i];
-  if (k.tid < 128) a.E[128 * (size_t)blockIdx.x + k.tid] = sh.E[k.tid >> 5][k.tid & 31];
+  for (int i = k.tid; i < P.n * AL; i += kGThreads) {
+    const int w = CL ? 2 * i + rank : i;
+    gS[w] = k.S[w];
+  }
+  if (k.tid < 128 && (!CL || (k.tid >> 5) == rank)) a.E[128 * prob + k.tid] = sh.E[k.tid >> 5][k.tid & 31];
 }
 
-template <int A, int NP, bool SM>
+template <int A, int NP, bool SM, bool CL>
 int gapt_launch_t(const GAptArgs &a, int n_prob, size_t smem, bool init, cudaStream_t st) {
-  PC_CUDA_TRY(cudaFuncSetAttribute(gapt_kernel<A, NP, SM>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)smem));
-  gapt_kernel<A, NP, SM><<<n_prob, kGThreads, smem, st>>>(a, init ? 1 : 0);
+  auto kern = gapt_kernel<A, NP, SM, CL>;
+  PC_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  if (!CL) {
+    kern<<<n_prob, kGThreads, smem, st>>>(a, init ? 1 : 0);
+  } else {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(2 * n_prob));
+    cfg.blockDim = dim3((unsigned)kGThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, a, 0));
+  }
   PC_CUDA_TRY(cudaGetLastError());
   return PC_OK;
 }
@@ -1176,22 +1250,29 @@ size_t gapt_smem_bytes(int n, int A, int Imax, int m) {
   return sizeof(uint32_t) * (((base + 1) & ~(size_t)1) + 2 * (size_t)n + (size_t)m);
 }
 
-int gapt_launch(const GAptArgs &a, int n_prob, int A, int Imax, bool staged, size_t smem, bool init,
+int gapt_launch(const GAptArgs &a, int n_prob, int A, int Imax, bool staged, size_t smem, bool init, bool split,
                 cudaStream_t st) {
   const bool small = Imax <= 7;   // 3 planes hold every field count
+  if (split && A == 2) {
+    if (small)
+      return staged ? gapt_launch_t<2, 3, true, true>(a, n_prob, smem, init, st)
+                    : gapt_launch_t<2, 3, false, true>(a, n_prob, smem, init, st);
+    return staged ? gapt_launch_t<2, 7, true, true>(a, n_prob, smem, init, st)
+                  : gapt_launch_t<2, 7, false, true>(a, n_prob, smem, init, st);
+  }
   switch (A * 4 + (small ? 0 : 2) + (staged ? 1 : 0)) {
-    case 4: return gapt_launch_t<1, 3, false>(a, n_prob, smem, init, st);
-    case 5: return gapt_launch_t<1, 3, true>(a, n_prob, smem, init, st);
-    case 6: return gapt_launch_t<1, 7, false>(a, n_prob, smem, init, st);
-    case 7: return gapt_launch_t<1, 7, true>(a, n_prob, smem, init, st);
-    case 8: return gapt_launch_t<2, 3, false>(a, n_prob, smem, init, st);
-    case 9: return gapt_launch_t<2, 3, true>(a, n_prob, smem, init, st);
-    case 10: return gapt_launch_t<2, 7, false>(a, n_prob, smem, init, st);
-    case 11: return gapt_launch_t<2, 7, true>(a, n_prob, smem, init, st);
-    case 16: return gapt_launch_t<4, 3, false>(a, n_prob, smem, init, st);
-    case 17: return gapt_launch_t<4, 3, true>(a, n_prob, smem, init, st);
-    case 18: return gapt_launch_t<4, 7, false>(a, n_prob, smem, init, st);
-    case 19: return gapt_launch_t<4, 7, true>(a, n_prob, smem, init, st);
+    case 4: return gapt_launch_t<1, 3, false, false>(a, n_prob, smem, init, st);
+    case 5: return gapt_launch_t<1, 3, true, false>(a, n_prob, smem, init, st);
+    case 6: return gapt_launch_t<1, 7, false, false>(a, n_prob, smem, init, st);
+    case 7: return gapt_launch_t<1, 7, true, false>(a, n_prob, smem, init, st);
+    case 8: return gapt_launch_t<2, 3, false, false>(a, n_prob, smem, init, st);
+    case 9: return gapt_launch_t<2, 3, true, false>(a, n_prob, smem, init, st);
+    case 10: return gapt_launch_t<2, 7, false, false>(a, n_prob, smem, init, st);
+    case 11: return gapt_launch_t<2, 7, true, false>(a, n_prob, smem, init, st);
+    case 16: return gapt_launch_t<4, 3, false, false>(a, n_prob, smem, init, st);
+    case 17: return gapt_launch_t<4, 3, true, false>(a, n_prob, smem, init, st);
+    case 18: return gapt_launch_t<4, 7, false, false>(a, n_prob, smem, init, st);
+    case 19: return gapt_launch_t<4, 7, true, false>(a, n_prob, smem, init, st);
     default: return fail(PC_EINVAL, "n_labels must be 1, 2 or 4");
   }
 }

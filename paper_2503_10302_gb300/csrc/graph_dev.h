@@ -55,6 +55,7 @@ struct GAptArgs {
   uint32_t *spins;              // [n][A] words per problem
   int32_t *E;                   // [n_prob][4][32]
   uint32_t *best_bits;          // [ceil(n/32)] words per problem
+  uint32_t *best_bits2;         // rank 1's candidates of split problems, same layout
   long long *best;              // [n_prob][4]: E, sweep, slot, hit sweep
   const long long *target;      // [n_prob]
   unsigned long long *stats;    // counters per problem
@@ -89,7 +90,8 @@ struct GSqaArgs {
 // in shared memory as well (m adjacency entries).
 size_t gapt_smem_bytes(int n, int A, int Imax, int m);
 // Imax: the batch's largest field bound (selects the bit-plane count).
-int gapt_launch(const GAptArgs &a, int n_prob, int A, int Imax, bool staged, size_t smem, bool init,
+// split: two labels, a cluster of two CTAs per problem (one label each).
+int gapt_launch(const GAptArgs &a, int n_prob, int A, int Imax, bool staged, size_t smem, bool init, bool split,
                 cudaStream_t st);
 size_t gsqa_smem_bytes(int n, int P, int Imax, int m, int CS);
 // How an anneal of R runs is cut: clusters of CS CTAs per group of `runs` (32

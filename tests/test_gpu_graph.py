@@ -310,3 +310,34 @@ def test_gsqa_run_groups_and_clusters_fill_the_gpu(pc, orc, P, R):
     ctx.close()
     E2, s2 = orc.gsqa_anneal(g.rp, g.col, g.w, P, 0.2, gamma, R, run0=8, seed=17, want_spins=True)
     assert np.array_equal(s1, s2) and np.array_equal(E1, E2)
+
+
+@pytest.mark.parametrize("n_prob", [76, 77])
+def test_gapt_two_labels_on_one_or_two_ctas(pc, orc, n_prob):
+    """Two labels run as a cluster of two CTAs while twice the problems fit the
+    SMs, else as one CTA: states, best states, hits and statistics equal the
+    oracle either way, across launches and with a target."""
+    graphs = [W.random_graph(30 + i % 7, 3.0, i, wmax=2) for i in range(n_prob)]
+    trip = [(g.rp, g.col, g.w) for g in graphs]
+    betas = [W.geometric_ladder(5 + i % 3, 0.3, 2.0) for i in range(n_prob)]
+    ctx = pc.Context(0, 9)
+    pc.pc_gapt_load(ctx.h, trip, betas, 2, 3)
+    pc.pc_gapt_run(ctx.h, 7, 1, True)
+    pc.pc_gapt_run(ctx.h, 30, 1, True)
+    pc.pc_gapt_run(ctx.h, 5, 2, False)
+    ref = orc.GApt(trip, betas, n_labels=2, seed=9, entry0=3)
+    ref.run(7)
+    ref.run(30)
+    ref.run(5, 2, False)
+    for i in (0, 1, n_prob - 1):
+        T = len(betas[i])
+        s, e, _ = ref.state(i)
+        assert np.array_equal(pc.pc_gapt_get_spins(ctx.h, i, T, 2, graphs[i].n), s)
+        assert np.array_equal(pc.pc_gapt_get_energies(ctx.h, i, T, 2), e)
+        got, want = pc.pc_gapt_get_best(ctx.h, i, graphs[i].n), ref.best(i)
+        for key in ("E", "sweep", "buf", "hit_sweep"):
+            assert got[key] == want[key], (i, key)
+        assert np.array_equal(got["spins"], want["spins"])
+        for a, b in zip(pc.pc_gapt_get_stats(ctx.h, i, T, 2), ref.stats(i)):
+            assert np.array_equal(a, b)
+    ctx.close()
