@@ -23,18 +23,7 @@
 #include "device.cuh"
 #include "internal.h"
 
-// Build-time tuning knobs of the anneal kernel (defaults are the tuned
-// values): keep one site's constants in registers across sweeps, unroll the
-// loop over slice blocks, CTAs per SM the register budget is sized for.
-#ifndef PC_SQA_HOIST
-#define PC_SQA_HOIST 1
-#endif
-#ifndef PC_SQA_UNROLL
-#define PC_SQA_UNROLL 1
-#endif
-#ifndef PC_SQA_MINB
-#define PC_SQA_MINB 1
-#endif
+// Threads per CTA of the anneal kernel (build-time knob).
 #ifndef PC_SQA_TPB
 #define PC_SQA_TPB 512
 #endif
@@ -101,51 +90,87 @@ struct SiteK {
   int nb[6];
   int eps[6];        // +-1, 0 for an absent bond
   uint32_t K;
-  uint32_t kb;       // absent bonds k: 2k in every byte (threshold index I + 6 = 2C + k)
+  uint32_t kb;       // absent bonds k: 4k in every byte (threshold index I + 6 = 2C + k)
   int q;
 };
 
-__device__ __forceinline__ SiteK site_consts(const pc::SqaArgs &a, int s, const uint16_t *jn) {
+// The same in 20 bytes per site of shared memory, for lattices with more
+// sites than threads: v = the neighbours as 16-bit pairs and eps_0 .. eps_3
+// as bytes, u = eps_4, eps_5, #(J = -1) + 128 q, 4k.
+struct SitePack {
+  uint4 v;
+  uint32_t u;
+};
+
+__device__ __forceinline__ SitePack site_pack(const pc::SqaArgs &a, int s, const uint16_t *jn) {
   const Site t = site_of(a, s, jn);
-  SiteK k;
-  k.q = t.q;
-  int nneg = 0, nmiss = 0;
+  uint32_t nb[6], eps[6], nneg = 0, nmiss = 0;
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
-    k.nb[d] = neighbour(a, t, d);
-    const int neg = (t.jb >> d) & 1, miss = (t.jb >> (8 + d)) & 1;
-    k.eps[d] = miss ? 0 : 1 - 2 * neg;
-    nneg += miss ? 0 : neg;
+    nb[d] = (uint32_t)neighbour(a, t, d);
+    const uint32_t neg = (t.jb >> d) & 1u, miss = (t.jb >> (8 + d)) & 1u;
+    eps[d] = miss ? 0u : (neg ? 0xFFu : 1u);
+    nneg += miss ? 0u : neg;
     nmiss += miss;
   }
-  k.K = 0x11111111u * (uint32_t)nneg;
-  k.kb = 0x01010101u * (uint32_t)(2 * nmiss);
+  SitePack k;
+  k.v = make_uint4(nb[0] | (nb[1] << 16), nb[2] | (nb[3] << 16), nb[4] | (nb[5] << 16),
+                   eps[0] | (eps[1] << 8) | (eps[2] << 16) | (eps[3] << 24));
+  k.u = eps[4] | (eps[5] << 8) | ((nneg + 128u * (uint32_t)t.q) << 16) | (nmiss << 26);
   return k;
 }
 
-// Threshold tables in static shared memory, so that a byte of a packed
-// index word is directly an address offset: [2 sweeps][40 entries], entry
-// I + 6 + 13 m for in-slice field I = -6..6 and time count m = 0..2;
-// top halves (Th, 16-bit, 2-byte steps) and full values (Tf).
-__shared__ __align__(16) uint16_t s_Th[2][pc::kSqaTab];
-__shared__ __align__(16) uint32_t s_Tf[2][pc::kSqaTab];
+// Byte B of x as a signed value (prmt's sign mode spreads its top bit over
+// the upper bytes).
+template <int B>
+__device__ __forceinline__ int signed_byte(uint32_t x) {
+  uint32_t r;
+  asm("prmt.b32 %0, %1, 0, %2;" : "=r"(r) : "r"(x), "n"(0x8880 + 0x1111 * B));
+  return (int)r;
+}
+
+__device__ __forceinline__ SiteK site_unpack(const SitePack &p) {
+  SiteK k;
+  k.nb[0] = (int)(p.v.x & 0xFFFFu); k.nb[1] = (int)(p.v.x >> 16);
+  k.nb[2] = (int)(p.v.y & 0xFFFFu); k.nb[3] = (int)(p.v.y >> 16);
+  k.nb[4] = (int)(p.v.z & 0xFFFFu); k.nb[5] = (int)(p.v.z >> 16);
+  k.eps[0] = signed_byte<0>(p.v.w); k.eps[1] = signed_byte<1>(p.v.w);
+  k.eps[2] = signed_byte<2>(p.v.w); k.eps[3] = signed_byte<3>(p.v.w);
+  k.eps[4] = signed_byte<0>(p.u);   k.eps[5] = signed_byte<1>(p.u);
+  k.K = 0x11111111u * ((p.u >> 16) & 7u);
+  k.kb = __byte_perm(p.u, 0u, 0x3333u);
+  k.q = (int)((p.u >> 23) & 1u);
+  return k;
+}
+
+// Threshold rows of two sweeps (the current one and the next, which arrives
+// by asynchronous copy meanwhile), entry I + 6 + kRowStep m for in-slice field
+// I = -6..6 and time count m = 0..2: 23 words per step of m put the 21 entries
+// of a lattice without absent bonds (even I) into 21 banks.  Each row starts
+// on a 256-byte boundary of the shared window, so that a byte of a packed
+// offset word and the row's address make an entry's address in one byte
+// permute.  The copy replaces a load, a wait and two stores by two warps at
+// the start of each sweep (512 spins, 64 slices: 52.6 -> 51.9 ms with the
+// kernels by HOIST).
+constexpr uint32_t kRowStep = 23;
+__shared__ __align__(256) uint32_t s_Tf[2][64];
+
+__device__ __forceinline__ uint32_t entry_addr(uint32_t Dlo, uint32_t Dhi, uint32_t tb, int i) {
+  return __byte_perm((i & 1) ? Dhi : Dlo, tb, 0x7650u + (uint32_t)(i >> 1));
+}
 
 // Eq. neuron for the 8 nibbles of one word.  Byte k of Dlo / Dhi is the
-// byte offset of the threshold of nibble 2k / 2k+1 in s_Th (index * 2 plus
-// 80 for the odd sweep's buffer).  The main half v decides against the top
-// half t of the threshold: d = v - t is negative iff v < t, and d = 0 is a
-// tie, which the main half cannot decide.
-__device__ __forceinline__ uint32_t decide_word(const uint4 &x, uint32_t Dlo, uint32_t Dhi, bool &tie) {
+// byte offset of the threshold of nibble 2k / 2k+1 in the row at tb.  The
+// main half v decides against the top half t of the threshold: d = v - t is
+// negative iff v < t, and d = 0 is a tie, which the main half cannot decide.
+__device__ __forceinline__ uint32_t decide_word(const uint4 &x, uint32_t Dlo, uint32_t Dhi, uint32_t tb, bool &tie) {
   uint32_t w = 0;
   uint32_t tp = 1u;   // product of the differences (mod 2^32): 0 when some half equals its threshold
-  const char *base = reinterpret_cast<const char *>(&s_Th[0][0]);
 #pragma unroll
   for (int i = 7; i >= 0; --i) {
-    const uint32_t off = __byte_perm((i & 1) ? Dhi : Dlo, 0u, 0x4440u + (uint32_t)(i >> 1));
-    const uint32_t th = *reinterpret_cast<const uint16_t *>(base + off);
-    const uint32_t xw = word_of(x, i >> 1);
-    const uint32_t v = (i & 1) ? (xw >> 16) : (xw & 0xFFFFu);
-    const uint32_t d = v - th;   // both below 2^16: bit 31 set iff v < th
+    uint32_t th;
+    asm("ld.shared.u16 %0, [%1+2];" : "=r"(th) : "r"(entry_addr(Dlo, Dhi, tb, i)));
+    const uint32_t d = half_lo(x, i) - th;   // both below 2^16: bit 31 set iff v < th
     // the top 4 bits of d enter w as its new nibble 0, so after the loop
     // bit 3 of nibble i is the sign of half i's difference
     w = __funnelshift_l(d, w, 4);
@@ -157,12 +182,11 @@ __device__ __forceinline__ uint32_t decide_word(const uint4 &x, uint32_t Dlo, ui
   return (w >> 3) & 0x11111111u;
 }
 
-__device__ __noinline__ uint32_t settle_ties(uint32_t w, uint4 x, uint4 y, uint32_t Dlo, uint32_t Dhi) {
-  const char *base = reinterpret_cast<const char *>(&s_Tf[0][0]);
+__device__ __noinline__ uint32_t settle_ties(uint32_t w, uint4 x, uint4 y, uint32_t Dlo, uint32_t Dhi, uint32_t tb) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
-    const uint32_t off = __byte_perm((i & 1) ? Dhi : Dlo, 0u, 0x4440u + (uint32_t)(i >> 1));
-    const uint32_t t = *reinterpret_cast<const uint32_t *>(base + 2 * off);
+    uint32_t t;
+    asm("ld.shared.u32 %0, [%1];" : "=r"(t) : "r"(entry_addr(Dlo, Dhi, tb, i)));
     const uint32_t v = half_hi(x, i);
     if (v == (t & 0xFFFF0000u)) {
       const uint32_t u = v | half_lo(y, i);
@@ -171,6 +195,16 @@ __device__ __noinline__ uint32_t settle_ties(uint32_t w, uint4 x, uint4 y, uint3
   }
   return w;
 }
+
+// Starts the asynchronous copy of a threshold row into shared memory.
+__device__ __forceinline__ void fetch_row(const uint32_t *row, uint32_t *dst) {
+  for (uint32_t e = threadIdx.x; e < 39u; e += blockDim.x) {   // small runs have fewer threads than entries
+    const uint32_t d = e + (kRowStep - 13u) * ((e >= 13u ? 1u : 0u) + (e >= 26u ? 1u : 0u));
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst + d)),
+                 "l"(row + e) : "memory");
+  }
+}
+__device__ __forceinline__ void rows_landed() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // NB consecutive words as one vector access (NB = 1, 2, 4, 8; else scalar).
 template <int NB>
@@ -207,66 +241,78 @@ __device__ __forceinline__ void store_words(uint32_t *p, const uint32_t (&v)[NB]
   }
 }
 
-// All NB words of one (site, colour) in one sweep.
-template <int NB>
-__device__ __forceinline__ void update_site(const pc::SqaArgs &a, const uint32_t *Wo, uint32_t *Wc,
-                                            int s, const SiteK &k, int c, uint32_t sw,
-                                            uint32_t boff, uint32_t ent) {
+// Words b0 .. b0 + WT - 1 of one (site, colour) in one sweep.
+template <int NB, int WT>
+__device__ __forceinline__ void update_site(const pc::SqaArgs &a, const uint32_t *Wo, uint32_t *Wc, int s, int b0,
+                                            const SiteK &k, int c, uint32_t sw, uint32_t tb, uint32_t ent) {
   const int e = c ^ k.q;   // slice parity of this word's nibbles
-  const uint32_t c2 = (uint32_t)c << 16;
-  uint32_t O[NB], C[NB], w[NB];
-  load_words<NB>(Wo + (size_t)s * NB, O);
+  const uint32_t c2 = ((uint32_t)c << 16) | (uint32_t)b0;
+  uint32_t O[WT], C[WT], w[WT];
+  load_words<WT>(Wo + s * NB + b0, O);
+  // time neighbours k-1, k+1 of word b: the other colour's word and that
+  // word shifted by one nibble (funnel shift through the adjacent block, of
+  // which the parity needs the next (e = 1) or the previous one)
+  uint32_t M[WT];
+  {
+    const int bx = e ? (b0 + WT == NB ? 0 : b0 + WT) : (b0 == 0 ? NB - 1 : b0 - 1);
+    const uint32_t X = WT == NB ? (e ? O[0] : O[WT - 1]) : Wo[s * NB + bx];
+    uint32_t lo = e ? O[0] : X;
+    const uint32_t sh = e ? 4u : 28u;
 #pragma unroll
-  for (int b = 0; b < NB; ++b) C[b] = k.K;
+    for (int i = 0; i < WT; ++i) {
+      const uint32_t hi = e ? (i + 1 == WT ? X : O[i + 1 == WT ? i : i + 1]) : O[i];
+      M[i] = O[i] + __funnelshift_r(lo, hi, sh);
+      lo = hi;
+    }
+  }
+#pragma unroll
+  for (int b = 0; b < WT; ++b) C[b] = k.K;
 #pragma unroll
   for (int d = 0; d < 6; ++d) {
-    uint32_t Nw[NB];
-    load_words<NB>(Wo + (size_t)k.nb[d] * NB, Nw);
+    uint32_t Nw[WT];
+    load_words<WT>(Wo + k.nb[d] * NB + b0, Nw);
 #pragma unroll
-    for (int b = 0; b < NB; ++b) C[b] += (uint32_t)k.eps[d] * Nw[b];
+    for (int b = 0; b < WT; ++b) C[b] += (uint32_t)k.eps[d] * Nw[b];
   }
-  // time neighbours k-1, k+1 of word b: the other colour's word and that
-  // word shifted by one nibble (funnel shift through the adjacent block);
-  // byte offsets 2 (2C + k + 13 m) + 80 (odd sweep): at most 156
-  const uint32_t kb = k.kb + boff;
+  // byte offsets 4 (2C + k + 23 m): at most 232
   auto offsets = [&](int b, uint32_t &Dlo, uint32_t &Dhi) {
-    const int bp = (b + 1 == NB) ? 0 : b + 1, bm = (b == 0) ? NB - 1 : b - 1;
-    const uint32_t lo = e ? O[b] : O[bm];
-    const uint32_t hi = e ? O[bp] : O[b];
-    const uint32_t M = O[b] + __funnelshift_r(lo, hi, e ? 4u : 28u);
-    Dlo = ((C[b] & 0x0F0F0F0Fu) << 2) + (M & 0x0F0F0F0Fu) * 26u + kb;
-    Dhi = (((C[b] >> 4) & 0x0F0F0F0Fu) << 2) + ((M >> 4) & 0x0F0F0F0Fu) * 26u + kb;
+    const uint32_t m = M[b];
+    Dlo = ((C[b] & 0x0F0F0F0Fu) << 3) + (m & 0x0F0F0F0Fu) * (4u * kRowStep) + k.kb;
+    Dhi = (((C[b] >> 4) & 0x0F0F0F0Fu) << 3) + ((m >> 4) & 0x0F0F0F0Fu) * (4u * kRowStep) + k.kb;
+  };
+  const uint32_t c3 = (ent << 8) | TAG_SQA_SWEEP;
+  auto settle = [&](int b, uint32_t Dlo, uint32_t Dhi) {
+    const uint4 x = philox((uint32_t)s, sw, c2 + (uint32_t)b, c3, a.k0, a.k1);
+    const uint4 y = philox((uint32_t)s, sw, c2 + (uint32_t)b, (ent << 8) | TAG_SQA_REFINE, a.k0, a.k1);
+    w[b] = settle_ties(w[b], x, y, Dlo, Dhi, tb);
   };
   // up to 4 words, the decisions form one branch-free block and ties
   // (probability 2^-16 per spin) are settled after it; with more words the
   // register budget settles each word's ties at once
   uint32_t tmask = 0u;
 #pragma unroll
-  for (int b = 0; b < NB; ++b) {
+  for (int b = 0; b < WT; ++b) {
     uint32_t Dlo, Dhi;
     offsets(b, Dlo, Dhi);
-    const uint4 x = philox((uint32_t)s, sw, c2 | (uint32_t)b, (ent << 8) | TAG_SQA_SWEEP, a.k0, a.k1);
+    const uint4 x = philox((uint32_t)s, sw, c2 + (uint32_t)b, c3, a.k0, a.k1);
     bool tie = false;
-    w[b] = decide_word(x, Dlo, Dhi, tie);
-    if constexpr (NB <= 4) {
+    w[b] = decide_word(x, Dlo, Dhi, tb, tie);
+    if constexpr (WT <= 4) {
       tmask |= tie ? (1u << b) : 0u;
     } else if (tie) {
-      const uint4 y = philox((uint32_t)s, sw, c2 | (uint32_t)b, (ent << 8) | TAG_SQA_REFINE, a.k0, a.k1);
-      w[b] = settle_ties(w[b], x, y, Dlo, Dhi);
+      settle(b, Dlo, Dhi);
     }
   }
-  if (NB <= 4 && tmask) {
+  if (WT <= 4 && tmask) {
 #pragma unroll
-    for (int b = 0; b < NB; ++b) {
+    for (int b = 0; b < WT; ++b) {
       if (!((tmask >> b) & 1u)) continue;
       uint32_t Dlo, Dhi;
       offsets(b, Dlo, Dhi);
-      const uint4 x = philox((uint32_t)s, sw, c2 | (uint32_t)b, (ent << 8) | TAG_SQA_SWEEP, a.k0, a.k1);
-      const uint4 y = philox((uint32_t)s, sw, c2 | (uint32_t)b, (ent << 8) | TAG_SQA_REFINE, a.k0, a.k1);
-      w[b] = settle_ties(w[b], x, y, Dlo, Dhi);
+      settle(b, Dlo, Dhi);
     }
   }
-  store_words<NB>(Wc + (size_t)s * NB, w);
+  store_words<WT>(Wc + s * NB + b0, w);
 }
 
 __device__ __forceinline__ uint64_t global_ns() {
@@ -290,10 +336,11 @@ __device__ __forceinline__ bool wait_at_least(const int *flag, int want, uint64_
 // Anneal of sweeps [s0, s1) of one run.  s0 == 0 draws the random initial
 // state, otherwise the state comes from the run's slot in global memory;
 // s1 == S computes the final slice energies, otherwise the state goes back.
-template <int NB>
+template <int NB, int WT, bool HOIST>
 __device__ __forceinline__ void anneal_span(const pc::SqaArgs &a, uint32_t *W, int32_t *Eacc,
-                                            const uint16_t *jn, const SiteK &kh, bool hoist,
+                                            const uint16_t *jn, const uint4 *sv, const uint32_t *su, const SiteK &kh,
                                             int run, int s0, int s1) {
+  constexpr int parts = NB / WT;   // threads per site
   const int N = a.N, P = a.P;
   const uint32_t ent = a.run0 + (uint32_t)run;
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -312,35 +359,29 @@ __device__ __forceinline__ void anneal_span(const pc::SqaArgs &a, uint32_t *W, i
   } else {
     for (int idx = tid; idx < 2 * NB * N; idx += nt) W[idx] = __ldcg(gstate + idx);
   }
-  for (int e = tid; e < pc::kSqaTab; e += nt) {   // small runs have fewer threads than entries
-    const uint32_t t = s0 < a.S ? a.table[(size_t)s0 * pc::kSqaTab + e] : 0u;
-    s_Tf[s0 & 1][e] = t;
-    s_Th[s0 & 1][e] = (uint16_t)(t >> 16);
-  }
+  if (s0 < a.S) fetch_row(a.table + (size_t)s0 * pc::kSqaTab, s_Tf[s0 & 1]);
+  rows_landed();
+  const int sh = tid / parts, bh = (tid - sh * parts) * WT;   // the thread's site and first word, one item per thread
   __syncthreads();
 
   for (int sw = s0; sw < s1; ++sw) {
-    // the transverse coupling of this sweep lives in its threshold table;
-    // prefetch the next sweep's table into the other buffer
-    if (sw + 1 < a.S)
-      for (int e = tid; e < pc::kSqaTab; e += nt) {
-        const uint32_t t = a.table[(size_t)(sw + 1) * pc::kSqaTab + e];
-        s_Tf[(sw + 1) & 1][e] = t;
-        s_Th[(sw + 1) & 1][e] = (uint16_t)(t >> 16);
-      }
-    const uint32_t boff = (sw & 1) ? 0x50505050u : 0u;   // 80 bytes: the odd sweep's table
+    // the transverse coupling of this sweep lives in its threshold row; the
+    // next sweep's row lands in the other buffer meanwhile
+    if (sw + 1 < a.S) fetch_row(a.table + (size_t)(sw + 1) * pc::kSqaTab, s_Tf[(sw + 1) & 1]);
+    const uint32_t tb = (uint32_t)__cvta_generic_to_shared(s_Tf[sw & 1]);
 #pragma unroll 1
     for (int c = 0; c < 2; ++c) {
       const uint32_t *Wo = W + (1 - c) * NB * N;
       uint32_t *Wc = W + c * NB * N;
-      if (hoist) {
-        if (tid < N) update_site<NB>(a, Wo, Wc, tid, kh, c, (uint32_t)sw, boff, ent);
+      if constexpr (HOIST) {
+        if (sh < N) update_site<NB, WT>(a, Wo, Wc, sh, bh, kh, c, (uint32_t)sw, tb, ent);
       } else {
-        for (int s = tid; s < N; s += nt) {
-          const SiteK k = site_consts(a, s, jn);
-          update_site<NB>(a, Wo, Wc, s, k, c, (uint32_t)sw, boff, ent);
+        for (int it = tid; it < N * parts; it += nt) {
+          const int s = it / parts, b0 = (it - s * parts) * WT;
+          update_site<NB, WT>(a, Wo, Wc, s, b0, site_unpack(SitePack{sv[s], su[s]}), c, (uint32_t)sw, tb, ent);
         }
       }
+      if (c) rows_landed();
       __syncthreads();
     }
   }
@@ -434,23 +475,31 @@ __device__ __forceinline__ void anneal_span(const pc::SqaArgs &a, uint32_t *W, i
 // queue; chunk k of a run waits (bounded) until chunk k-1 of that run has
 // stored its state.  Time-slicing the runs keeps every SM busy when the
 // number of runs is not a multiple of the number of SMs.
-template <int NB, bool PERSIST>
-__global__ void __launch_bounds__(PC_SQA_TPB, PC_SQA_MINB) sqa_kernel(const pc::SqaArgs a) {
+template <int NB, int WT, bool HOIST, bool PERSIST>
+__global__ void __launch_bounds__(PC_SQA_TPB, 1) sqa_kernel(const pc::SqaArgs a) {
   extern __shared__ __align__(16) uint32_t smem[];
   __shared__ int s_item;
   const int N = a.N, P = a.P;
   uint32_t *W = smem;                                       // [2][NB][N]
-  int32_t *Eacc = reinterpret_cast<int32_t *>(W + 2 * NB * N);   // [P]
-  uint16_t *jn = reinterpret_cast<uint16_t *>(Eacc + P);    // [N]
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int i = tid; i < N; i += nt) jn[i] = a.jneg[i];
+  const int np = HOIST ? 0 : N;
+  uint4 *sv = reinterpret_cast<uint4 *>(W + 2 * NB * N);    // [np] SitePack::v (2 NB N words: a multiple of 4)
+  uint32_t *su = reinterpret_cast<uint32_t *>(sv + np);     // [np] SitePack::u
+  int32_t *Eacc = reinterpret_cast<int32_t *>(su + np);     // [P]
+  uint16_t *jn = reinterpret_cast<uint16_t *>(Eacc + P);    // [N]
+  for (int i = tid; i < N; i += nt) {
+    jn[i] = a.jneg[i];
+    if constexpr (!HOIST) {
+      const SitePack k = site_pack(a, i, jn);
+      sv[i] = k.v;
+      su[i] = k.u;
+    }
+  }
   __syncthreads();
-  // one site per thread (N <= blockDim): its constants stay in registers
-  const bool hoist = PC_SQA_HOIST && N <= nt;
   SiteK kh;
-  if (hoist && tid < N) kh = site_consts(a, tid, jn);
+  if (HOIST && tid / (NB / WT) < N) kh = site_unpack(site_pack(a, tid / (NB / WT), jn));
   if constexpr (!PERSIST) {
-    anneal_span<NB>(a, W, Eacc, jn, kh, hoist, blockIdx.x, 0, a.S);
+    anneal_span<NB, WT, HOIST>(a, W, Eacc, jn, sv, su, kh, blockIdx.x, 0, a.S);
   } else {
     for (;;) {
       if (tid == 0) s_item = atomicAdd(a.queue, 1) + a.first_item;
@@ -464,7 +513,7 @@ __global__ void __launch_bounds__(PC_SQA_TPB, PC_SQA_MINB) sqa_kernel(const pc::
         if (tid == 0 && !wait_at_least(a.done + run, chunk, a.wait_ns)) atomicExch(a.err, 1);
         __syncthreads();
       }
-      anneal_span<NB>(a, W, Eacc, jn, kh, hoist, run, s0, s1);
+      anneal_span<NB, WT, HOIST>(a, W, Eacc, jn, sv, su, kh, run, s0, s1);
       __syncthreads();
       if (tid == 0) {
         __threadfence();
@@ -485,29 +534,51 @@ __global__ void philox_kernel(const uint32_t *ctr, uint32_t *out, int64_t n, uin
   out[4 * i + 3] = x.w;
 }
 
-template <int NB>
-int launch_nb(const pc::SqaArgs &a, int R, cudaStream_t st) {
-  const size_t smem = pc::sqa_smem_bytes(a.N, a.P);
-  int tpb = ((a.N + 31) / 32) * 32;
-  if (tpb > PC_SQA_TPB) tpb = PC_SQA_TPB;
+// Words of a site that a thread updates: all of them up to 5 (and 7), else a
+// half, which fits the registers as one block of decisions (128 slices, 512
+// spins, 128 runs, 1000 sweeps: 8 words per thread 7.19 ms, 4 6.41 ms, 2
+// 7.15 ms; 96 slices, 630 spins open: 6 words 3.67 ms, 3 3.44 ms, 2 3.52 ms).
+// Twice the threads with half the words and registers (1024 x 64) ran slower
+// everywhere (64 slices, 512 spins: 64.3 against 52.6 ms).
+constexpr int words_per_thread(int NB) { return NB == 8 ? 4 : NB == 6 ? 3 : NB; }
+
+template <int NB, bool HOIST>
+int launch_h(const pc::SqaArgs &a, int R, int tpb, cudaStream_t st) {
+  constexpr int WT = words_per_thread(NB);
+  // the packed site constants only where a thread has more than one item
+  const size_t smem = pc::sqa_smem_bytes(a.N, a.P) - (HOIST ? 20 * (size_t)a.N : 0);
   if (!a.state) {
-    PC_CUDA_TRY(cudaFuncSetAttribute(sqa_kernel<NB, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PC_CUDA_TRY(cudaFuncSetAttribute(sqa_kernel<NB, WT, HOIST, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
-    sqa_kernel<NB, false><<<R, tpb, smem, st>>>(a);
+    sqa_kernel<NB, WT, HOIST, false><<<R, tpb, smem, st>>>(a);
   } else {
-    PC_CUDA_TRY(cudaFuncSetAttribute(sqa_kernel<NB, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    PC_CUDA_TRY(cudaFuncSetAttribute(sqa_kernel<NB, WT, HOIST, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      (int)smem));
     int dev = 0, sms = 0, per_sm = 0;
     PC_CUDA_TRY(cudaGetDevice(&dev));
     PC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sqa_kernel<NB, true>, tpb, smem));
+    PC_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sqa_kernel<NB, WT, HOIST, true>, tpb, smem));
     if (per_sm < 1) per_sm = 1;
     int grid = sms * per_sm;
     if (grid > a.n_items) grid = a.n_items;
-    sqa_kernel<NB, true><<<grid, tpb, smem, st>>>(a);
+    sqa_kernel<NB, WT, HOIST, true><<<grid, tpb, smem, st>>>(a);
   }
   PC_CUDA_TRY(cudaGetLastError());
   return PC_OK;
+}
+
+// HOIST: one item (a thread's words of one site) per thread, whose constants
+// stay in registers across the sweeps; else the threads loop over the items
+// and unpack the constants from shared memory (about 20 instructions; computed
+// anew from the site's coordinates they were about 60 per site and colour, and
+// with one kernel for both forms the registers were allotted for both).  64
+// slices: 15 x 15 x 12 open, 132 runs, 1000 sweeps 19.8 -> 17.0 ms, 12^3 6.57
+// -> 5.19 ms and 16^3 8.45 -> 4.57 ms (64 and 16 runs, 500 and 200 sweeps).
+template <int NB>
+int launch_nb(const pc::SqaArgs &a, int R, cudaStream_t st) {
+  const int items = a.N * (NB / words_per_thread(NB));
+  if (items <= PC_SQA_TPB) return launch_h<NB, true>(a, R, ((items + 31) / 32) * 32, st);
+  return launch_h<NB, false>(a, R, PC_SQA_TPB, st);
 }
 
 }  // namespace
@@ -516,7 +587,7 @@ namespace pc {
 
 size_t sqa_smem_bytes(int N, int P) {
   const int NB = P / 16;
-  return (size_t)2 * NB * N * 4 + (size_t)P * 4 + (size_t)N * 2;
+  return (size_t)2 * NB * N * 4 + (size_t)P * 4 + (size_t)N * 2 + (size_t)N * 20;
 }
 
 int sqa_launch(const SqaArgs &a, int R, cudaStream_t st) {

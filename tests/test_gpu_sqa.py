@@ -231,3 +231,33 @@ def test_sqa_schedule_follows_the_number_of_runs(pc, orc, P, R, S, spins):
         assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1])
     else:
         assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("dims,per,P", [
+    ((8, 8, 8), (1, 1, 1), 64),      # 512 items: one per thread
+    ((8, 8, 10), (1, 1, 1), 64),     # 640: the threads loop
+    ((9, 7, 10), (0, 0, 1), 64),     # the same with absent bonds and vacancies
+    ((8, 8, 4), (1, 1, 1), 128),     # two items per site, 512
+    ((12, 6, 4), (0, 0, 1), 128),    # 576, the last round of threads partly idle
+    ((8, 8, 4), (1, 1, 1), 96),      # three words per item
+    ((8, 6, 6), (0, 0, 1), 96),
+    ((8, 8, 10), (1, 1, 1), 80),     # five and seven words of a site in one thread
+    ((8, 8, 10), (0, 0, 1), 112),
+    ((2, 2, 2), (1, 1, 1), 16),      # one warp for a threshold row of 39 entries
+])
+def test_sqa_items_per_thread(pc, orc, dims, per, P):
+    """Anneals with one item per thread keep its site's constants in registers,
+    larger ones unpack them from shared memory: both equal the oracle bit for
+    bit."""
+    J, present, seed, R = W.ea_couplings(dims, 1000, 31), None, 31, 2
+    if per != (1, 1, 1):
+        dims, present, J = W.pad_odd_open(dims, per, J)
+        dims = tuple(int(v) for v in dims)
+    gamma = W.linear_gamma_schedule(12)
+    ctx = pc.Context(0, seed)
+    pc.pc_sqa_setup_bc(ctx.h, dims, per, J, P, 0.05, gamma, present)
+    E, s = pc.pc_sqa_run(ctx.h, R, 3, P, int(np.prod(dims)), want_spins=True)
+    ctx.close()
+    E2, s2 = orc.sqa_anneal(dims, J, P, 0.05, gamma, R, run0=3, seed=seed, want_spins=True, periodic=per,
+                            present=present)
+    assert np.array_equal(E, E2) and np.array_equal(s, s2)
