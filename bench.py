@@ -52,7 +52,7 @@ L, P, R, T, SWEEPS = 8, 64, 256, 0.05, 10000
 ALG_OPS_PER_FLIP = 20.0
 # The same count for this implementation's packing (one Philox call feeds 8
 # spins through 16-bit halves, one word holds 8 spins' fields): 5 + 2 + 6.5
-# + 0.5 = 14; an ncu capture of the anneal kernel counts 15.5 executed
+# + 0.5 = 14; an ncu capture of the anneal kernel before its last change counts 15.5 executed
 # thread instructions per update.  Reported beside the roofline, not in it.
 PACKED_OPS_PER_FLIP = 14.0
 NCU_INSTR_PER_FLIP = 15.5
