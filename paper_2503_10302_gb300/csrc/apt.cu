@@ -1522,7 +1522,12 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     if (MODE == pc::APT_MODE_PILOT)
       for (int i = threadIdx.x; i < k.T * a.n_bins; i += blockDim.x) smem[k.oHist + i] = 0u;
   }
-  __syncthreads();
+  // a split problem's first swap step writes the peer's exchange words and
+  // stage: only once the peer runs and has set them up
+  if (SPLIT && MODE == pc::APT_MODE_APT)
+    cooperative_groups::this_cluster().sync();
+  else
+    __syncthreads();
 
   if (MODE == pc::APT_MODE_ENERGY) {
     colour_phase<false, true>(1, 0u);

@@ -656,3 +656,26 @@ def test_features_and_resampling_match_oracle(pc):
     for ln in (1, 2, 20, 33, 34):
         beta = np.sort(np.random.default_rng(ln).random(ln)) + 0.5
         assert np.array_equal(pc.pc_resample_ladder(beta, 32), mlp.resample_ladder(beta, 32))
+
+
+@pytest.mark.parametrize("groups", [1, 3])
+def test_first_swap_step_of_small_split_problems(pc, orc, groups):
+    """Split problems of a few sites and uneven halves (one CTA loads three
+    times the other's groups, and its first sweep is over soonest): many
+    launches of one attempt, each of which begins with the exchange across the
+    two CTAs, equal the oracle's chains."""
+    shapes = [(2, 2, 2), (4, 2, 2), (4, 4, 4)]
+    dims = np.array(shapes, np.int32)
+    J = [W.ea_couplings(s, 19, i) for i, s in enumerate(shapes)]
+    betas = [W.geometric_ladder(32), W.geometric_ladder(31), W.geometric_ladder(25)]
+    b = W.AptBatch(dims, J, betas, 2)
+    ctx = pc.Context(0, 61)
+    pc.pc_apt_load(ctx.h, dims, J, betas, 2, 0)
+    pc.pc_apt_set_launch(ctx.h, 512, 0, 2, groups)
+    assert pc.pc_apt_is_split(ctx.h) == 1
+    apt = orc.Apt(dims, J, betas, 2, seed=61)
+    for _ in range(40):
+        pc.pc_apt_run(ctx.h, 1, 1, True)
+    apt.run(40, 1, True)
+    _compare(pc, apt, ctx, b)
+    ctx.close()
