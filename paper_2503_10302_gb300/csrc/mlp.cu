@@ -11,6 +11,7 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -57,7 +58,7 @@ struct Products {
   Product p[2];
   int loss_n;              // samples of the loss sum (0: none)
   const float *loss_s;
-  float *loss, *loss2;     // loss2: a second destination or NULL
+  float *loss;
 };
 
 // A 32 x 32 tile per block of 128 threads, 2 x 4 outputs per thread, K in
@@ -70,7 +71,7 @@ struct Products {
 // in order.
 constexpr int kTile = 32, kGemmThreads = 128;
 
-__device__ __forceinline__ void loss_sum(int B, const float *loss_s, float *loss, float *loss2, float *part) {
+__device__ __forceinline__ void loss_sum(int B, const float *loss_s, float *loss, float *part) {
   // 256 partial sums in fixed order, two per thread
   for (int t = threadIdx.x; t < 256; t += kGemmThreads) {
     float s = 0.f;
@@ -82,11 +83,7 @@ __device__ __forceinline__ void loss_sum(int B, const float *loss_s, float *loss
     if ((int)threadIdx.x < w) part[threadIdx.x] += part[threadIdx.x + w];
     __syncthreads();
   }
-  if (threadIdx.x == 0) {
-    const float l = part[0] / (float)(B * kOut);
-    *loss = l;
-    if (loss2) *loss2 = l;
-  }
+  if (threadIdx.x == 0) *loss = part[0] / (float)(B * kOut);
 }
 
 __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(const __grid_constant__ Products P) {
@@ -96,7 +93,7 @@ __global__ void __launch_bounds__(kGemmThreads) gemm_kernel(const __grid_constan
   int tile = (int)blockIdx.x;
   if (P.loss_n) {
     if (tile == 0) {
-      loss_sum(P.loss_n, P.loss_s, P.loss, P.loss2, &As[0][0]);
+      loss_sum(P.loss_n, P.loss_s, P.loss, &As[0][0]);
       return;
     }
     --tile;
@@ -225,11 +222,15 @@ __global__ void head_kernel(int B, const float *O, const float *Y, float beta_mi
 
 // Adam (Kingma & Ba): m = b1 m + (1-b1) g; v = b2 v + (1-b2) g^2;
 // p -= lr * (m / c1) / (sqrt(v / c2) + eps) with c1 = 1 - b1^t, c2 = 1 - b2^t.
+// The pass's last kernel also hands out the loss (loss_out may be NULL): all
+// reads of the minibatch are done by then, so the caller may have the loss in
+// the minibatch's own memory.
 __global__ void adam_kernel(int n, float *p, const float *g, float *m, float *v, float lr, float b1,
-                            float b2, float c1, float c2, float eps) {
+                            float b2, float c1, float c2, float eps, const float *loss, float *loss_out) {
   let_next();
   wait_previous();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0 && loss_out) *loss_out = *loss;
   if (i >= n) return;
   const float gi = g[i];
   const float mi = b1 * m[i] + (1.f - b1) * gi;
@@ -333,9 +334,8 @@ int forward(pc_mlp *mm, int batch, const float *X, float *beta_dev) {
   return PC_OK;
 }
 
-// Loss (also to loss2_dev, if given) and gradients into mm->grads for X, Y
-// on the device.
-int backward(pc_mlp *mm, int batch, const float *X, const float *Y, float *loss2_dev = nullptr) {
+// Loss and gradients into mm->loss and mm->grads for X, Y on the device.
+int backward(pc_mlp *mm, int batch, const float *X, const float *Y) {
   cudaStream_t st = mm->ctx->stream;
   int rc = forward(mm, batch, X, nullptr);
   if (rc) return rc;
@@ -360,7 +360,6 @@ int backward(pc_mlp *mm, int batch, const float *X, const float *Y, float *loss2
       P.loss_n = batch;
       P.loss_s = mm->loss_s.p;
       P.loss = mm->loss.p;
-      P.loss2 = loss2_dev;
     }
     if ((rc = gemm(st, P))) return rc;
     if (l > 0) dZ = mm->dH[l - 1].p;
@@ -368,14 +367,27 @@ int backward(pc_mlp *mm, int batch, const float *X, const float *Y, float *loss2
   return PC_OK;
 }
 
-int adam(pc_mlp *mm, float lr) {
+// loss_out: where the kernel stores the loss as well, or NULL.
+int adam(pc_mlp *mm, float lr, float *loss_out = nullptr) {
   mm->t += 1;
   const float b1 = 0.9f, b2 = 0.999f, eps = 1e-8f;
   const float c1 = (float)(1.0 - std::pow(0.9, (double)mm->t));
   const float c2 = (float)(1.0 - std::pow(0.999, (double)mm->t));
   const int n = (int)mm->n_params;
   return launch_next(adam_kernel, (n + 255) / 256, 256, mm->ctx->stream, n, mm->params.p, mm->grads.p, mm->m.p,
-                     mm->v.p, lr, b1, b2, c1, c2, eps);
+                     mm->v.p, lr, b1, b2, c1, c2, eps, mm->loss.p, loss_out);
+}
+
+// Whether a kernel on `device` may store a float at p: aligned memory of that
+// device.  Anything else a copy can reach (another device, a byte offset).
+bool stores_directly(const float *p, int device) {
+  cudaPointerAttributes at = {};
+  if (reinterpret_cast<uintptr_t>(p) % sizeof(float)) return false;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == device;
 }
 
 }  // namespace
@@ -509,8 +521,13 @@ int pc_mlp_train_step_dev(pc_mlp *mm, int batch, const float *X_dev, const float
   PC_CUDA_TRY(cudaSetDevice(mm->ctx->device));
   int rc = ensure_batch(mm, batch);
   if (rc) return rc;
-  if ((rc = backward(mm, batch, X_dev, Y_dev, loss_dev))) return rc;
-  return adam(mm, lr);
+  if ((rc = backward(mm, batch, X_dev, Y_dev))) return rc;
+  // a copy is a node of its own between two kernels: the update stores the
+  // loss itself where it can
+  const bool direct = loss_dev && stores_directly(loss_dev, mm->device);
+  if (loss_dev && !direct)
+    PC_CUDA_TRY(cudaMemcpyAsync(loss_dev, mm->loss.p, 4, cudaMemcpyDeviceToDevice, mm->ctx->stream));
+  return adam(mm, lr, direct ? loss_dev : nullptr);
 } catch (...) {
   return pc::fail_exception();
 }

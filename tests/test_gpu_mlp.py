@@ -162,3 +162,56 @@ def test_training_reduces_loss(pc):
     assert losses[-1] < 0.05 * losses[0]
     m.close()
     ctx.close()
+
+
+def _dev_steps(pc, X, Y, loss_of, steps=2, capture=False):
+    """Parameters and losses of training steps on device buffers; loss_of(x)
+    gives each step's loss address from the minibatch's.  capture: the last
+    step runs as a captured graph."""
+    import torch
+    params = W.mlp_init(pc.MLP_SIZES, 8)
+    stream = torch.cuda.Stream()
+    ctx = pc.Context(0, 0)
+    pc.pc_set_stream(ctx.h, stream.cuda_stream)
+    m = pc.Mlp(ctx, params)
+    m.set_gap_weight(0.05)
+    out = torch.zeros(16, dtype=torch.uint8, device="cuda")
+    losses = []
+    for i in range(steps):
+        x, y = torch.from_numpy(X).cuda(), torch.from_numpy(Y).cuda()
+        torch.cuda.synchronize()
+        at = loss_of(x.data_ptr(), out.data_ptr())
+        if capture and i == steps - 1:
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=stream):
+                m.train_step_dev(len(X), x.data_ptr(), y.data_ptr(), 1e-3, at)
+            g.replay()
+        else:
+            m.train_step_dev(len(X), x.data_ptr(), y.data_ptr(), 1e-3, at)
+        torch.cuda.synchronize()
+        buf = out if 0 <= at - out.data_ptr() < 16 else x.flatten().view(torch.uint8)
+        off = at - buf.data_ptr()
+        losses.append(buf[off:off + 4].cpu().numpy().tobytes())
+    p = [v.tobytes() for layer in m.params() for v in layer]
+    m.close()
+    ctx.close()
+    return losses, p
+
+
+@pytest.mark.parametrize("where", ["in the minibatch", "at a byte offset"])
+def test_loss_may_go_anywhere_a_copy_reaches(pc, where):
+    """The loss of a device training step is stored after the minibatch's last
+    use, so its address may lie in the minibatch; an address that is no
+    multiple of 4 is reached by a copy.  Updates and losses are the same bytes
+    as with a buffer of its own."""
+    X, Y = _data(96, 9)
+    want = _dev_steps(pc, X, Y, lambda x, out: out)
+    got = _dev_steps(pc, X, Y, (lambda x, out: x + 4) if where == "in the minibatch" else (lambda x, out: out + 5))
+    assert got == want
+
+
+def test_captured_step_equals_plain_step(pc):
+    """Under stream capture the pass's kernels keep plain edges: the replayed
+    step gives the same bytes."""
+    X, Y = _data(200, 10)
+    assert _dev_steps(pc, X, Y, lambda x, out: out, capture=True) == _dev_steps(pc, X, Y, lambda x, out: out)
