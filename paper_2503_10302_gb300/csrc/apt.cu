@@ -128,8 +128,9 @@ struct __align__(16) Ctl {
   uint32_t open;     // bit a: axis a open; bit 3: vacancies
   uint32_t ent;
   // replica groups in quads: quad q holds groups [q gq, (q + 1) gq), W = 1 << lw
-  // words apart; the threads in nch chunks of tpc, chunk q sweeping quads q, q + nch, ..
-  int nq, gq, lw, nch, tpc;
+  // words apart; the threads in nch chunks of tpc, chunk q sweeping quads q, q + nch, ..,
+  // or, with more chunks than quads, part q % parts of quad q / parts
+  int nq, gq, lw, nch, tpc, parts;
   uint32_t k0, k1, tag_main, tag_ref;
   int joint, icm_big;
   int swt_len;       // entries of each pair's swap table in shared memory
@@ -321,17 +322,18 @@ __device__ __noinline__ uint32_t refine8_grp(uint32_t w, uint4 x, uint4 y, uint3
 // lane, so a thread reduces them after at most kFlushSites sites.
 constexpr int kFlushSites = 32;
 
-// The NG groups of quad `quad` at site (c, j): the neighbour vectors are
-// loaded first, then the NG decisions run as one branch-free block whose
-// Philox chains are independent, ties (about 2^-13 per word) are settled
-// after it, and the store comes last.  The field of 8 spins is
+// The NG groups from group g0 on at site (c, j), whose words start at Sq: the
+// neighbour vectors are loaded first, then the NG decisions run as one
+// branch-free block whose Philox chains are independent, ties (about 2^-13
+// per word) are settled after it, and the store comes last.  The field of 8
+// spins is
 // C = n_neg 0x11111111 + sum_d eps_d W_d with eps_d = +1 (J > 0), -1 (J < 0)
 // or 0 (absent bond): per nibble the count of satisfied present bonds
 // (W ^ 1 for a negative bond is 1 - W), exact mod 2^32 because every final
 // nibble lies in 0..6.
 template <int NG, int W, bool UPDATE, bool ENERGY, bool OPEN>
 __device__ __forceinline__ void quad_site(const Ctl &k, uint32_t *Sq, const uint32_t *jn, uint32_t tb0, int c, int j,
-                                          int quad, uint32_t sweep, const PhiloxB (&pb)[NG], uint32_t (&e8)[NG][2]) {
+                                          int g0, uint32_t sweep, const PhiloxB (&pb)[NG], uint32_t (&e8)[NG][2]) {
   const int H = k.H;
   const uint32_t *Wo = Sq + (1 - c) * H * W;
   uint32_t *Wc = Sq + (c * H + j) * W;
@@ -367,7 +369,7 @@ __device__ __forceinline__ void quad_site(const Ctl &k, uint32_t *Sq, const uint
 #pragma unroll
       for (int u = 0; u < NG; ++u) {
         if (!((tmask >> u) & 1u)) continue;
-        const int g = quad * k.gq + u;
+        const int g = g0 + u;
         const uint32_t c2 = ((uint32_t)c << 16) | (uint32_t)k.gmap[g];
         const uint4 x = philox((uint32_t)j, sweep, c2, (k.ent << 8) | k.tag_main, k.k0, k.k1);
         const uint4 y = philox((uint32_t)j, sweep, c2, (k.ent << 8) | k.tag_ref, k.k0, k.k1);
@@ -389,22 +391,22 @@ __device__ __forceinline__ void quad_site(const Ctl &k, uint32_t *Sq, const uint
   }
 }
 
-// Colour c of one quad: sites lt, lt + tpc, .. in blocks of at most
-// kFlushSites per thread, so that the byte lanes of the energy counts cannot
-// overflow.  Whole warps call it (the warp reductions).  The counts leave a
+// Colour c of NG groups of one quad, from its group u0 on: sites lt, lt + tpc,
+// .. in blocks of at most kFlushSites per thread, so that the byte lanes of the
+// energy counts cannot overflow.  Whole warps call it (the warp reductions).  The counts leave a
 // warp through one warp-wide add per packed word (two 16-bit lanes, at most
 // 32 x 192 each) and one atomic per buffer, all buffers' lanes at once.
 template <int NG, int W, bool UPDATE, bool ENERGY, bool OPEN>
-__device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int quad, int lt, int tpc) {
-  const int H = k.H;
-  uint32_t *Sq = dyn_smem() + k.oS + 2 * quad * H * W;
+__device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int quad, int lt, int tpc, int u0 = 0) {
+  const int H = k.H, g0 = quad * k.gq + u0;
+  uint32_t *Sq = dyn_smem() + k.oS + 2 * quad * H * W + u0;
   const uint32_t *jn = dyn_smem() + k.oJn;
-  const uint32_t tb0 = (uint32_t)__cvta_generic_to_shared(dyn_smem() + k.oThh) + 256u * (uint32_t)(quad * k.gq);
+  const uint32_t tb0 = (uint32_t)__cvta_generic_to_shared(dyn_smem() + k.oThh) + 256u * (uint32_t)g0;
   PhiloxB pb[NG];
   if (UPDATE) {
 #pragma unroll
     for (int u = 0; u < NG; ++u)
-      pb[u] = philox_b(sweep, ((uint32_t)c << 16) | (uint32_t)k.gmap[quad * k.gq + u], k.k0, k.k1);
+      pb[u] = philox_b(sweep, ((uint32_t)c << 16) | (uint32_t)k.gmap[g0 + u], k.k0, k.k1);
   }
   for (int b0 = 0; b0 < H; b0 += ENERGY ? kFlushSites * tpc : H) {
     const int b1 = ENERGY ? min(H, b0 + kFlushSites * tpc) : H;
@@ -412,7 +414,7 @@ __device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int qu
 #pragma unroll
     for (int u = 0; u < NG; ++u) e8[u][0] = e8[u][1] = 0u;
     for (int j = b0 + lt; j < b1; j += tpc)
-      quad_site<NG, W, UPDATE, ENERGY, OPEN>(k, Sq, jn, tb0, c, j, quad, sweep, pb, e8);
+      quad_site<NG, W, UPDATE, ENERGY, OPEN>(k, Sq, jn, tb0, c, j, g0, sweep, pb, e8);
     if (ENERGY) {
       const int lane = threadIdx.x & 31;
       uint32_t mine = 0u;
@@ -424,14 +426,14 @@ __device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int qu
           const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, (e8[u][m & 1] >> (8 * (m >> 1))) & 0x00FF00FFu);
           if ((lane >> 3) == u && (lane & 3) == m) mine = v;
         }
-      if (lane < 8 * NG) atomicAdd(&k.Eacc[8 * quad * k.gq + lane], (int)((lane & 4) ? mine >> 16 : mine & 0xFFFFu));
+      if (lane < 8 * NG) atomicAdd(&k.Eacc[8 * g0 + lane], (int)((lane & 4) ? mine >> 16 : mine & 0xFFFFu));
     }
   }
 }
 
 template <bool UPDATE, bool ENERGY, bool OPEN>
 __device__ __forceinline__ void colour_phase_t(Ctl &k, int c, uint32_t sweep) {
-  const int q = (int)threadIdx.x >= k.tpc ? 1 : 0, lt = (int)threadIdx.x - q * k.tpc;   // nch is 1 or 2
+  const int q = (int)threadIdx.x >= k.tpc ? 1 : 0, lt = (int)threadIdx.x - q * k.tpc;   // nch is 1 or 2: at most two quads
   for (int quad = q; quad < k.nq; quad += k.nch) {
     switch (k.gq) {
       case 4: quad_sites<4, 4, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc); break;
@@ -440,6 +442,31 @@ __device__ __forceinline__ void colour_phase_t(Ctl &k, int c, uint32_t sweep) {
       default: quad_sites<1, 1, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc); break;
     }
   }
+}
+
+// The same with more chunks than quads (a launch shape asked for by nch):
+// each of the `parts` chunks of a quad sweeps an even share of its groups,
+// two or one.
+template <bool UPDATE, bool ENERGY, bool OPEN>
+__device__ __forceinline__ void colour_parts_t(Ctl &k, int c, uint32_t sweep) {
+  const int q = (int)threadIdx.x / k.tpc, lt = (int)threadIdx.x - q * k.tpc;
+  const int quad = q / k.parts, per = (k.gq + k.parts - 1) / k.parts, u0 = (q - quad * k.parts) * per;
+  const int ng = min(per, k.gq - u0);
+  if (ng < 1 || quad * k.gq + u0 >= k.Gc) return;   // three groups in four parts, or no group there
+  if (ng == 2)
+    quad_sites<2, 4, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc, u0);
+  else if (k.lw == 2)
+    quad_sites<1, 4, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc, u0);
+  else
+    quad_sites<1, 2, UPDATE, ENERGY, OPEN>(k, c, sweep, quad, lt, k.tpc, u0);
+}
+template <bool UPDATE, bool ENERGY>
+__device__ __noinline__ void colour_parts(int c, uint32_t sweep) {
+  Ctl &k = ctl();
+  if (k.open)
+    colour_parts_t<UPDATE, ENERGY, true>(k, c, sweep);
+  else
+    colour_parts_t<UPDATE, ENERGY, false>(k, c, sweep);
 }
 
 // One colour phase of a sweep over the CTA's groups.  UPDATE: Eq. synapse +
@@ -452,6 +479,7 @@ __device__ __forceinline__ void colour_phase_t(Ctl &k, int c, uint32_t sweep) {
 template <bool UPDATE, bool ENERGY>
 __device__ __noinline__ void colour_phase(int c, uint32_t sweep) {
   Ctl &k = ctl();
+  if (k.parts > 1) return colour_parts<UPDATE, ENERGY>(c, sweep);
   if (k.open)
     colour_phase_t<UPDATE, ENERGY, true>(k, c, sweep);
   else
@@ -1444,6 +1472,7 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     k.lw = quad_shift(k.Gc);
     k.nch = a.cta_nch[cta];
     k.tpc = blockDim.x / k.nch;
+    k.parts = max(1, k.nch / k.nq);
     k.k0 = a.k0;
     k.k1 = a.k1;
     k.tag_main = a.tag_main;

@@ -55,13 +55,16 @@ struct Batch {
   std::vector<uint32_t> h_pbit, h_swaptab, h_swapidx;
 };
 
-// Split of a CTA's threads into nch chunks of tpb/nch threads, chunk q
-// sweeping the quads (up to four replica groups) q, q + nch, .. of every
-// site: `pref` where it fits (tpb a multiple of 32 nch, nch <= quads), else
-// the choice that minimises the longest thread's work (site rounds x quads).
-int choose_nch(int H, int Gc, int tpb, int pref) {
+}  // namespace
+
+// Split of a CTA's threads into nch chunks of tpb/nch threads, each sweeping
+// ceil(groups / nch) replica groups of every site: `pref` where it fits (tpb
+// a multiple of 32 pref, pref <= groups), else one chunk per quad (up to four
+// groups, one vector access per neighbour) or one for all quads, whichever
+// keeps the longest thread's work (site rounds x quads) smaller.
+int apt_chunks(int H, int Gc, int tpb, int pref) {
   const int nq = (Gc + 3) / 4;
-  if (pref > 0 && tpb % (32 * pref) == 0 && pref <= nq) return pref;
+  if (pref > 0 && tpb % (32 * pref) == 0 && pref <= Gc) return pref;
   int best = 1, best_cost = INT_MAX;
   for (int nch = 1; nch <= nq; nch *= 2) {
     if (tpb % (32 * nch)) continue;
@@ -74,6 +77,8 @@ int choose_nch(int H, int Gc, int tpb, int pref) {
   }
   return best;
 }
+
+namespace {
 
 // pack_jn16's words in (colour, j) order: coupling signs (bits 0-5), absent
 // bonds (bits 8-13) and the vacancy flag (bit 15) of site (c, j).
@@ -346,7 +351,7 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
         cp[1].push_back(i);
         cg0[1].push_back(g0);
         cgc[1].push_back(P.A * gu);
-        cnch[1].push_back(choose_nch(P.N / 2, P.A * gu, bt.tpb, bt.nch_pref));
+        cnch[1].push_back(apt_chunks(P.N / 2, P.A * gu, bt.tpb, bt.nch_pref));
       }
       const int gmx = P.A * std::max(h1, Glp - h1);
       for (int q = 0; q < 3; ++q)
@@ -360,7 +365,7 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
       cp[0].push_back(i);
       cg0[0].push_back(g0);
       cgc[0].push_back(gc);
-      cnch[0].push_back(choose_nch(P.N / 2, gc, bt.tpb, bt.nch_pref));
+      cnch[0].push_back(apt_chunks(P.N / 2, gc, bt.tpb, bt.nch_pref));
       for (int q = 0; q < 3; ++q)
         smem[0][q] = std::max(smem[0][q], apt_smem_bytes(P.N, gc, mode, icm, P.T, n_bins, kSwtLens[q]));
     }

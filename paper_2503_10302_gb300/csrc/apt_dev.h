@@ -59,6 +59,8 @@ struct AptArgs {
   uint32_t k0, k1;
 };
 
+// Thread chunks of a CTA with Gc groups of a lattice with H sites per colour.
+int apt_chunks(int H, int Gc, int tpb, int pref);
 size_t apt_smem_bytes(int N, int Gc, int mode, int icm, int T, int n_bins, int swt_len);
 int apt_launch(const AptArgs &a, int n_cta, int tpb, size_t smem, cudaStream_t st);
 int apt_init_launch(const AptArgs &a, int n_prob, int max_words, cudaStream_t st);

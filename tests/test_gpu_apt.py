@@ -679,3 +679,29 @@ def test_first_swap_step_of_small_split_problems(pc, orc, groups):
     apt.run(40, 1, True)
     _compare(pc, apt, ctx, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("labels,temps,nch", [(1, 16, 2), (1, 24, 2), (1, 32, 4), (2, 8, 2), (2, 24, 4), (2, 32, 8),
+                                              (4, 8, 4), (4, 16, 8), (4, 16, 4)])
+def test_thread_chunks_below_a_quad(pc, orc, labels, temps, nch):
+    """More thread chunks than quads: the chunks of a quad share its groups (4
+    as 2 + 2 or 1 each, 3 as 2 + 1, 2 as 1 + 1), with closed lattices, open
+    ones and vacancies; all equal the oracle."""
+    dims, per, J, present = [], [], [], []
+    for i, (d, p_) in enumerate([((4, 4, 4), (1, 1, 1)), ((5, 7, 6), (0, 0, 1)), ((8, 8, 6), (1, 1, 1))]):
+        Ji = W.ea_couplings(d, 23, i)
+        pd, pres, Jp = W.pad_odd_open(d, p_, Ji) if i == 1 else (np.array(d, np.int32), np.ones(int(np.prod(d)), np.uint8), Ji)
+        dims.append(pd); per.append(p_); J.append(Jp); present.append(pres)
+    dims = np.array(dims, np.int32)
+    betas = [W.geometric_ladder(temps)] * 3
+    b = W.AptBatch(dims, J, betas, labels)
+    ctx = pc.Context(0, 67)
+    pc.pc_apt_load_bc(ctx.h, dims, per, J, betas, labels, 0, present_list=present)
+    pc.pc_apt_set_launch(ctx.h, 256, nch, 1, 0)
+    apt = orc.Apt(dims, J, betas, labels, seed=67, periodic=np.array(per, np.uint8), present_list=present)
+    pc.pc_apt_run(ctx.h, 25, 1, labels > 1)
+    pc.pc_apt_run(ctx.h, 3, 4, False)
+    apt.run(25, 1, labels > 1, threads=8)
+    apt.run(3, 4, False, threads=8)
+    _compare(pc, apt, ctx, b)
+    ctx.close()
