@@ -66,6 +66,9 @@ struct SqaArgs {
 };
 size_t sqa_smem_bytes(int N, int P);
 int sqa_launch(const SqaArgs &a, int R, cudaStream_t st);
+// CTAs of the persistent schedule: R runs in n_items items on a GPU that holds
+// `resident` CTAs at a time.
+int sqa_grid(int resident, int R, int n_items);
 
 // ---------------------------------------------------------------- MLP (mlp.cu)
 pc_ctx *mlp_context(pc_mlp *m);

@@ -30,3 +30,14 @@ def test_thread_chunks_are_applied_where_they_fit(so, Gc, tpb):
         for pref in (1, 2, 4, 8):
             fits = pref <= Gc and tpb % (32 * pref) == 0
             assert _chunks(so, H, Gc, tpb, pref) == (pref if fits else own)
+
+
+def test_persistent_anneal_starts_no_cta_without_a_run(so):
+    """Items come chunk by chunk, R runs each: a grid of at most R CTAs takes
+    only first chunks to begin with, whatever the GPU holds at a time."""
+    f = getattr(so, "_ZN2pc8sqa_gridEiii")   # pc::sqa_grid(int, int, int)
+    f.restype, f.argtypes = ctypes.c_int, [ctypes.c_int] * 3
+    for resident in (1, 152, 304, 3648):
+        for R in (1, 2, 151, 153, 200, 304, 456, 4000, 100000):
+            for chunks in (1, 2, 24):
+                assert f(resident, R, R * chunks) == min(resident, R)
