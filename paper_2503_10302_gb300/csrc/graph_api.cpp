@@ -184,10 +184,28 @@ struct GImpl {
   DevBuf<unsigned long long> d_stats;
   size_t smem = 0, smem_staged = 0;
   bool staged = false;
+  int more_warps = 0;   // warps of a label beyond the first, over the colour classes; the batch's largest
   int64_t sweeps = 0, swaps = 0;
   int joint = 0;
   bool ready = false;
 };
+
+}  // namespace
+
+// Whether one label per CTA is faster than both on one.  Per sweep it saves
+// about 0.2 us for each warp that a label has beyond the first in a colour
+// class.  Cluster moves cost it about 1.3 us per attempt, two cluster barriers
+// and a copy.  32 temperatures, us per attempt with moves, two CTAs against one: 60 vertices
+// (no more warps) 16.7, 15.7; 216 of a 6^3 lattice (6) 10.5, 10.0, and with 4
+// sweeps per attempt (24) 16.6, 18.7; 288 of a 6 x 6 x 8 lattice (8) 11.5, 11.7;
+// 1000 of a 10^3 lattice (30) 18.0, 21.9; 64 dimer embeddings of L = 7 (19) 20.7,
+// 23.2.  Without moves two CTAs are up to 6 % faster at 40 to 128 vertices (60:
+// 2 % slower with 64 problems) and 1.7 times at 1000.
+bool gapt_split_pays(int more_warps, int sweeps_per_swap, int icm) {
+  return !icm || (int64_t)more_warps * sweeps_per_swap >= 8;
+}
+
+namespace {
 
 GImpl *gimpl(pc_ctx *c) { return static_cast<GImpl *>(c->graph_impl); }
 
@@ -314,6 +332,9 @@ int gload(pc_ctx *c, GImpl *im, int n_prob, const int32_t *n_vert, const int32_t
     P.bestbase = (uint32_t)bestw;
     P.statbase = (uint32_t)stats.size();
     for (int cc = 0; cc <= kGMaxColours; ++cc) P.off[cc] = g.off[cc];
+    int more = 0;
+    for (int cc = 0; cc < g.C; ++cc) more += (g.off[cc + 1] - g.off[cc] + 31) / 32 - 1;
+    im->more_warps = std::max(im->more_warps, more);
     vinfo.insert(vinfo.end(), g.vinfo.begin(), g.vinfo.end());
     adj.insert(adj.end(), g.adj.begin(), g.adj.end());
     for (int r = 0; r < 32; ++r)
@@ -410,9 +431,9 @@ int pc_gapt_run(pc_ctx *c, int64_t n_swaps, int sweeps_per_swap, int icm) try {
   a.spp = sweeps_per_swap;
   a.icm = icm ? 1 : 0;
   // two labels on two CTAs while every CTA has an SM to itself (the joint swap
-  // rule couples the labels): 64 dimer embeddings of L = 8, ICM, 35.7 -> 30.5 us
-  // per attempt
-  const bool split = im->A == 2 && !im->joint && 2 * im->n_prob <= c->sms;
+  // rule couples the labels) and it pays
+  const bool split =
+      im->A == 2 && !im->joint && 2 * im->n_prob <= c->sms && gapt_split_pays(im->more_warps, sweeps_per_swap, icm);
   int64_t left = n_swaps;
   while (left > 0) {
     const int chunk = (int)std::min<int64_t>(left, 256);

@@ -93,6 +93,8 @@ size_t gapt_smem_bytes(int n, int A, int Imax, int m);
 // split: two labels, a cluster of two CTAs per problem (one label each).
 int gapt_launch(const GAptArgs &a, int n_prob, int A, int Imax, bool staged, size_t smem, bool init, bool split,
                 cudaStream_t st);
+// The rule for split: more_warps sums ceil(class / 32) - 1 over the colour classes.
+bool gapt_split_pays(int more_warps, int sweeps_per_swap, int icm);
 size_t gsqa_smem_bytes(int n, int P, int Imax, int m, int CS);
 // How an anneal of R runs is cut: clusters of CS CTAs per group of `runs` (32
 // or 16) runs; alone: every CTA is to have an SM to itself.

@@ -341,3 +341,36 @@ def test_gapt_two_labels_on_one_or_two_ctas(pc, orc, n_prob):
         for a, b in zip(pc.pc_gapt_get_stats(ctx.h, i, T, 2), ref.stats(i)):
             assert np.array_equal(a, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("more", [0, 1])
+def test_gapt_hits_on_one_or_two_ctas(pc, orc, more):
+    """Two labels with targets that problems reach in the first launch, in a
+    later one or never, graphs of 30 to 1100 vertices among them: as many
+    problems as run on two CTAs each, and one more (one CTA each), equal the
+    oracle."""
+    ctx = pc.Context(0, 19)
+    n_prob = pc.pc_device_sm_count(ctx.h) // 2 + more
+    big = {0: W.sparse_random_graph(1100, 6.0, 3), 1: W.dimer_embedding((7, 6, 7), W.ea_couplings((7, 6, 7), 1000, 3))}
+    graphs = [big.get(i) or W.random_graph(30 + i % 7, 3.0, i, wmax=2) for i in range(n_prob)]
+    betas = [W.geometric_ladder(5 + i % 9, 0.3, 2.0) for i in range(n_prob)]
+    trip = [_trip(g) for g in graphs]
+    first = orc.GApt(trip, betas, n_labels=2, seed=19)
+    first.run(6)
+    early = [first.best(i)["E"] for i in range(n_prob)]
+    first.run(40)
+    late = [first.best(i)["E"] for i in range(n_prob)]
+    target = [(early, late, [e - 10 ** 6 for e in late])[i % 3][i] for i in range(n_prob)]
+    assert any(e > v for e, v in zip(early, late))
+    pc.pc_gapt_load(ctx.h, trip, betas, 2, 0)
+    ref = orc.GApt(trip, betas, n_labels=2, seed=19)
+    for i, t in enumerate(target):
+        pc.pc_gapt_set_target(ctx.h, i, t)
+        ref.set_target(i, t)
+    for k in (6, 40):
+        pc.pc_gapt_run(ctx.h, k, 1, True)
+        ref.run(k)
+    _compare(pc, ctx, ref, graphs, betas, 2)
+    hits = [ref.best(i)["hit_sweep"] for i in range(n_prob)]
+    assert all(0 < h <= 6 for h in hits[0::3]) and all(h < 0 for h in hits[2::3]) and any(h > 6 for h in hits[1::3])
+    ctx.close()

@@ -41,3 +41,15 @@ def test_persistent_anneal_starts_no_cta_without_a_run(so):
         for R in (1, 2, 151, 153, 200, 304, 456, 4000, 100000):
             for chunks in (1, 2, 24):
                 assert f(resident, R, R * chunks) == min(resident, R)
+
+
+def test_small_graphs_with_cluster_moves_stay_on_one_cta(so):
+    """Two labels on two CTAs: always without cluster moves, with them from 8
+    warps beyond the first of each colour class per attempt on (32 colours of
+    32 vertices: none)."""
+    f = getattr(so, "_ZN2pc15gapt_split_paysEiii")   # pc::gapt_split_pays(int, int, int)
+    f.restype, f.argtypes = ctypes.c_bool, [ctypes.c_int] * 3
+    for more in (0, 1, 4, 7, 8, 30, 127):
+        for spp in (1, 2, 4, 10, 2 ** 31 - 1):
+            assert f(more, spp, 0)
+            assert f(more, spp, 1) == (more * spp >= 8)
