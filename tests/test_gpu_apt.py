@@ -705,3 +705,25 @@ def test_thread_chunks_below_a_quad(pc, orc, labels, temps, nch):
     apt.run(3, 4, False, threads=8)
     _compare(pc, apt, ctx, b)
     ctx.close()
+
+
+@pytest.mark.parametrize("groups", [5, 7])
+def test_chains_with_a_partly_filled_second_quad(pc, orc, groups):
+    """Ladder chains and pilot runs of 5 or 7 replica groups in one CTA (a
+    batch as large as the GPU): the second quad has one group less than the
+    first, and the place left over reaches no output."""
+    ctx = pc.Context(0, 71)
+    n = pc.pc_device_sm_count(ctx.h)   # groups per CTA: all of an instance's on as many instances as SMs
+    sides = [(2, 2, 2), (4, 4, 4), (6, 4, 4)]
+    shapes = [sides[i % 3] for i in range(n)]
+    J = [W.ea_couplings(s, 29, i) for i, s in enumerate(shapes)]
+    kw = dict(n_chains=8 * groups - 3, sweeps=45, tail=35, max_len=4)
+    res = pc.pc_adaptive_ladder(ctx.h, shapes, J, entry0=2, **kw)
+    betas = W.geometric_ladder(groups)
+    hist = pc.pc_pilot_hist(ctx.h, shapes, J, betas, entry0=5, chains_per_beta=8, sweeps=40, burn=4)
+    ctx.close()
+    for i, s in enumerate(shapes):
+        beta, sig, ok = orc.adaptive_ladder(s, J[i], entry=2 + i, seed=71, **kw)
+        assert np.array_equal(res[i][0], beta) and np.array_equal(res[i][1], sig) and res[i][2] == ok
+        ref = orc.pilot_hist(s, J[i], betas, entry=5 + i, seed=71, chains_per_beta=8, sweeps=40, burn=4)
+        assert np.array_equal(hist[i], ref)
