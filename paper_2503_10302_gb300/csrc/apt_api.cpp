@@ -332,10 +332,10 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
   // [0]: one-CTA part, [1]: two-CTA-cluster part
   std::vector<int> cp[2], cg0[2], cgc[2], cnch[2];
   // swap-table entries per pair in shared memory: the most that fit (energy
-  // gaps up to 510, 126; none where a part is too large: 32 temperatures x 4
-  // labels on 16^3)
-  constexpr int kSwtLens[3] = {256, 64, 0};
-  size_t smem[2][3] = {};
+  // gaps up to 510, or 126, which the largest CTA has room for: 64 replicas of
+  // 16^3 with cluster moves and 32 temperatures take 226,448 bytes)
+  constexpr int kLens = 2, kSwtLens[kLens] = {256, 64};
+  size_t smem[2][kLens] = {};
   for (int i : order) {
     const AptProbDev &P = bt.prob[(size_t)i];
     const int G = bt.G[(size_t)i];
@@ -354,7 +354,7 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
         cnch[1].push_back(apt_chunks(P.N / 2, P.A * gu, bt.tpb, bt.nch_pref));
       }
       const int gmx = P.A * std::max(h1, Glp - h1);
-      for (int q = 0; q < 3; ++q)
+      for (int q = 0; q < kLens; ++q)
         smem[1][q] = std::max(smem[1][q], apt_smem_bytes(P.N, gmx, mode, icm, P.T, n_bins, kSwtLens[q]));
       continue;
     }
@@ -366,13 +366,13 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
       cg0[0].push_back(g0);
       cgc[0].push_back(gc);
       cnch[0].push_back(apt_chunks(P.N / 2, gc, bt.tpb, bt.nch_pref));
-      for (int q = 0; q < 3; ++q)
+      for (int q = 0; q < kLens; ++q)
         smem[0][q] = std::max(smem[0][q], apt_smem_bytes(P.N, gc, mode, icm, P.T, n_bins, kSwtLens[q]));
     }
   }
-  int fit[2] = {2, 2};
+  int fit[2] = {kLens - 1, kLens - 1};
   for (int part = 0; part < 2; ++part)
-    for (int q = 2; q >= 0; --q)
+    for (int q = kLens - 1; q >= 0; --q)
       if (smem[part][q] <= (size_t)c->smem_optin) fit[part] = q;
   bt.n_u = (int)cp[0].size();
   bt.n_s = (int)cp[1].size();

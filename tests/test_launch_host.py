@@ -53,3 +53,14 @@ def test_small_graphs_with_cluster_moves_stay_on_one_cta(so):
         for spp in (1, 2, 4, 10, 2 ** 31 - 1):
             assert f(more, spp, 0)
             assert f(more, spp, 1) == (more * spp >= 8)
+
+
+def test_the_largest_cta_stages_swap_tables(so):
+    """64 replicas of a 16^3 lattice with cluster moves and 32 temperatures fit
+    a CTA's 232,448 bytes with 64 swap-table entries per pair, not with 256: the
+    shorter length is the last one a schedule needs."""
+    f = getattr(so, "_ZN2pc14apt_smem_bytesEiiiiiii")   # pc::apt_smem_bytes(N, groups, mode, icm, T, n_bins, entries)
+    f.restype, f.argtypes = ctypes.c_size_t, [ctypes.c_int] * 7
+    assert f(4096, 8, 0, 1, 32, 0, 64) == 226448 <= 232448 < f(4096, 8, 0, 1, 32, 0, 256)
+    assert max(f(n, g, 0, i, t, 0, 64) for n in (8, 1728, 4096) for g in range(1, 9) for i in (0, 1)
+               for t in (1, 9, 32)) == 226448
