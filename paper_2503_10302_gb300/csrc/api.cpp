@@ -383,8 +383,13 @@ static int sqa_enqueue(pc_ctx *c, int R, uint32_t run0, int32_t *E_dev, int32_t 
   // one item; slicing it only adds hand-offs through global memory (8 runs of
   // 1024 spins, 100 sweeps: 100 slices of one sweep, 0.45 ms; whole runs
   // 0.19 ms).  Else an item holds at least 2^19 spin updates (about 50 us of an
-  // SM), far above a hand-off's few microseconds.  Runs of one item that are
-  // short skip the queue as well.
+  // SM), far above a hand-off's few microseconds.  Short runs of one item skip
+  // the queue, whose state buffer, counters and status read they would pay for;
+  // above 2^22 updates (0.4 ms) that no longer shows, and the two kernels differ
+  // by their builds alone: the plain one takes 0.97-1.0 of the queue's time
+  // with up to 7 words per site (12^3 x 64 slices 4.85 against 4.90 ms, 10^3 x 16
+  // 6.36 against 6.52) and 0.89 to 1.014 with 8 (6^3 2.93 against 3.27, 12^3 3.91
+  // against 3.86).
   const int64_t upd = (int64_t)a.N * a.P * a.S;
   const bool level = R > c->sms || first_chunk > 0;
   if (a.S > 0 && (level || upd > (1 << 22))) {

@@ -9,11 +9,12 @@
 // Layout.  Replicas ("buffers") of one problem are packed eight to a 32-bit
 // word, one spin per nibble (bit 0 = +1): group g holds buffers 8g..8g+7.
 // Sites are split by checkerboard colour c = (x+y+z)&1 and indexed inside a
-// colour by j = lin >> 1, so a word S[g][c][j] carries site (c, j) of eight
-// replicas.  All replicas of a problem share the couplings, hence one word
-// gives the nibble-packed satisfied-bond counts of eight replicas with six
-// XOR/ADD pairs, and one Philox4x32-10 call gives their eight 16-bit
-// uniforms.
+// colour by j = lin >> 1.  Between launches global memory holds a word per
+// (g, c, j), group by group; a CTA keeps up to four groups of a site side by
+// side (a quad, the array S at Ctl), so that they move as one vector access.
+// All replicas of a problem share the couplings, hence one word gives the
+// nibble-packed satisfied-bond counts of eight replicas with six multiply-adds,
+// and one Philox4x32-10 call gives their eight 16-bit uniforms.
 //
 // Replica slots are fixed: temperature r with ICM label a lives in buffer
 // a*Tp + r (Tp = 8 ceil(T/8)), so the two labels of temperature r sit in the
@@ -122,7 +123,7 @@ struct __align__(16) Ctl {
   // the Glp groups per label (APT; ladder / pilot: A = 1, groups g0 ..);
   // split problems run as a cluster of two CTAs, rank 0 holding the hotter
   // (lower-beta, first) half
-  int Gu, Glp, split, rank;
+  int Gu, Glp, rank;
   int nbonds;        // bonds present (3N with periodic axes)
   int nreal;         // spins present (N without vacancies)
   uint32_t open;     // bit a: axis a open; bit 3: vacancies
@@ -712,16 +713,6 @@ __device__ __forceinline__ void icm_cluster_seeds(Ctl &k) {
   }
 }
 
-// ICMop of Algorithm S2 for every temperature at once.  With A labels per
-// temperature (2 or 4) the labels of temperature r = 8h + i sit in nibble i
-// of groups l*Gl + h, and pair p of the temperature's random matching owns
-// bit 4i + h A/2 + p of the per-site overlap word X, so the overlaps of
-// eight pairs come from one XOR (two labels) or three masked XORs (four).
-// The seed of a pair is the k-th site (canonical order c*H + j) with its
-// bit set, k = floor(x0 n_minus / 2^32); its cluster grows by a flood fill
-// V <- V | (X & OR_nbr V) until no cluster changes.  Clusters larger than
-// N/2 flip one whole replica (x1 bit 0: the pair's first or second label),
-// smaller ones flip in both replicas; then the energies are updated.
 // Overlap bits of one site: the XOR of the two labels' words of each pair,
 // pair bit 4i + h A/2 + p for nibble i of group h.  p points at the
 // site's words of quad 0, p1 at those of quad 1.
@@ -845,6 +836,15 @@ __device__ __forceinline__ void icm_flips(Ctl &k) {
     site_flip<A, GL>(k, S + kk * W, S + (N + kk) * W, V[pos[kk]], fm);
 }
 
+// ICMop of Algorithm S2 for every temperature at once.  With A labels per
+// temperature (2 or 4) the labels of temperature r = 8h + i sit in nibble i
+// of groups l Gu + h, and pair p of the temperature's random matching owns bit
+// 4i + h A/2 + p of the per-site overlap word X.  The seed of a pair is the
+// k-th site (canonical order c*H + j) with its bit set, k = floor(x0 n_minus /
+// 2^32); its cluster grows by a flood fill V <- V | (X & OR_nbr V) until no
+// cluster changes.  Clusters larger than half of the spins present flip one
+// whole replica (x1 bit 0: the pair's first or second label), smaller ones
+// flip in both replicas.  The caller recounts the energies.
 template <bool CSEED>
 __device__ __noinline__ void icm_all(uint32_t t) {
   Ctl &k = ctl();
@@ -1458,7 +1458,6 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     k.g0 = a.cta_g0[cta];
     k.Gc = a.cta_gc[cta];
     k.Bc = min(8 * k.Gc, P.B - 8 * k.g0);
-    k.split = SPLIT;
     k.rank = rank;
     if (MODE == pc::APT_MODE_APT || MODE == pc::APT_MODE_ENERGY) {
       k.Gu = k.Gc / k.A;   // A is 1, 2 or 4

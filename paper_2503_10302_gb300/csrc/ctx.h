@@ -73,7 +73,7 @@ struct SqaState {
   Lattice lat{};
   int P = 0, S = 0;
   double T = 0;
-  std::vector<uint32_t> table;   // [S][24]
+  std::vector<uint32_t> table;   // [S][kSqaTab]
   std::vector<int32_t> jq;       // [S]
   DevBuf<uint16_t> d_jneg;
   int nbonds = 0;
