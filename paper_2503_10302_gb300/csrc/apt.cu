@@ -122,16 +122,17 @@ struct __align__(16) Ctl {
   // this CTA holds, for every label, the temperature groups [g0, g0 + Gu) of
   // the Glp groups per label (APT; ladder / pilot: A = 1, groups g0 ..);
   // split problems run as a cluster of two CTAs, rank 0 holding the hotter
-  // (lower-beta, first) half
-  int Gu, Glp, rank;
+  // (lower-beta, first) half.  parts: thread chunks per quad, where there are
+  // more chunks than quads (PARTS kernels): chunk q sweeps part q % parts of
+  // quad q / parts
+  int Gu, Glp, parts, rank;
   int nbonds;        // bonds present (3N with periodic axes)
   int nreal;         // spins present (N without vacancies)
   uint32_t open;     // bit a: axis a open; bit 3: vacancies
   uint32_t ent;
   // replica groups in quads: quad q holds groups [q gq, (q + 1) gq), W = 1 << lw
-  // words apart; the threads in nch chunks of tpc, chunk q sweeping quads q, q + nch, ..,
-  // or, with more chunks than quads, part q % parts of quad q / parts
-  int nq, gq, lw, nch, tpc, parts;
+  // words apart; the threads in nch chunks of tpc, chunk q sweeping quads q, q + nch, ..
+  int nq, gq, lw, nch, tpc;
   uint32_t k0, k1, tag_main, tag_ref;
   int joint, icm_big;
   int swt_len;       // entries of each pair's swap table in shared memory
@@ -323,18 +324,19 @@ __device__ __noinline__ uint32_t refine8_grp(uint32_t w, uint4 x, uint4 y, uint3
 // lane, so a thread reduces them after at most kFlushSites sites.
 constexpr int kFlushSites = 32;
 
-// The NG groups from group g0 on at site (c, j), whose words start at Sq: the
-// neighbour vectors are loaded first, then the NG decisions run as one
-// branch-free block whose Philox chains are independent, ties (about 2^-13
-// per word) are settled after it, and the store comes last.  The field of 8
-// spins is
+// The NG groups of quad `quad` from its group u0 on at site (c, j), whose words
+// start at Sq: the neighbour vectors are loaded first, then the NG decisions
+// run as one branch-free block whose Philox chains are independent, ties
+// (about 2^-13 per word) are settled after it, and the store comes last.  The
+// field of 8 spins is
 // C = n_neg 0x11111111 + sum_d eps_d W_d with eps_d = +1 (J > 0), -1 (J < 0)
 // or 0 (absent bond): per nibble the count of satisfied present bonds
 // (W ^ 1 for a negative bond is 1 - W), exact mod 2^32 because every final
 // nibble lies in 0..6.
 template <int NG, int W, bool UPDATE, bool ENERGY, bool OPEN>
 __device__ __forceinline__ void quad_site(const Ctl &k, uint32_t *Sq, const uint32_t *jn, uint32_t tb0, int c, int j,
-                                          int g0, uint32_t sweep, const PhiloxB (&pb)[NG], uint32_t (&e8)[NG][2]) {
+                                          int quad, int u0, uint32_t sweep, const PhiloxB (&pb)[NG],
+                                          uint32_t (&e8)[NG][2]) {
   const int H = k.H;
   const uint32_t *Wo = Sq + (1 - c) * H * W;
   uint32_t *Wc = Sq + (c * H + j) * W;
@@ -370,7 +372,7 @@ __device__ __forceinline__ void quad_site(const Ctl &k, uint32_t *Sq, const uint
 #pragma unroll
       for (int u = 0; u < NG; ++u) {
         if (!((tmask >> u) & 1u)) continue;
-        const int g = g0 + u;
+        const int g = quad * k.gq + u0 + u;
         const uint32_t c2 = ((uint32_t)c << 16) | (uint32_t)k.gmap[g];
         const uint4 x = philox((uint32_t)j, sweep, c2, (k.ent << 8) | k.tag_main, k.k0, k.k1);
         const uint4 y = philox((uint32_t)j, sweep, c2, (k.ent << 8) | k.tag_ref, k.k0, k.k1);
@@ -394,20 +396,21 @@ __device__ __forceinline__ void quad_site(const Ctl &k, uint32_t *Sq, const uint
 
 // Colour c of NG groups of one quad, from its group u0 on: sites lt, lt + tpc,
 // .. in blocks of at most kFlushSites per thread, so that the byte lanes of the
-// energy counts cannot overflow.  Whole warps call it (the warp reductions).  The counts leave a
-// warp through one warp-wide add per packed word (two 16-bit lanes, at most
-// 32 x 192 each) and one atomic per buffer, all buffers' lanes at once.
+// energy counts cannot overflow.  Whole warps call it (the warp reductions).
+// The counts leave a warp through one warp-wide add per packed word (two 16-bit
+// lanes, at most 32 x 192 each) and one atomic per buffer, all buffers' lanes
+// at once.
 template <int NG, int W, bool UPDATE, bool ENERGY, bool OPEN>
 __device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int quad, int lt, int tpc, int u0 = 0) {
-  const int H = k.H, g0 = quad * k.gq + u0;
+  const int H = k.H;
   uint32_t *Sq = dyn_smem() + k.oS + 2 * quad * H * W + u0;
   const uint32_t *jn = dyn_smem() + k.oJn;
-  const uint32_t tb0 = (uint32_t)__cvta_generic_to_shared(dyn_smem() + k.oThh) + 256u * (uint32_t)g0;
+  const uint32_t tb0 = (uint32_t)__cvta_generic_to_shared(dyn_smem() + k.oThh) + 256u * (uint32_t)(quad * k.gq + u0);
   PhiloxB pb[NG];
   if (UPDATE) {
 #pragma unroll
     for (int u = 0; u < NG; ++u)
-      pb[u] = philox_b(sweep, ((uint32_t)c << 16) | (uint32_t)k.gmap[g0 + u], k.k0, k.k1);
+      pb[u] = philox_b(sweep, ((uint32_t)c << 16) | (uint32_t)k.gmap[quad * k.gq + u0 + u], k.k0, k.k1);
   }
   for (int b0 = 0; b0 < H; b0 += ENERGY ? kFlushSites * tpc : H) {
     const int b1 = ENERGY ? min(H, b0 + kFlushSites * tpc) : H;
@@ -415,7 +418,7 @@ __device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int qu
 #pragma unroll
     for (int u = 0; u < NG; ++u) e8[u][0] = e8[u][1] = 0u;
     for (int j = b0 + lt; j < b1; j += tpc)
-      quad_site<NG, W, UPDATE, ENERGY, OPEN>(k, Sq, jn, tb0, c, j, g0, sweep, pb, e8);
+      quad_site<NG, W, UPDATE, ENERGY, OPEN>(k, Sq, jn, tb0, c, j, quad, u0, sweep, pb, e8);
     if (ENERGY) {
       const int lane = threadIdx.x & 31;
       uint32_t mine = 0u;
@@ -427,7 +430,8 @@ __device__ __forceinline__ void quad_sites(Ctl &k, int c, uint32_t sweep, int qu
           const uint32_t v = __reduce_add_sync(0xFFFFFFFFu, (e8[u][m & 1] >> (8 * (m >> 1))) & 0x00FF00FFu);
           if ((lane >> 3) == u && (lane & 3) == m) mine = v;
         }
-      if (lane < 8 * NG) atomicAdd(&k.Eacc[8 * g0 + lane], (int)((lane & 4) ? mine >> 16 : mine & 0xFFFFu));
+      if (lane < 8 * NG)
+        atomicAdd(&k.Eacc[8 * (quad * k.gq + u0) + lane], (int)((lane & 4) ? mine >> 16 : mine & 0xFFFFu));
     }
   }
 }
@@ -480,11 +484,22 @@ __device__ __noinline__ void colour_parts(int c, uint32_t sweep) {
 template <bool UPDATE, bool ENERGY>
 __device__ __noinline__ void colour_phase(int c, uint32_t sweep) {
   Ctl &k = ctl();
-  if (k.parts > 1) return colour_parts<UPDATE, ENERGY>(c, sweep);
   if (k.open)
     colour_phase_t<UPDATE, ENERGY, true>(k, c, sweep);
   else
     colour_phase_t<UPDATE, ENERGY, false>(k, c, sweep);
+}
+
+// PARTS: the CTAs of this kernel may have more chunks than quads.  The choice
+// is the kernel's, because a test per phase costs every launch that has no use
+// for it (one function for both forms: adaptive ladders of 64 x L = 12 189.8 ->
+// 194.7 ms, of 20 x L = 6 5.13 -> 5.37 ms).
+template <bool UPDATE, bool ENERGY, bool PARTS>
+__device__ __forceinline__ void colour(int c, uint32_t sweep) {
+  if (PARTS && ctl().parts > 1)
+    colour_parts<UPDATE, ENERGY>(c, sweep);
+  else
+    colour_phase<UPDATE, ENERGY>(c, sweep);
 }
 
 // Energies of label 0 only (two labels): its groups lead quad 0, all threads
@@ -1423,10 +1438,11 @@ __device__ __noinline__ void swap_step(uint32_t t) {
   PROF_MARK(15, pt);
 }
 
-// MODE (pc::APT_MODE_*) and SPLIT (a cluster of two CTAs per problem) are
-// template arguments, so that each kernel carries only its own code (the
-// launcher picks the instantiation from a.mode and a.split).
-template <int MODE, bool SPLIT, bool CSEED>
+// MODE (pc::APT_MODE_*), SPLIT (a cluster of two CTAs per problem), CSEED (the
+// cluster-seed rule) and PARTS (thread chunks below a quad) are template
+// arguments, so that each kernel carries only its own code (the launcher picks
+// the instantiation from the arguments).
+template <int MODE, bool SPLIT, bool CSEED, bool PARTS>
 __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArgs a) {
   uint32_t *const smem = dyn_smem();
   Ctl &k = ctl();
@@ -1469,7 +1485,7 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     k.nq = quads_of(k.Gc);
     k.gq = quad_groups(k.Gc);
     k.lw = quad_shift(k.Gc);
-    k.nch = a.cta_nch[cta];
+    k.nch = PARTS ? a.cta_nch[cta] : min(a.cta_nch[cta], k.nq);
     k.tpc = blockDim.x / k.nch;
     k.parts = max(1, k.nch / k.nq);
     k.k0 = a.k0;
@@ -1558,7 +1574,7 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     __syncthreads();
 
   if (MODE == pc::APT_MODE_ENERGY) {
-    colour_phase<false, true>(1, 0u);
+    colour<false, true, PARTS>(1, 0u);
     __syncthreads();
     for (int b = threadIdx.x; b < 8 * k.Gc; b += blockDim.x) k.E[b] = k.nbonds - 2 * k.Eacc[b];
     __syncthreads();
@@ -1571,14 +1587,14 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
       const uint32_t t = (uint32_t)(t0 + it);
       const uint32_t sf = (uint32_t)(s0 + (int64_t)it * spp);
       for (int qq = 0; qq < spp; ++qq) {
-        colour_phase<true, false>(0, sf + (uint32_t)qq);
+        colour<true, false, PARTS>(0, sf + (uint32_t)qq);
         __syncthreads();
         PROF_MARK(0, pt);
         // energies are read only after the attempt's last sweep
         if (qq + 1 < spp)
-          colour_phase<true, false>(1, sf + (uint32_t)qq);
+          colour<true, false, PARTS>(1, sf + (uint32_t)qq);
         else
-          colour_phase<true, true>(1, sf + (uint32_t)qq);
+          colour<true, true, PARTS>(1, sf + (uint32_t)qq);
         __syncthreads();
         PROF_MARK(1, pt);
       }
@@ -1593,7 +1609,7 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
         if (k.A == 2)
           label0_energies();
         else
-          colour_phase<false, true>(1, 0u);   // the pairs change with the temperature
+          colour<false, true, PARTS>(1, 0u);   // the pairs change with the temperature
         __syncthreads();
         PROF_MARK(9, pt);
         if (threadIdx.x < 32) {
@@ -1609,15 +1625,15 @@ __global__ void __launch_bounds__(512) apt_kernel(const __grid_constant__ AptArg
     // ladder and pilot chains: energies from window_from on only
     for (int it = 0; it < a.n_iter; ++it) {
       const uint32_t s = (uint32_t)(s0 + it);
-      colour_phase<true, false>(0, s);
+      colour<true, false, PARTS>(0, s);
       __syncthreads();
       const bool count = MODE == pc::APT_MODE_LADDER ? (int64_t)it >= a.window_from : (int64_t)s >= a.window_from;
       if (!count) {
-        colour_phase<true, false>(1, s);
+        colour<true, false, PARTS>(1, s);
         __syncthreads();
         continue;
       }
-      colour_phase<true, true>(1, s);
+      colour<true, true, PARTS>(1, s);
       __syncthreads();
       // the next energy pass is two barriers away
       for (int b = threadIdx.x; b < 8 * k.Gc; b += blockDim.x) {
@@ -1766,10 +1782,10 @@ size_t apt_smem_bytes(int N, int Gc, int mode, int icm, int T, int n_bins, int s
   return (words + (size_t)N) * 4;
 }
 
-template <int MODE, bool CSEED>
+template <int MODE, bool CSEED, bool PARTS>
 int apt_launch_mode(const AptArgs &a, int n_cta, int tpb, size_t smem, cudaStream_t st) {
   if (!a.split) {
-    apt_kernel<MODE, false, CSEED><<<n_cta, tpb, smem, st>>>(a);
+    apt_kernel<MODE, false, CSEED, PARTS><<<n_cta, tpb, smem, st>>>(a);
   } else {
     // split problems: consecutive CTA pairs form one cluster
     cudaLaunchConfig_t cfg = {};
@@ -1789,7 +1805,7 @@ int apt_launch_mode(const AptArgs &a, int n_cta, int tpb, size_t smem, cudaStrea
       attr[1].val.priority = a.prio;
       cfg.numAttrs = 2;
     }
-    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, apt_kernel<MODE, true, CSEED>, a));
+    PC_CUDA_TRY(cudaLaunchKernelEx(&cfg, apt_kernel<MODE, true, CSEED, PARTS>, a));
   }
   PC_CUDA_TRY(cudaGetLastError());
   return PC_OK;
@@ -1805,27 +1821,30 @@ int apt_launch(const AptArgs &a, int n_cta, int tpb, size_t smem, cudaStream_t s
   PC_CUDA_TRY(cudaGetDevice(&dev));
   if (dev < 0 || dev >= 64) return fail(PC_EINVAL, "device index out of range");
   if (smem > set_for[dev]) {
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_APT, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_APT, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_APT, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_APT, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_LADDER, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_LADDER, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_PILOT, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_PILOT, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_ENERGY, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    PC_CUDA_TRY(cudaFuncSetAttribute(apt_kernel<pc::APT_MODE_ENERGY, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    const void *const kernels[] = {
+        (const void *)apt_kernel<pc::APT_MODE_APT, false, false, false>, (const void *)apt_kernel<pc::APT_MODE_APT, true, false, false>,
+        (const void *)apt_kernel<pc::APT_MODE_APT, false, true, false>,  (const void *)apt_kernel<pc::APT_MODE_APT, true, true, false>,
+        (const void *)apt_kernel<pc::APT_MODE_APT, false, false, true>,  (const void *)apt_kernel<pc::APT_MODE_APT, true, false, true>,
+        (const void *)apt_kernel<pc::APT_MODE_APT, false, true, true>,   (const void *)apt_kernel<pc::APT_MODE_APT, true, true, true>,
+        (const void *)apt_kernel<pc::APT_MODE_LADDER, false, false, false>, (const void *)apt_kernel<pc::APT_MODE_LADDER, true, false, false>,
+        (const void *)apt_kernel<pc::APT_MODE_PILOT, false, false, false>,  (const void *)apt_kernel<pc::APT_MODE_PILOT, true, false, false>,
+        (const void *)apt_kernel<pc::APT_MODE_ENERGY, false, false, false>, (const void *)apt_kernel<pc::APT_MODE_ENERGY, true, false, false>};
+    for (const void *k : kernels)
+      PC_CUDA_TRY(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     set_for[dev] = smem;
   }
   switch (a.mode) {
     case pc::APT_MODE_APT:
-      // the cluster-seed ICM rule has an instantiation of its own, so the
-      // default rule's code is compiled without it
-      return a.icm_seed ? apt_launch_mode<pc::APT_MODE_APT, true>(a, n_cta, tpb, smem, st)
-                        : apt_launch_mode<pc::APT_MODE_APT, false>(a, n_cta, tpb, smem, st);
-    case pc::APT_MODE_LADDER: return apt_launch_mode<pc::APT_MODE_LADDER, false>(a, n_cta, tpb, smem, st);
-    case pc::APT_MODE_PILOT: return apt_launch_mode<pc::APT_MODE_PILOT, false>(a, n_cta, tpb, smem, st);
-    case pc::APT_MODE_ENERGY: return apt_launch_mode<pc::APT_MODE_ENERGY, false>(a, n_cta, tpb, smem, st);
+      // the cluster-seed ICM rule and chunks below a quad have instantiations
+      // of their own, so the default's code is compiled without them
+      if (a.parts)
+        return a.icm_seed ? apt_launch_mode<pc::APT_MODE_APT, true, true>(a, n_cta, tpb, smem, st)
+                          : apt_launch_mode<pc::APT_MODE_APT, false, true>(a, n_cta, tpb, smem, st);
+      return a.icm_seed ? apt_launch_mode<pc::APT_MODE_APT, true, false>(a, n_cta, tpb, smem, st)
+                        : apt_launch_mode<pc::APT_MODE_APT, false, false>(a, n_cta, tpb, smem, st);
+    case pc::APT_MODE_LADDER: return apt_launch_mode<pc::APT_MODE_LADDER, false, false>(a, n_cta, tpb, smem, st);
+    case pc::APT_MODE_PILOT: return apt_launch_mode<pc::APT_MODE_PILOT, false, false>(a, n_cta, tpb, smem, st);
+    case pc::APT_MODE_ENERGY: return apt_launch_mode<pc::APT_MODE_ENERGY, false, false>(a, n_cta, tpb, smem, st);
     default: return fail(PC_EINVAL, "unknown kernel mode");
   }
 }

@@ -51,6 +51,7 @@ struct Batch {
   int split_h = 0;       // split problems: temperature groups per label on rank 0 (0: half)
   size_t smem = 0;       // max of the two parts
   size_t smem_u = 0, smem_s = 0;
+  bool parts = false;    // some CTA has more thread chunks than quads of groups
   int swt_u = 0, swt_s = 0;   // swap-table entries per pair in shared memory, by part
   std::vector<uint32_t> h_pbit, h_swaptab, h_swapidx;
 };
@@ -272,6 +273,7 @@ AptArgs base_args(pc_ctx *c, Batch &bt) {
   a.icm_big = 1;
   a.icm_seed = 0;
   a.swt_len = bt.split ? bt.swt_s : bt.swt_u;
+  a.parts = bt.parts;
   return a;
 }
 
@@ -384,6 +386,9 @@ int schedule(pc_ctx *c, Batch &bt, const std::vector<char> &active, int mode, in
   bt.smem_s = smem[1][fit[1]];
   const size_t smem_max = std::max(bt.smem_u, bt.smem_s);
   bt.n_cta = bt.n_u + bt.n_s;
+  bt.parts = false;
+  for (int part = 0; part < 2; ++part)
+    for (size_t i = 0; i < cgc[part].size(); ++i) bt.parts = bt.parts || cnch[part][i] > (cgc[part][i] + 3) / 4;
   for (int part = 0; part < 2; ++part)
     for (int g : cgc[part])
       if (g < 1 || g > kMaxGcCta) return fail(PC_EINVAL, "internal: a CTA would hold more than 64 replicas");

@@ -57,6 +57,7 @@ struct AptArgs {
   int64_t window_from;
   uint32_t tag_init, tag_main, tag_ref;
   uint32_t k0, k1;
+  int parts;              // host side only: some CTA has more thread chunks than quads
 };
 
 // Thread chunks of a CTA with Gc groups of a lattice with H sites per colour.
