@@ -31,9 +31,10 @@ constexpr int kDims[kLayers + 1] = {kIn, kHid, kHid, kHid, kOut};
 // (launch_next); wait_previous then waits until that kernel has finished and
 // its writes are visible, so that order and results are those of plain
 // launches.  The products call let_next after their main loop: called at the
-// start, the waiting blocks crowded onto few SMs (1024 samples, 12 steps: 2.51
-// ms plain, 3.98 early, 2.50 late; 256 samples, 10 steps: 1.15, 1.15, 0.93 ms;
-// 64 samples, 5 steps: 0.58, 0.46, 0.46 ms).
+// start, the waiting blocks crowded onto few SMs (1024 samples, 12 steps: 2.53
+// ms plain, 3.98 early, 2.53 late; 256 samples, 10 steps: 1.15, 1.15, 0.95 ms;
+// 64 samples, 5 steps: 0.59, 0.46, 0.46 ms; called again on the same
+// minibatches, host work and the weights' readback included).
 __device__ __forceinline__ void let_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
@@ -66,9 +67,9 @@ struct Products {
 // these layers (256 x 256 x 259 and below) is not arithmetic but how many
 // SMs take part and the latency of each K step: a 64 x 64 tile put 256 x 256
 // on 16 SMs and waited for every load (48 us per product).  With 64 blocks,
-// the loads ahead and 11 instead of 19 launches a training step of 256
-// samples went from 0.40 to 0.11 ms (0.09 with the launches of launch_next).  Every output is one fmaf chain over k
-// in order.
+// the loads ahead and 10 instead of 19 launches a training step of 256
+// samples went from 0.40 to 0.11 ms (0.09 with the launches of launch_next).
+// Every output is one fmaf chain over k in order.
 constexpr int kTile = 32, kGemmThreads = 128;
 
 __device__ __forceinline__ void loss_sum(int B, const float *loss_s, float *loss, float *part) {
