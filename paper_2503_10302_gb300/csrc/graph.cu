@@ -168,28 +168,24 @@ __device__ __forceinline__ void counts2_bytes(const uint32_t (&P)[NP], int g, ui
 }
 
 // Adds the neighbours [e0, e1) of one vertex, label a, into the planes;
-// returns their sum of |w|.  Four neighbours at a time: their entries, then
-// their words, are loaded before the first is added, because each neighbour
-// is a chain of two dependent loads (one at a time, the chains of a vertex's
-// neighbours ran one after the other).
+// returns their sum of |w|.  One neighbour at a time: its entry and word are
+// two dependent loads, but the warps of a colour class hide them, and four
+// loaded ahead (the last repeated past the end) cost more instructions than
+// they saved (64 graphs of 15 x 15 x 12, 32 temperatures, one label 20.2
+// against 19.7 us per attempt; 152 random graphs of 4096 vertices, four labels
+// 157.6 against 153.3).
 template <int A, int NP, bool SM>
 __device__ __forceinline__ int vfield(const char *dynb, const uint32_t *ad, int e0, int e1, int a,
                                       uint32_t (&P)[NP]) {
   int W = 0;
-  for (int e = e0; e < e1; e += 4) {
-    uint32_t en[4], t[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) en[i] = ld_adj<SM>(ad, min(e + i, e1 - 1));
-#pragma unroll
-    for (int i = 0; i < 4; ++i) t[i] = *reinterpret_cast<const uint32_t *>(dynb + (en[i] >> 8) + 4 * a);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      if (e + i >= e1) break;
-      const int w = ent_w(en[i]);
-      const uint32_t wabs = (uint32_t)(w < 0 ? -w : w);
-      vadd<NP>(P, w < 0 ? ~t[i] : t[i], wabs);
-      W += (int)wabs;
-    }
+  for (int e = e0; e < e1; ++e) {
+    const uint32_t en = ld_adj<SM>(ad, e);
+    const int w = ent_w(en);
+    uint32_t t = *reinterpret_cast<const uint32_t *>(dynb + (en >> 8) + 4 * a);
+    if (w < 0) t = ~t;
+    const uint32_t wabs = (uint32_t)(w < 0 ? -w : w);
+    vadd<NP>(P, t, wabs);
+    W += (int)wabs;
   }
   return W;
 }
@@ -493,8 +489,7 @@ __device__ void g_swap(const GCta &k, GShared &sh, uint32_t t, int joint, const 
 // vertex itself past its last neighbour: OR with its own word is harmless) in
 // registers, so that a pass is one set of independent loads instead of a
 // chain of vertex, entry and word loads per neighbour (64 dimer embeddings of
-// L = 8, 2 labels, ICM: 46.8 -> 35.5 us per attempt with the unrolled field
-// sums).
+// L = 8, 2 labels, ICM, one CTA per problem: 46.8 -> 35.5 us per attempt).
 template <int VPT, bool SM>
 __device__ __forceinline__ void g_fill_regs(const GCta &k) {
   uint32_t nb[VPT][4], x[VPT], c[VPT];
