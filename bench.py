@@ -52,16 +52,16 @@ L, P, R, T, SWEEPS = 8, 64, 256, 0.05, 10000
 ALG_OPS_PER_FLIP = 20.0
 # The same count for this implementation's packing (one Philox call feeds 8
 # spins through 16-bit halves, one word holds 8 spins' fields): 5 + 2 + 6.5
-# + 0.5 = 14; an ncu capture of the anneal kernel before its last change counts 15.5 executed
+# + 0.5 = 14; an ncu capture of the anneal kernel counts 15.0 executed
 # thread instructions per update.  Reported beside the roofline, not in it.
 PACKED_OPS_PER_FLIP = 14.0
-NCU_INSTR_PER_FLIP = 15.5
+NCU_INSTR_PER_FLIP = 15.0
 # DRAM bytes (read + write) of one full-size anneal launch, from one ncu
 # capture of the anneal kernel (mean of 3 timed launches), valid while the
 # kernel sources hash to TRAFFIC_SRC_SHA256; otherwise the bench reports
 # null.
-TRAFFIC_BYTES = 2218837          # mean of 3 timed launches: 1.68, 2.59, 2.39 MB
-TRAFFIC_SRC_SHA256 = "3bd5699b4935d0d8c167ac12c4ffe6ed4250f6acb66f74492ec0c50f32983131"
+TRAFFIC_BYTES = 2305877          # mean of 3 timed launches: 1.99, 2.70, 2.23 MB
+TRAFFIC_SRC_SHA256 = "24351453e4357b8c01ce34feffa70a976c31b131abdc277b544805c1317a0dac"
 TRAFFIC_SOURCES = ("paper_2503_10302_gb300/csrc/sqa.cu", "paper_2503_10302_gb300/csrc/device.cuh",
                    "paper_2503_10302_gb300/csrc/internal.h")
 # Shared-memory (LSU data pipe) throughput as a fraction of its peak, from the
@@ -69,9 +69,9 @@ TRAFFIC_SOURCES = ("paper_2503_10302_gb300/csrc/sqa.cu", "paper_2503_10302_gb300
 # integer-issue bound sits under.  The anneal kernel's is valid under
 # TRAFFIC_SRC_SHA256; the APT kernel's two, from the 20-attempt launches of
 # the 64 x L = 12 and mixed batches, under APT_SRC_SHA256.
-SMEM_FRAC_SQA = 0.294
-SMEM_FRAC_APT = {"apt_icm_64xL12": 0.247, "apt_icm_mixed256": 0.286}
-APT_SRC_SHA256 = "0e52ceec74429d7da634e643c1347d1e6caa8e972f7294bef1046754e4f30b92"
+SMEM_FRAC_SQA = 0.313
+SMEM_FRAC_APT = {"apt_icm_64xL12": 0.266, "apt_icm_mixed256": 0.298}
+APT_SRC_SHA256 = "f69bdfb904dda9bea5282871a20403b64158d7dbc14348034fe01a50e2472b44"
 APT_SOURCES = ("paper_2503_10302_gb300/csrc/apt.cu", "paper_2503_10302_gb300/csrc/apt_dev.h",
                "paper_2503_10302_gb300/csrc/device.cuh")
 WORKLOAD = f"DT-SQA 3D +-J L={L} periodic, P={P} slices, R={R} runs, T={T}, Gamma 3.0->1e-3 over {SWEEPS} sweeps"
