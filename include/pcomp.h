@@ -175,8 +175,9 @@ int pc_apt_is_split(pc_ctx *ctx, int *split);
 int pc_apt_autotune(pc_ctx *ctx, int trial_swaps, int icm, int *tpb, int *nch, int *split,
                     int *split_groups);
 /* Set the launch shape directly: tpb threads per CTA (a multiple of 64 in
- * [64, 512]), nch thread chunks (0, 1, 2, 4 or 8; applied where it fits,
- * else the cost model decides), split_pref (0 .. 3) as pc_apt_set_split, and
+ * [64, 512]), nch thread chunks (0, 1, 2, 4 or 8; applied where every chunk
+ * has whole warps and at least one replica group, else the cost model
+ * decides), split_pref (0 .. 3) as pc_apt_set_split, and
  * split_groups (0 .. 3) the temperature groups per label of the hotter CTA of
  * a split problem (0: half; clamped to leave the colder CTA one). */
 int pc_apt_set_launch(pc_ctx *ctx, int tpb, int nch, int split_pref, int split_groups);
